@@ -353,17 +353,11 @@ xspec_taps_kernel(const float2 *__restrict__ P, const int32_t *__restrict__ o, i
                    [&](float2 *x, const float2 *tc, const float2 *tf) { row_dit(x, N, pl, tc, tf); });
 }
 
-template <int... R>
-constexpr int last_of() {
-    constexpr int r[] = {R...};
-    return r[sizeof...(R) - 1];
-}
-
 template <int T, int N, int... R>
 __global__ void __launch_bounds__(T, 2)
 xspec_taps_fixed_kernel(const float2 *__restrict__ P, const int32_t *__restrict__ o, int o_row_stride, int K,
                         float2 *__restrict__ grad_w) {
-    xspec_taps_row(P, o, o_row_stride, K, N, 31, last_of<R...>(), grad_w,
+    xspec_taps_row(P, o, o_row_stride, K, N, 31, last_radix<R...>(), grad_w,
                    [](float2 *x, const float2 *tc, const float2 *tf) { dit_seq<N, N, false, T, R...>(x, tc, tf); });
 }
 

@@ -98,40 +98,11 @@ azimuth_mig_combine_kernel(const float2 *__restrict__ X, const float2 *__restric
 // the planes' products straight into its first DIT pass (blocks of Rk, twiddles 1) and writes its last pass to
 // out (dit_last_global): two shared-memory round trips per transform fewer than staging the rows.
 
-// DIF passes on blocks of M for the radices R, Rest..., the innermost one (M == R) left out.
-template <int N, int M, int T, int R, int... Rest>
-__device__ __forceinline__ void dif_middle(float2 *x, const float2 *tc, const float2 *tf) {
-    if constexpr (sizeof...(Rest) > 0) {
-        dif_pass_c<N, M, R, false, T>(x, tc, tf);
-        dif_middle<N, M / R, T, Rest...>(x, tc, tf);
-    }
-}
-
-// DIT passes for the radices R, Rest... (plan order; blocks of M for R), the innermost one left out.
-template <int N, int M, int T, int R, int... Rest>
-__device__ __forceinline__ void dit_middle(float2 *x, const float2 *tc, const float2 *tf) {
-    if constexpr (sizeof...(Rest) > 0) {
-        dit_middle<N, M / R, T, Rest...>(x, tc, tf);
-        dit_pass_c<N, M, R, false, T>(x, tc, tf);
-    }
-}
-
-template <int... R>
-struct LastRadix;
-template <int R>
-struct LastRadix<R> {
-    static constexpr int value = R;
-};
-template <int R, int... Rest>
-struct LastRadix<R, Rest...> {
-    static constexpr int value = sizeof...(Rest) ? LastRadix<Rest...>::value : R;
-};
-
 template <int T, int N, int R1, int... Rs>
 __global__ void __launch_bounds__(T, 2)
 azimuth_spectrum_fixed_kernel(const float2 *__restrict__ S, float2 *__restrict__ X) {
     extern __shared__ float2 sm[];
-    constexpr int RK = LastRadix<R1, Rs...>::value;
+    constexpr int RK = last_radix<R1, Rs...>();
     float2 *x = sm;
     float2 *tw = x + padded_len(N);
     const size_t row = (size_t)blockIdx.x * N;
@@ -141,7 +112,7 @@ azimuth_spectrum_fixed_kernel(const float2 *__restrict__ S, float2 *__restrict__
     griddep_launch_dependents();
     griddep_wait();                                  // S is complete (no-op without a programmatic predecessor)
     dif_first_global<N, R1, T, false>(S + row, x, tc, tf);
-    dif_middle<N, N / R1, T, Rs...>(x, tc, tf);
+    dif_middle<N, N / R1, T, WholeCta, Rs...>(x, tc, tf);
 #pragma unroll 1
     for (int b = threadIdx.x; b < N / RK; b += T) {   // last DIF pass: blocks of RK, twiddles 1, to X
         float2 v[RK];
@@ -158,7 +129,7 @@ __global__ void __launch_bounds__(T, 2)
 azimuth_mig_combine_fixed_kernel(const float2 *__restrict__ X, const float2 *__restrict__ H, int n_bins, int n_rng,
                                  int d_lo, int n_d, float2 *__restrict__ out) {
     extern __shared__ float2 sm[];
-    constexpr int RK = LastRadix<R1, Rs...>::value;
+    constexpr int RK = last_radix<R1, Rs...>();
     float2 *x = sm;
     float2 *tw = x + padded_len(N);
     const int r = blockIdx.x;
@@ -190,7 +161,7 @@ azimuth_mig_combine_fixed_kernel(const float2 *__restrict__ X, const float2 *__r
         for (int q = 0; q < RK; ++q) x[b * RK + q] = v[q];
     }
     __syncthreads();
-    dit_middle<N, N / R1, T, Rs...>(x, tc, tf);
+    dit_middle<N, N / R1, T, WholeCta, Rs...>(x, tc, tf);
     dit_last_global<N, R1, T>(x, out + (size_t)r * N, tc, tf);
 }
 

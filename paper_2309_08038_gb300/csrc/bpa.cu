@@ -28,7 +28,7 @@
 // Grid: (azimuth tiles of 256 pixels, rows).  Once S is staged in shared memory the nominal kernel is bound by
 // shared-memory bandwidth (two 8-byte window reads per sample) and the supplied-error kernel by FP32 + SFU issue.
 
-#include "rosar_internal.cuh"
+#include "bpa_geometry.cuh"
 
 namespace rosar {
 namespace {
@@ -40,10 +40,6 @@ constexpr int BPA_WR = 6;     // range rows of the staged S window
 template <bool NOMINAL> constexpr int bpa_dc() { return NOMINAL ? 512 : 256; }
 template <bool NOMINAL> constexpr int bpa_wc() { return BPA_THREADS + bpa_dc<NOMINAL>(); }   // window columns (pulses)
 template <bool NOMINAL> constexpr int bpa_smem() { return BPA_WR * bpa_wc<NOMINAL>() * 8; }
-
-__device__ __forceinline__ float2 read_bin(const float2 *__restrict__ S, int l, int L, size_t col, int n_az) {
-    return (l >= 0 && l < L) ? __ldg(S + (size_t)l * n_az + col) : make_float2(0.f, 0.f);
-}
 
 // Per chunk of offsets the bins a pixel of row r reads lie in a few rows near r (x = r + (R_n - rho)/dR, within a
 // couple of bins over a +-30 degree aperture): a window of rows around the chunk's range of x and the pulses
@@ -88,13 +84,7 @@ bpa_kernel(const float2 *__restrict__ S, BpaParams p, const float *__restrict__ 
     const float rho = (float)rho_d;
     const float R = (float)(p.r0 + rho_d);
     const float r0 = (float)p.r0;
-    if (threadIdx.x == 0) {
-        double q = p.two_f_over_c_d * rho_d;
-        q -= floor(q);
-        double s, c;
-        sincospi(2.0 * q, &s, &c);
-        rowph = make_float2((float)c, (float)-s);
-    }
+    if (threadIdx.x == 0) rowph = row_phase(p, rho_d);
 
     float2 acc = make_float2(0.f, 0.f);
     const int d_beg = -(M_ap / 2), d_end = M_ap - M_ap / 2;
@@ -108,27 +98,13 @@ bpa_kernel(const float2 *__restrict__ S, BpaParams p, const float *__restrict__ 
         for (int i = threadIdx.x; i < nd; i += BPA_THREADS) {
             float s, c;
             sincospif((float)(dc + i) / (float)n_az, &s, &c);   // sin/cos(pi*d/n_az)
-            // nominal geometry: x and the weight of this offset
-            const float s2 = s * s;
-            const float num = 4.f * R * r0 * s2;                // R_n^2 - rho^2
-            const float Rn2 = fmaf(rho, rho, num);
-            float delta, alpha;
-            if (Rn2 > 0.f) {
-                const float inv = rsqrtf(Rn2);
-                const float Rn = Rn2 * inv;
-                delta = __fdividef(num, Rn + rho);
-                alpha = fmaxf(0.f, fmaf(-2.f * R, s2, rho) * inv);
-            } else {
-                delta = 0.f;
-                alpha = 1.f;
-            }
-            const float x = fmaf(delta, p.inv_dR, rf);
+            float x, delta, alpha;
+            nominal_tap(s, R, r0, rho, rf, p.inv_dR, x, delta, alpha);
             xlo = fminf(xlo, x);
             xhi = fmaxf(xhi, x);
             if (NOMINAL) {
-                float ps, pc;
-                sincospif(2.f * p.two_f_over_c * delta, &ps, &pc);
-                dtab[i] = make_float4(x, alpha * pc, -alpha * ps, 0.f);
+                const float2 a = nominal_weight(p.two_f_over_c, delta, alpha);
+                dtab[i] = make_float4(x, a.x, a.y, 0.f);
             } else {
                 dtab[i] = make_float4(s, c, x, 0.f);
             }
@@ -276,6 +252,8 @@ rosar_status launch_bpa(const float2 *S, const BpaParams &p, const float *dphi, 
     dim3 grid((n_az + BPA_THREADS - 1) / BPA_THREADS, n_rng);
     static int done[4][kMaxDevices] = {};
     const bool nominal = dphi == nullptr && dr == nullptr;
+    if (nominal && bpa_fft_applies(p, n_rng, n_az, M_ap))
+        return launch_bpa_fft(S, p, L, n_rng, n_az, M_ap, interp, out, s);
     const int v = (nominal ? 0 : 2) + (interp ? 1 : 0);
     static const void *const ks[4] = {(const void *)bpa_kernel<true, false>, (const void *)bpa_kernel<true, true>,
                                       (const void *)bpa_kernel<false, false>, (const void *)bpa_kernel<false, true>};

@@ -165,6 +165,11 @@ rosar_status launch_time_domain_plan(const float *win, const float2 *w, const in
 rosar_status launch_time_domain_planned(const float2 *raw, const TdParams &p, int K, bool bpa, const void *plan,
                                         float2 *out, cudaStream_t s);
 
+// The frequency-domain form (bpa_fft.cu), nominal geometry only: whether it is taken, and its launch.
+bool bpa_fft_applies(const BpaParams &p, int n_rng, int n_az, int M_ap);
+rosar_status launch_bpa_fft(const float2 *S, const BpaParams &p, int L, int n_rng, int n_az, int M_ap, int interp,
+                            float2 *out, cudaStream_t s);
+
 rosar_status launch_bpa(const float2 *S, const BpaParams &p, const float *dphi, const float *dr, int L, int n_rng,
                         int n_az, int M_ap, int interp, float2 *out, cudaStream_t s);
 

@@ -3,7 +3,8 @@
 // (batch.cu): in-place decimation-in-frequency forward transform (digit-reversed output) and
 // its transposed decimation-in-time sequence, radices 16, 8, 4, 2, 5, 3 and a prime-factor 15.
 // The pass functions run on the whole CTA (blockDim.x threads, any count) and end with a barrier
-// (row_filter_fused and dit_last_global, whose last pass writes global memory, do not).
+// (row_filter_fused and dit_last_global, whose last pass writes global memory, do not); the compile-time passes
+// can also run on one of several equal groups of a CTA's threads (ThreadGroup).
 #pragma once
 
 #include <map>
@@ -105,6 +106,44 @@ __device__ __forceinline__ void small_dft<15>(float2 *v) {
     for (int k1 = 0; k1 < 3; ++k1)
 #pragma unroll
         for (int k2 = 0; k2 < 5; ++k2) v[(10 * k1 + 6 * k2) % 15] = b[k1][k2];
+}
+
+// 10 = 2 x 5 and 12 = 3 x 4 the same way: 10: n = 5 n1 + 2 n2, k = 5 k1 + 6 k2; 12: n = 4 n1 + 3 n2, k = 4 k1 + 9 k2.
+template <>
+__device__ __forceinline__ void small_dft<10>(float2 *v) {
+    float2 b[2][5];
+#pragma unroll
+    for (int n2 = 0; n2 < 5; ++n2) {
+        const float2 p = v[(2 * n2) % 10], q = v[(5 + 2 * n2) % 10];
+        b[0][n2] = cadd(p, q);
+        b[1][n2] = csub(p, q);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 2; ++k1) {
+        small_dft<5>(b[k1]);
+#pragma unroll
+        for (int k2 = 0; k2 < 5; ++k2) v[(5 * k1 + 6 * k2) % 10] = b[k1][k2];
+    }
+}
+
+template <>
+__device__ __forceinline__ void small_dft<12>(float2 *v) {
+    float2 b[3][4];
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) {
+        float2 a[3];
+#pragma unroll
+        for (int n1 = 0; n1 < 3; ++n1) a[n1] = v[(4 * n1 + 3 * n2) % 12];
+        small_dft<3>(a);
+#pragma unroll
+        for (int k1 = 0; k1 < 3; ++k1) b[k1][n2] = a[k1];
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+        small_dft<4>(b[k1]);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) v[(4 * k1 + 9 * k2) % 12] = b[k1][k2];
+    }
 }
 
 template <int R>
@@ -216,8 +255,20 @@ __device__ __forceinline__ void stage(int R, float2 *x, int N, int M, const floa
 // Compile-time plans: the same passes for a row length N and a radix sequence fixed at compile time, run by
 // exactly T threads.  Strides, block counts and the quotient by the stride become constants and the
 // per-pass radix dispatch disappears; results are identical to the run-time plan with the same radices.
-template <int... R>
-struct Radices {};
+// Who runs a compile-time pass: the whole CTA (its thread index, __syncthreads), or one of the CTA's groups of T
+// consecutive threads (index within the group, named barrier 1 + group), so that groups transform different rows.
+struct WholeCta {
+    static __device__ __forceinline__ int tid() { return threadIdx.x; }
+    static __device__ __forceinline__ void sync() { __syncthreads(); }
+};
+
+template <int T>
+struct ThreadGroup {
+    static __device__ __forceinline__ int tid() { return threadIdx.x % T; }
+    static __device__ __forceinline__ void sync() {
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / T), "n"(T) : "memory");
+    }
+};
 
 // Butterfly idx of a pass with nblk = N/M blocks of s = M/R butterflies: blocks vary fastest across threads
 // when there are at least 16 blocks of odd length M (the 16 lanes of a 64-bit shared-memory phase then stride
@@ -234,11 +285,11 @@ __device__ __forceinline__ void butterfly_index(int idx, int &blk, int &j) {
     }
 }
 
-template <int N, int M, int R, bool PAD, int T>
+template <int N, int M, int R, bool PAD, int T, typename G = WholeCta>
 __device__ __forceinline__ void dif_pass_c(float2 *x, const float2 *tc, const float2 *tf) {
     constexpr int s = M / R, tstep = N / M, nb = N / R;
 #pragma unroll 1
-    for (int idx = threadIdx.x; idx < nb; idx += T) {
+    for (int idx = G::tid(); idx < nb; idx += T) {
         int blk, j;
         butterfly_index<N, M, R>(idx, blk, j);
         const int base = blk * M + j;
@@ -252,14 +303,14 @@ __device__ __forceinline__ void dif_pass_c(float2 *x, const float2 *tc, const fl
 #pragma unroll
         for (int q = 1; q < R; ++q) x[cpad<PAD>(base + q * s)] = cmul(v[q], wq[q]);
     }
-    __syncthreads();
+    G::sync();
 }
 
-template <int N, int M, int R, bool PAD, int T>
+template <int N, int M, int R, bool PAD, int T, typename G = WholeCta>
 __device__ __forceinline__ void dit_pass_c(float2 *x, const float2 *tc, const float2 *tf) {
     constexpr int s = M / R, tstep = N / M, nb = N / R;
 #pragma unroll 1
-    for (int idx = threadIdx.x; idx < nb; idx += T) {
+    for (int idx = G::tid(); idx < nb; idx += T) {
         int blk, j;
         butterfly_index<N, M, R>(idx, blk, j);
         const int base = blk * M + j;
@@ -273,7 +324,7 @@ __device__ __forceinline__ void dit_pass_c(float2 *x, const float2 *tc, const fl
 #pragma unroll
         for (int r = 0; r < R; ++r) x[cpad<PAD>(base + r * s)] = v[r];
     }
-    __syncthreads();
+    G::sync();
 }
 
 // DIF passes in plan order, the block length M shrinking by each radix.
@@ -288,6 +339,30 @@ template <int N, int M, bool PAD, int T, int R, int... Rest>
 __device__ __forceinline__ void dit_seq(float2 *x, const float2 *tc, const float2 *tf) {
     if constexpr (sizeof...(Rest) > 0) dit_seq<N, M / R, PAD, T, Rest...>(x, tc, tf);
     dit_pass_c<N, M, R, PAD, T>(x, tc, tf);
+}
+
+// DIF passes on blocks of M for the radices R, Rest..., the innermost one (M == R) left out.
+template <int N, int M, int T, typename G, int R, int... Rest>
+__device__ __forceinline__ void dif_middle(float2 *x, const float2 *tc, const float2 *tf) {
+    if constexpr (sizeof...(Rest) > 0) {
+        dif_pass_c<N, M, R, false, T, G>(x, tc, tf);
+        dif_middle<N, M / R, T, G, Rest...>(x, tc, tf);
+    }
+}
+
+// DIT passes for the radices R, Rest... (plan order; blocks of M for R), the innermost one left out.
+template <int N, int M, int T, typename G, int R, int... Rest>
+__device__ __forceinline__ void dit_middle(float2 *x, const float2 *tc, const float2 *tf) {
+    if constexpr (sizeof...(Rest) > 0) {
+        dit_middle<N, M / R, T, G, Rest...>(x, tc, tf);
+        dit_pass_c<N, M, R, false, T, G>(x, tc, tf);
+    }
+}
+
+template <int... R>
+constexpr int last_radix() {
+    constexpr int r[] = {R...};
+    return r[sizeof...(R) - 1];
 }
 
 // The whole row filter conj(DIT(conj(H . DIF(src)))) with the first and last passes on global memory and the
