@@ -262,6 +262,34 @@ ROSAR_API rosar_status rosar_bpa_time_plan(const float *win, const rosar_radar *
 ROSAR_API rosar_status rosar_bpa_time_planned(const rosar_c32 *raw, const void *plan, int n_az, int L, int n_rng,
                                               int M_ap, rosar_c32 *out, void *stream);
 
+/*
+ * The time-domain forms by transforms, with scratch from the caller.  The fast-time phasors of a row's taps are
+ * those of a range bin times a factor smooth in the tap's distance, which a few planes (P, at most 32) interpolate to
+ * float32 accuracy; the image is then P range transforms and one azimuth transform each way instead of K*L
+ * multiply-adds a pixel.  Same sums as rosar_bpa_time / rosar_sas_time (shared offsets), closer to them than the
+ * tensor-core forms (about 1e-6 relative L2 against 1e-5).  A pulse with a sample that is not finite makes the
+ * pixels whose taps read it NaN, as there.
+ *   rosar_time_domain_fft_plan_bytes: size of the plan (bpa = 1: rosar_bpa_time's taps, K = M_ap; 0: SAS), or 0
+ *     where this form is not offered: sizes it does not exist for (n_rng > L, L > 2048, pulse counts without a long
+ *     enough transform, an arm of very many range bins), sizes too small for it to pay, or invalid arguments.  Never
+ *     equal to rosar_time_domain_plan_bytes.
+ *   rosar_time_domain_fft_workspace_bytes: scratch of one image call.
+ *   rosar_*_time_fft_plan: writes the plan (device, 256-byte aligned); arguments as rosar_*_time_plan.
+ *   rosar_*_time_fft: the image from raw (as rosar_*_time_planned), the plan and a workspace (device, 256-byte
+ *     aligned, one per call in flight).
+ */
+ROSAR_API size_t rosar_time_domain_fft_plan_bytes(const rosar_radar *radar, int bpa, int n_az, int L, int n_rng, int K);
+ROSAR_API size_t rosar_time_domain_fft_workspace_bytes(int bpa, int n_az, int L, int n_rng, int K);
+ROSAR_API rosar_status rosar_bpa_time_fft_plan(const float *win, const rosar_radar *radar, int n_az, int L, int n_rng,
+                                               int M_ap, void *plan, size_t plan_bytes, void *stream);
+ROSAR_API rosar_status rosar_sas_time_fft_plan(const float *win, const rosar_c32 *w, const int32_t *o,
+                                               const rosar_radar *radar, int n_az, int L, int n_rng, int K, int centred,
+                                               void *plan, size_t plan_bytes, void *stream);
+ROSAR_API rosar_status rosar_bpa_time_fft(const rosar_c32 *raw, const void *plan, int n_az, int L, int n_rng, int M_ap,
+                                          void *workspace, size_t workspace_bytes, rosar_c32 *out, void *stream);
+ROSAR_API rosar_status rosar_sas_time_fft(const rosar_c32 *raw, const void *plan, int n_az, int L, int n_rng, int K,
+                                          void *workspace, size_t workspace_bytes, rosar_c32 *out, void *stream);
+
 /* ------------------------------------------------------------------------
  * Frequency-domain form of the sparse azimuth filter.  Eq. (43) with a fixed
  * row is a circular convolution of S[r][.] with g_r, g_r[(-o_k) mod n_az] += w[r][k];

@@ -274,8 +274,8 @@ rosar_status plan_params(const char *what, const rosar_radar *radar, int n_az, i
     return ROSAR_OK;
 }
 
-rosar_status planned_params(const char *what, const rosar_c32 *raw, const void *plan, int n_az, int L, int n_rng, int K,
-                            const rosar_c32 *out, TdParams *p) {
+rosar_status planned_params(const char *what, const rosar_c32 *raw, const void *plan, size_t plan_bytes, int n_az, int L,
+                            int n_rng, int K, const rosar_c32 *out, TdParams *p) {
     if (!raw || !plan || !out) return set_error(ROSAR_ERR_INVALID_ARG, "%s: null raw, plan or out", what);
     if (n_az < 1 || n_rng < 1 || K < 1 || L < 16 || L > 65536)
         return set_error(ROSAR_ERR_INVALID_ARG, "%s: need n_az, n_rng, K >= 1 and 16 <= L <= 65536", what);
@@ -287,7 +287,7 @@ rosar_status planned_params(const char *what, const rosar_c32 *raw, const void *
         return set_error(ROSAR_ERR_INVALID_ARG, "%s: misaligned pointer", what);
     const size_t ob = sizeof(rosar_c32) * (size_t)n_rng * n_az;
     if (overlaps(out, ob, raw, sizeof(rosar_c32) * (size_t)n_az * L) ||
-        overlaps(out, ob, plan, time_domain_plan_bytes(n_rng, L, K)))
+        overlaps(out, ob, plan, plan_bytes))
         return set_error(ROSAR_ERR_INVALID_ARG, "%s: out overlaps raw or the plan", what);
     *p = TdParams{};
     p->n_az = n_az;
@@ -316,7 +316,8 @@ rosar_status rosar_sas_time_planned(const rosar_c32 *raw, const void *plan, int 
                                     rosar_c32 *out, void *stream) {
     clear_error();
     TdParams p;
-    rosar_status st = planned_params("sas_time_planned", raw, plan, n_az, L, n_rng, K, out, &p);
+    rosar_status st = planned_params("sas_time_planned", raw, plan, time_domain_plan_bytes(n_rng, L, K), n_az, L, n_rng,
+                                     K, out, &p);
     if (st != ROSAR_OK) return st;
     return launch_time_domain_planned(reinterpret_cast<const float2 *>(raw), p, K, false, plan,
                                       reinterpret_cast<float2 *>(out), static_cast<cudaStream_t>(stream));
@@ -337,11 +338,105 @@ rosar_status rosar_bpa_time_planned(const rosar_c32 *raw, const void *plan, int 
                                     rosar_c32 *out, void *stream) {
     clear_error();
     TdParams p;
-    rosar_status st = planned_params("bpa_time_planned", raw, plan, n_az, L, n_rng, M_ap, out, &p);
+    rosar_status st = planned_params("bpa_time_planned", raw, plan, time_domain_plan_bytes(n_rng, L, M_ap), n_az, L, n_rng,
+                                     M_ap, out, &p);
     if (st != ROSAR_OK) return st;
     if (M_ap > n_az) return set_error(ROSAR_ERR_INVALID_ARG, "bpa_time_planned: M_ap=%d exceeds n_az=%d", M_ap, n_az);
     return launch_time_domain_planned(reinterpret_cast<const float2 *>(raw), p, M_ap, true, plan,
                                       reinterpret_cast<float2 *>(out), static_cast<cudaStream_t>(stream));
+}
+
+namespace {
+// Sizes of the transform form for valid arguments, else false (nothing is reported: the direct call says why).
+bool fft_form(const rosar_radar *radar, int bpa, int n_az, int L, int n_rng, int K, TdParams *p, size_t *plan_bytes,
+              size_t *ws_bytes) {
+    if (!radar || (bpa != 0 && bpa != 1)) return false;
+    if (plan_params("time_domain_fft", radar, n_az, L, n_rng, K, true, reinterpret_cast<const void *>(16), SIZE_MAX, p) !=
+        ROSAR_OK)
+        return false;
+    return time_domain_lr_applies(*p, bpa == 1, K, plan_bytes, ws_bytes);
+}
+
+rosar_status fft_plan(const char *what, const float *win, const float2 *w, const int32_t *o, const rosar_radar *radar,
+                      int bpa, int n_az, int L, int n_rng, int K, int centred, void *plan, size_t plan_bytes, void *stream) {
+    TdParams p;
+    rosar_status st = plan_params(what, radar, n_az, L, n_rng, K, centred == 1, plan, SIZE_MAX, &p);
+    if (st != ROSAR_OK) return st;
+    size_t need = 0, ws = 0;
+    if (!time_domain_lr_applies(p, bpa == 1, K, &need, &ws))
+        return set_error(ROSAR_ERR_UNSUPPORTED, "%s: no transform form for n_az=%d L=%d n_rng=%d K=%d", what, n_az, L,
+                         n_rng, K);
+    if (plan_bytes < need)
+        return set_error(ROSAR_ERR_INVALID_ARG, "%s: plan of %zu bytes < %zu needed", what, plan_bytes, need);
+    if (misaligned(plan, 256)) return set_error(ROSAR_ERR_INVALID_ARG, "%s: plan must be 256-byte aligned", what);
+    if ((win && misaligned(win, 4)) || (w && misaligned(w, 8)) || (o && misaligned(o, 4)))
+        return set_error(ROSAR_ERR_INVALID_ARG, "%s: misaligned pointer", what);
+    return launch_time_domain_lr_plan(win, w, o, p, K, bpa == 1, plan, static_cast<cudaStream_t>(stream));
+}
+
+rosar_status fft_image(const char *what, const rosar_c32 *raw, const void *plan, int bpa, int n_az, int L, int n_rng,
+                       int K, void *workspace, size_t workspace_bytes, rosar_c32 *out, void *stream) {
+    TdParams p;
+    // how many planes the plan holds is known to the device alone: at least two
+    const size_t plane = sizeof(rosar_c32) * (size_t)n_rng * n_az;
+    rosar_status st = planned_params(what, raw, plan, n_rng > 0 && n_az > 0 ? 2 * plane : 1, n_az, L, n_rng, K, out, &p);
+    if (st != ROSAR_OK) return st;
+    if (!workspace) return set_error(ROSAR_ERR_INVALID_ARG, "%s: null workspace", what);
+    const size_t need = time_domain_lr_workspace(bpa == 1, n_az, L, n_rng, K);
+    if (need == 0)
+        return set_error(ROSAR_ERR_UNSUPPORTED, "%s: no transform form for n_az=%d L=%d n_rng=%d K=%d", what, n_az, L,
+                         n_rng, K);
+    if (workspace_bytes < need)
+        return set_error(ROSAR_ERR_INVALID_ARG, "%s: workspace of %zu bytes < %zu needed", what, workspace_bytes, need);
+    if (misaligned(workspace, 256) || misaligned(plan, 256))
+        return set_error(ROSAR_ERR_INVALID_ARG, "%s: plan and workspace must be 256-byte aligned", what);
+    const size_t ob = sizeof(rosar_c32) * (size_t)n_rng * n_az;
+    if (overlaps(workspace, need, raw, sizeof(rosar_c32) * (size_t)n_az * L) || overlaps(workspace, need, out, ob) ||
+        overlaps(workspace, need, plan, 2 * plane))
+        return set_error(ROSAR_ERR_INVALID_ARG, "%s: workspace overlaps another argument", what);
+    return launch_time_domain_lr(reinterpret_cast<const float2 *>(raw), n_az, L, n_rng, K, bpa == 1, plan, workspace,
+                                 reinterpret_cast<float2 *>(out), static_cast<cudaStream_t>(stream));
+}
+}  // namespace
+
+size_t rosar_time_domain_fft_plan_bytes(const rosar_radar *radar, int bpa, int n_az, int L, int n_rng, int K) {
+    TdParams p;
+    size_t plan = 0, ws = 0;
+    const bool ok = fft_form(radar, bpa, n_az, L, n_rng, K, &p, &plan, &ws);
+    clear_error();
+    return ok ? plan : 0;
+}
+
+size_t rosar_time_domain_fft_workspace_bytes(int bpa, int n_az, int L, int n_rng, int K) {
+    return time_domain_lr_workspace(bpa == 1, n_az, L, n_rng, K);
+}
+
+rosar_status rosar_bpa_time_fft_plan(const float *win, const rosar_radar *radar, int n_az, int L, int n_rng, int M_ap,
+                                     void *plan, size_t plan_bytes, void *stream) {
+    clear_error();
+    return fft_plan("bpa_time_fft_plan", win, nullptr, nullptr, radar, 1, n_az, L, n_rng, M_ap, 1, plan, plan_bytes, stream);
+}
+
+rosar_status rosar_sas_time_fft_plan(const float *win, const rosar_c32 *w, const int32_t *o, const rosar_radar *radar,
+                                     int n_az, int L, int n_rng, int K, int centred, void *plan, size_t plan_bytes,
+                                     void *stream) {
+    clear_error();
+    if (centred != 0 && centred != 1) return set_error(ROSAR_ERR_INVALID_ARG, "sas_time_fft_plan: centred must be 0 or 1");
+    if (!w || !o) return set_error(ROSAR_ERR_INVALID_ARG, "sas_time_fft_plan: null w or o");
+    return fft_plan("sas_time_fft_plan", win, reinterpret_cast<const float2 *>(w), o, radar, 0, n_az, L, n_rng, K, centred,
+                    plan, plan_bytes, stream);
+}
+
+rosar_status rosar_bpa_time_fft(const rosar_c32 *raw, const void *plan, int n_az, int L, int n_rng, int M_ap,
+                                void *workspace, size_t workspace_bytes, rosar_c32 *out, void *stream) {
+    clear_error();
+    return fft_image("bpa_time_fft", raw, plan, 1, n_az, L, n_rng, M_ap, workspace, workspace_bytes, out, stream);
+}
+
+rosar_status rosar_sas_time_fft(const rosar_c32 *raw, const void *plan, int n_az, int L, int n_rng, int K,
+                                void *workspace, size_t workspace_bytes, rosar_c32 *out, void *stream) {
+    clear_error();
+    return fft_image("sas_time_fft", raw, plan, 0, n_az, L, n_rng, K, workspace, workspace_bytes, out, stream);
 }
 
 rosar_status rosar_image(const rosar_c32 *raw, const float *win, const rosar_c32 *w, const int32_t *o,

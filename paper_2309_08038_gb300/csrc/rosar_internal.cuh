@@ -170,6 +170,15 @@ bool bpa_fft_applies(const BpaParams &p, int n_rng, int n_az, int M_ap);
 rosar_status launch_bpa_fft(const float2 *S, const BpaParams &p, int L, int n_rng, int n_az, int M_ap, int interp,
                             float2 *out, cudaStream_t s);
 
+// The same by transforms (time_domain_lr.cu): whether it is taken for these sizes and what it needs, the plan
+// (geometry only), the image from a plan and a workspace.
+bool time_domain_lr_applies(const TdParams &p, bool bpa, int K, size_t *plan_bytes, size_t *ws_bytes);
+size_t time_domain_lr_workspace(bool bpa, int n_az, int L, int n_rng, int K);
+rosar_status launch_time_domain_lr_plan(const float *win, const float2 *w, const int32_t *o, const TdParams &p, int K,
+                                        bool bpa, void *plan, cudaStream_t s);
+rosar_status launch_time_domain_lr(const float2 *raw, int n_az, int L, int n_rng, int K, bool bpa, const void *plan,
+                                   void *workspace, float2 *out, cudaStream_t s);
+
 rosar_status launch_bpa(const float2 *S, const BpaParams &p, const float *dphi, const float *dr, int L, int n_rng,
                         int n_az, int M_ap, int interp, float2 *out, cudaStream_t s);
 

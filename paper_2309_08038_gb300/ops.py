@@ -134,8 +134,21 @@ def image_fft_host(raw_host, win, H, raw_dev, workspace, out_dev, out_host, stre
     return out_host
 
 
+def _scratch(nbytes, device, stream):
+    """Device scratch of one call: allocated on the current stream, kept until `stream` has passed the call."""
+    t = torch.empty(nbytes, dtype=torch.uint8, device=device)
+    if stream is not None:
+        t.record_stream(stream)
+    return t
+
+
+def _up256(n):
+    return (n + 255) & ~255
+
+
 def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None):
-    """rosar_bpa_time: time-domain back-projection (Eq. (14)) of the raw cube [n_az, L] onto rows 0..n_rng-1."""
+    """rosar_bpa_time: time-domain back-projection (Eq. (14)) of the raw cube [n_az, L] onto rows 0..n_rng-1; by
+    transforms (rosar_bpa_time_fft, plan and workspace allocated here) where the library offers that for the sizes."""
     lib = _lib.load()
     require(raw, torch.complex64, "raw", ndim=2)
     n_az, L = raw.shape
@@ -145,6 +158,15 @@ def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None):
         out = torch.empty((n_rng, n_az), dtype=torch.complex64, device=raw.device)
     require(out, torch.complex64, "out", shape=(n_rng, n_az))
     st = radar.as_struct()
+    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 1, n_az, L, n_rng, M_ap)
+    if nbytes and raw.data_ptr() % 16 == 0:
+        at, ws = _up256(nbytes), lib.rosar_time_domain_fft_workspace_bytes(1, n_az, L, n_rng, M_ap)
+        scratch = _scratch(at + ws, raw.device, stream)
+        h = stream_handle(stream)
+        check(lib.rosar_bpa_time_fft_plan(ptr(win), ctypes.byref(st), n_az, L, n_rng, M_ap, scratch.data_ptr(), nbytes, h))
+        check(lib.rosar_bpa_time_fft(ptr(raw), scratch.data_ptr(), n_az, L, n_rng, M_ap, scratch.data_ptr() + at, ws,
+                                     ptr(out), h))
+        return out
     check(lib.rosar_bpa_time(ptr(raw), ptr(win), ctypes.byref(st), n_az, L, n_rng, M_ap, ptr(out),
                              stream_handle(stream)))
     return out
@@ -152,7 +174,7 @@ def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None):
 
 def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
     """rosar_sas_time: time-domain sparse-aperture imaging (Algorithm 2) of the raw cube [n_az, L]; one output
-    row per row of w [n_rng, K]."""
+    row per row of w [n_rng, K].  Shared offsets by transforms (rosar_sas_time_fft) where the library offers that."""
     lib = _lib.load()
     require(raw, torch.complex64, "raw", ndim=2)
     n_az, L = raw.shape
@@ -165,6 +187,16 @@ def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
         out = torch.empty((n_rng, n_az), dtype=torch.complex64, device=raw.device)
     require(out, torch.complex64, "out", shape=(n_rng, n_az))
     st = radar.as_struct()
+    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, n_az, L, n_rng, K) if stride == 0 else 0
+    if nbytes and raw.data_ptr() % 16 == 0:
+        at, ws = _up256(nbytes), lib.rosar_time_domain_fft_workspace_bytes(0, n_az, L, n_rng, K)
+        scratch = _scratch(at + ws, raw.device, stream)
+        h = stream_handle(stream)
+        check(lib.rosar_sas_time_fft_plan(ptr(win), ptr(w), ptr(o), ctypes.byref(st), n_az, L, n_rng, K,
+                                          1 if centred else 0, scratch.data_ptr(), nbytes, h))
+        check(lib.rosar_sas_time_fft(ptr(raw), scratch.data_ptr(), n_az, L, n_rng, K, scratch.data_ptr() + at, ws,
+                                     ptr(out), h))
+        return out
     check(lib.rosar_sas_time(ptr(raw), ptr(win), ptr(w), ptr(o), stride, ctypes.byref(st), n_az, L, n_rng, K,
                              1 if centred else 0, ptr(out), stream_handle(stream)))
     return out
@@ -172,9 +204,10 @@ def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
 
 @dataclass(frozen=True)
 class TimeDomainPlan:
-    """The precomputed B operand of the tensor-core time-domain forms (rosar_*_time_plan): a uint8 device tensor
-    of rosar_time_domain_plan_bytes(n_rng, L, K) bytes (the taps' B tiles in ascending offset order and the
-    sorted offsets), with the shape it was made for."""
+    """What the time-domain forms compute once per weight design, with the shape it was made for: a uint8 device
+    tensor, either the transform form's plan (rosar_*_time_fft_plan, where the library offers it for the sizes) or the
+    precomputed B operand of the tensor-core forms (rosar_*_time_plan: rosar_time_domain_plan_bytes(n_rng, L, K)
+    bytes, which the other's size never equals)."""
 
     data: torch.Tensor
     n_az: int
@@ -189,56 +222,63 @@ def _plan_tensor(n_rng, L, K, device):
 
 
 def sas_time_plan(win, w, o, radar: Radar, n_az, L, centred=True, stream=None):
-    """rosar_sas_time_plan: the B operand of rosar_sas_time for the weights w [n_rng, K] and shared offsets o [K]."""
+    """rosar_sas_time_plan or rosar_sas_time_fft_plan for the weights w [n_rng, K] and shared offsets o [K]."""
     lib = _lib.load()
     require(w, torch.complex64, "w", ndim=2)
     n_rng, K = w.shape
     require(o, torch.int32, "o", shape=(K,))
     if win is not None:
         require(win, torch.float32, "win", shape=(L,))
-    data = _plan_tensor(n_rng, L, K, w.device)
     st = radar.as_struct()
-    check(lib.rosar_sas_time_plan(ptr(win), ptr(w), ptr(o), ctypes.byref(st), n_az, L, n_rng, K, 1 if centred else 0,
-                                  ptr(data), data.numel(), stream_handle(stream)))
+    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, n_az, L, n_rng, K)
+    data = torch.empty(nbytes, dtype=torch.uint8, device=w.device) if nbytes else _plan_tensor(n_rng, L, K, w.device)
+    make = lib.rosar_sas_time_fft_plan if nbytes else lib.rosar_sas_time_plan
+    check(make(ptr(win), ptr(w), ptr(o), ctypes.byref(st), n_az, L, n_rng, K, 1 if centred else 0, ptr(data),
+               data.numel(), stream_handle(stream)))
     return TimeDomainPlan(data, n_az, L, n_rng, K)
 
 
-def sas_time_planned(raw, plan: TimeDomainPlan, out=None, stream=None):
-    """rosar_sas_time_planned: rosar_sas_time of raw [n_az, L] with a plan from sas_time_plan (which holds the
-    offsets)."""
+def _planned(raw, plan, bpa, direct, transforms, out, stream):
     lib = _lib.load()
     require(raw, torch.complex64, "raw", shape=(plan.n_az, plan.L))
     if out is None:
         out = torch.empty((plan.n_rng, plan.n_az), dtype=torch.complex64, device=raw.device)
     require(out, torch.complex64, "out", shape=(plan.n_rng, plan.n_az))
-    check(lib.rosar_sas_time_planned(ptr(raw), ptr(plan.data), plan.n_az, plan.L, plan.n_rng, plan.K, ptr(out),
-                                     stream_handle(stream)))
+    sizes = (plan.n_az, plan.L, plan.n_rng, plan.K)
+    if plan.data.numel() == lib.rosar_time_domain_plan_bytes(plan.n_rng, plan.L, plan.K):
+        check(direct(ptr(raw), ptr(plan.data), *sizes, ptr(out), stream_handle(stream)))
+    else:
+        ws = lib.rosar_time_domain_fft_workspace_bytes(bpa, *sizes)
+        scratch = _scratch(ws, raw.device, stream)
+        check(transforms(ptr(raw), ptr(plan.data), *sizes, ptr(scratch), ws, ptr(out), stream_handle(stream)))
     return out
 
 
+def sas_time_planned(raw, plan: TimeDomainPlan, out=None, stream=None):
+    """rosar_sas_time_planned or rosar_sas_time_fft: rosar_sas_time of raw [n_az, L] with a plan from sas_time_plan
+    (which holds the offsets)."""
+    lib = _lib.load()
+    return _planned(raw, plan, 0, lib.rosar_sas_time_planned, lib.rosar_sas_time_fft, out, stream)
+
+
 def bpa_time_plan(win, radar: Radar, n_az, L, n_rng, M_ap, device=None, stream=None):
-    """rosar_bpa_time_plan: the B operand of rosar_bpa_time (M_ap taps of the nominal geometry)."""
+    """rosar_bpa_time_plan or rosar_bpa_time_fft_plan: the plan of rosar_bpa_time (M_ap taps of the nominal geometry)."""
     lib = _lib.load()
     if win is not None:
         require(win, torch.float32, "win", shape=(L,))
     device = win.device if win is not None else (device or torch.device("cuda"))
-    data = _plan_tensor(n_rng, L, M_ap, device)
     st = radar.as_struct()
-    check(lib.rosar_bpa_time_plan(ptr(win), ctypes.byref(st), n_az, L, n_rng, M_ap, ptr(data), data.numel(),
-                                  stream_handle(stream)))
+    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 1, n_az, L, n_rng, M_ap)
+    data = torch.empty(nbytes, dtype=torch.uint8, device=device) if nbytes else _plan_tensor(n_rng, L, M_ap, device)
+    make = lib.rosar_bpa_time_fft_plan if nbytes else lib.rosar_bpa_time_plan
+    check(make(ptr(win), ctypes.byref(st), n_az, L, n_rng, M_ap, ptr(data), data.numel(), stream_handle(stream)))
     return TimeDomainPlan(data, n_az, L, n_rng, M_ap)
 
 
 def bpa_time_planned(raw, plan: TimeDomainPlan, out=None, stream=None):
-    """rosar_bpa_time_planned: rosar_bpa_time of raw [n_az, L] with a plan from bpa_time_plan."""
+    """rosar_bpa_time_planned or rosar_bpa_time_fft: rosar_bpa_time of raw [n_az, L] with a plan from bpa_time_plan."""
     lib = _lib.load()
-    require(raw, torch.complex64, "raw", shape=(plan.n_az, plan.L))
-    if out is None:
-        out = torch.empty((plan.n_rng, plan.n_az), dtype=torch.complex64, device=raw.device)
-    require(out, torch.complex64, "out", shape=(plan.n_rng, plan.n_az))
-    check(lib.rosar_bpa_time_planned(ptr(raw), ptr(plan.data), plan.n_az, plan.L, plan.n_rng, plan.K, ptr(out),
-                                     stream_handle(stream)))
-    return out
+    return _planned(raw, plan, 1, lib.rosar_bpa_time_planned, lib.rosar_bpa_time_fft, out, stream)
 
 
 def image(raw, win, w, o, workspace=None, out=None, stream=None):
