@@ -328,13 +328,11 @@ ROSAR_API rosar_status rosar_image_fft(const rosar_c32 *raw, const float *win, c
 /*
  * rosar_image_fft for a sequence of n_scans scans that share win and H (Eq. (38) then
  * Eq. (43) per scan, Sec. III-D): out[s] equals rosar_image_fft(raw[s]) bit for bit.
- * Where a pipelined plan exists for (L, n_az) (rosar_image_fft_scans_pipelined), the
- * launches overlap consecutive scans: one launch runs the azimuth rows of scan s-1 together
- * with the range compression of scan s, the two scans alternating between the halves of
- * the workspace; otherwise the scans run one after the other through rosar_image_fft.
+ * Two launches for the whole sequence: the range compression of every scan into the place
+ * of its image, then every row filtered where it lies.
  *   raw       [n_scans][n_az][L] complex, pulse-major (in)
  *   win, H    as rosar_image_fft (in)
- *   workspace [2][L][n_az] complex (scratch)
+ *   workspace [2][L][n_az] complex (scratch; not read, contents unspecified)
  *   out       [n_scans][L][n_az] complex (out)
  * Limits as rosar_image_fft; n_scans >= 1.  No argument may overlap another (except
  * win/H, which are read only).  Errors as rosar_image_fft.
@@ -342,7 +340,8 @@ ROSAR_API rosar_status rosar_image_fft(const rosar_c32 *raw, const float *win, c
 ROSAR_API rosar_status rosar_image_fft_scans(const rosar_c32 *raw, const float *win, const rosar_c32 *H, int n_scans,
                                              int n_az, int L, rosar_c32 *workspace, rosar_c32 *out, void *stream);
 
-/* 1 if rosar_image_fft_scans overlaps consecutive scans for this (L, n_az), else 0. */
+/* 1 for the (L, n_az) whose sequences once had a pipelined kernel of their own (64 x 360, 128 and 256 x 1800, 128, 256
+ * and 512 x 3600), else 0.  Every sequence runs as described above. */
 ROSAR_API int rosar_image_fft_scans_pipelined(int L, int n_az);
 
 /*
@@ -510,10 +509,13 @@ ROSAR_API rosar_status rosar_range_compress_adjoint_scans(const rosar_c32 *g, co
                                                           int L, int centred, rosar_c32 *grad_raw, void *stream);
 
 /* ------------------------------------------------------------------------
- * Batched form: many scans of uneven n_az, L and K imaged by ONE persistent
- * kernel launch, captured once in a CUDA graph.
+ * Batched form: many scans of uneven n_az, L and K imaged by one launch of a
+ * captured CUDA graph.
  *
- * The persistent CTAs pull tiles from an atomic ticket counter: range tiles
+ * Scans that all have a plan H, with the default tuning, run as one kernel per range
+ * length and one per row length over all scans of that length; nothing waits on the
+ * device.  Any other batch or tuning (gather tiles, an interleave, a CTA count, flags,
+ * the test hook) is one persistent kernel.  Its CTAs pull tiles from an atomic ticket counter: range tiles
  * (P pulses of one scan through the range FFT, as rosar_range_compress) and
  * azimuth tiles (one row segment of one scan through the gather-MAC filter, as
  * rosar_sparse_azimuth).  An azimuth tile waits, on the device, until every range
@@ -543,7 +545,7 @@ typedef struct rosar_scan {
 
 typedef struct rosar_batch_tuning {
     int az_tile;            /* azimuth outputs per tile: 256, 512, 1024 or 2048; 0 selects 1024 */
-    int ctas_per_sm;        /* persistent CTAs per SM; 0 or more than fit selects the occupancy limit */
+    int ctas_per_sm;        /* persistent CTAs per SM; more than fit selects the occupancy limit, as 0 does */
     int interleave;         /* 0: every range tile first, then every azimuth tile; 1: scan by scan;
                                d in [2, 8]: range tiles run d-1 scans ahead of azimuth tiles */
     int spin_limit;         /* polls (~0.1 us apart) before a dependency wait gives up; 0 selects 2^24 */
@@ -577,7 +579,8 @@ ROSAR_API rosar_status rosar_batch_launch(rosar_batch *batch, void *stream);
 /* Waits for `stream`, then reports ROSAR_OK or ROSAR_ERR_TIMEOUT (a dependency wait gave up). */
 ROSAR_API rosar_status rosar_batch_status(rosar_batch *batch, void *stream);
 
-/* Number of tiles (range, azimuth), persistent CTAs and shared bytes per CTA; any pointer may be NULL. */
+/* Number of tiles (range, azimuth), CTAs (of the persistent kernel, or of all launches by length) and the most shared
+ * bytes a CTA needs; any pointer may be NULL. */
 ROSAR_API rosar_status rosar_batch_info(const rosar_batch *batch, int *range_tiles, int *azimuth_tiles,
                                         int *ctas, int *smem_bytes);
 

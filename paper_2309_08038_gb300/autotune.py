@@ -122,7 +122,7 @@ def batch_candidates(fft_tiles: bool = True):
 def _batch_key(scans) -> str:
     shapes = sorted((tuple(s["raw"].shape), s["w"].shape[1], s["o"].dim(), s.get("H") is not None) for s in scans)
     h = hashlib.sha1(repr(shapes).encode()).hexdigest()[:16]
-    return f"batch2/{_gpu()}/{len(scans)}scans/{h}"
+    return f"batch3/{_gpu()}/{len(scans)}scans/{h}"
 
 
 def tune_batch(scans, candidates=None, reps: int = 3, use_cache: bool = True) -> dict:

@@ -1,4 +1,4 @@
-"""Batched form: many uneven scans imaged by one persistent, graph-captured launch (rosar_batch_*)."""
+"""Batched form: many uneven scans imaged by one launch of a captured graph (rosar_batch_*)."""
 
 from __future__ import annotations
 
@@ -35,7 +35,8 @@ DISCARD_S = 2     # ROSAR_BATCH_DISCARD_S
 
 
 class Batch:
-    """A set of scans bound to one CUDA graph [counter reset -> persistent kernel].
+    """A set of scans bound to one CUDA graph: launches over the scans of one length (every scan with H, default
+    tuning), or [counter reset -> persistent kernel].
 
     Each scan is a dict with CUDA tensors raw [n_az, L], w [L, K], o [K] or [L, K], and optionally
     win [L], S [L, n_az] (workspace), out [L, n_az] (allocated here when missing) and H [L, n_az]

@@ -23,7 +23,7 @@
 
 #include <cooperative_groups.h>
 
-#include "row_fft.cuh"
+#include "batch_rows.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -39,48 +39,74 @@ struct Layout {
     size_t bytes;
 };
 
-// The row filter on one CTA: stage the H row and the twiddle table, wait for S, forward DIF, product with
-// H (digit-reversed order, carries 1/N) between conjugations, DIT, store.  FWD/DIT run the passes.
-// Row b of S/out uses row (b mod h_rows) of H (a stack of scans sharing one plan); conj_h applies conj(H), the
-// adjoint filter.
-// phase (optional): [n_rows / h_rows][N] per-column factors; row b is multiplied by phase row b / h_rows before
-// the filter (the scans of a stack each with its own phase correction).  spec (optional): [n_rows][N] the rows'
-// forward transforms (digit-reversed order, before the product with H), for the weight gradient.
-struct RowMap {
-    int h_rows;
-    int conj_h;
+// What one CTA filters: a row of S through a row of H (conj_h: conj(H), the adjoint filter) into a row of out, which
+// may be the row of S itself.  phase (optional): [N] per-column factors applied as the row is loaded.  spec (optional):
+// [N] receives the row's forward transform (digit-reversed order, before the product with H), for the weight gradient.
+struct RowRef {
+    const float2 *S, *H;
+    float2 *out;
+    bool conj_h;
     const float2 *phase;
     float2 *spec;
 };
 
-template <typename FWD, typename INV>
-__device__ __forceinline__ void row_filter(const float2 *__restrict__ S, const float2 *__restrict__ H, int N, int pad_shift,
-                                           const Layout &lay, RowMap map, float2 *__restrict__ out, FWD fwd, INV inv) {
+// Rows of a stack: row b of S and out uses row (b mod h_rows) of H (a stack of scans sharing one plan) and phase row
+// b / h_rows (each scan its own phase correction); phase [n_rows / h_rows][N], spec [n_rows][N].
+struct StackRows {
+    const float2 *S, *H;
+    float2 *out;
+    int h_rows, conj_h;
+    const float2 *phase;
+    float2 *spec;
+
+    __device__ __forceinline__ RowRef at(int b, int N) const {
+        const size_t row = (size_t)b * N;
+        return RowRef{S + row, H + (size_t)(b % h_rows) * N, out + row, conj_h != 0,
+                      phase ? phase + (size_t)(b / h_rows) * N : nullptr, spec ? spec + row : nullptr};
+    }
+};
+
+// Rows of the scans of a batch that have this length, each scan with its own plan.
+struct BatchRows {
+    ScanGroup g;
+
+    __device__ __forceinline__ RowRef at(int b, int N) const {
+        int r;
+        const ScanDev &sc = g.find(b, r);
+        const size_t row = (size_t)r * N;
+        return RowRef{sc.S + row, sc.H + row, sc.out + row, false, nullptr, nullptr};
+    }
+};
+
+// The row filter on one CTA: stage the H row and the twiddle table, wait for S, forward DIF, product with
+// H (digit-reversed order, carries 1/N) between conjugations, DIT, store.
+template <typename ROWS, int MAXT>
+__global__ void __launch_bounds__(MAXT, (MAXT == 384 ? 2 : 1))
+azimuth_fft_kernel(ROWS rows, int N, RowPlan pl, Layout lay) {
     extern __shared__ float2 sm[];
+    const int pad_shift = pl.pad_shift;
     float2 *x = sm;
     float2 *hb = x + padded_len(N);
     float2 *tw = lay.stage_h ? hb + padded_len(N) : hb;
-    const size_t row = (size_t)blockIdx.x * N;
-    const size_t hrow = (size_t)(blockIdx.x % map.h_rows) * N;
-    const float hs = map.conj_h ? -1.f : 1.f;
+    const RowRef ref = rows.at(blockIdx.x, N);
+    const float hs = ref.conj_h ? -1.f : 1.f;
     // prologue independent of S: the H row and the twiddle table
     if (lay.stage_h)
-        for (int n = threadIdx.x; n < N; n += blockDim.x) cp_async8(hb + rpad(n, pad_shift), H + hrow + n);
+        for (int n = threadIdx.x; n < N; n += blockDim.x) cp_async8(hb + rpad(n, pad_shift), ref.H + n);
     cp_async_commit();
     const float2 *tc, *tf;
     build_twiddles(N, lay.full_tab != 0, tw, &tc, &tf);
     griddep_wait();                          // S is complete (no-op unless launched to overlap its producer)
-    for (int n = threadIdx.x; n < N; n += blockDim.x) cp_async8(x + rpad(n, pad_shift), S + row + n);
+    for (int n = threadIdx.x; n < N; n += blockDim.x) cp_async8(x + rpad(n, pad_shift), ref.S + n);
     cp_async_commit();
     cp_async_wait<0>();
-    if (map.phase) {                         // each thread scales the elements it staged
-        const float2 *ph = map.phase + (size_t)(blockIdx.x / map.h_rows) * N;
-        for (int n = threadIdx.x; n < N; n += blockDim.x) x[rpad(n, pad_shift)] = cmul(x[rpad(n, pad_shift)], __ldg(ph + n));
-    }
+    if (ref.phase)                           // each thread scales the elements it staged
+        for (int n = threadIdx.x; n < N; n += blockDim.x)
+            x[rpad(n, pad_shift)] = cmul(x[rpad(n, pad_shift)], __ldg(ref.phase + n));
     __syncthreads();
-    fwd(x, tc, tf);
-    if (map.spec)
-        for (int n = threadIdx.x; n < N; n += blockDim.x) map.spec[row + n] = x[rpad(n, pad_shift)];
+    row_dif(x, N, pl, tc, tf);
+    if (ref.spec)
+        for (int n = threadIdx.x; n < N; n += blockDim.x) ref.spec[n] = x[rpad(n, pad_shift)];
     if (lay.stage_h) {
         for (int n = threadIdx.x; n < N; n += blockDim.x) {   // spectrum times H (same digit-reversed order, carries 1/N), conjugated
             float2 h = hb[rpad(n, pad_shift)];
@@ -91,47 +117,30 @@ __device__ __forceinline__ void row_filter(const float2 *__restrict__ S, const f
     } else {
 #pragma unroll 4
         for (int n = threadIdx.x; n < N; n += blockDim.x) {
-            float2 h = __ldg(H + hrow + n);
+            float2 h = __ldg(ref.H + n);
             h.y *= hs;
             const float2 y = cmul(h, x[rpad(n, pad_shift)]);
             x[rpad(n, pad_shift)] = make_float2(y.x, -y.y);
         }
     }
     __syncthreads();
-    inv(x, tc, tf);
+    row_dit(x, N, pl, tc, tf);
     for (int n = threadIdx.x; n < N; n += blockDim.x) {
         const float2 y = x[rpad(n, pad_shift)];
-        out[row + n] = make_float2(y.x, -y.y);
+        ref.out[n] = make_float2(y.x, -y.y);
     }
 }
 
-template <int MAXT>
-__global__ void __launch_bounds__(MAXT, (MAXT == 384 ? 2 : 1))
-azimuth_fft_kernel(const float2 *__restrict__ S, const float2 *__restrict__ H, int N, RowPlan pl, Layout lay, RowMap map,
-                   float2 *__restrict__ out) {
-    row_filter(S, H, N, pl.pad_shift, lay, map, out,
-               [&](float2 *x, const float2 *tc, const float2 *tf) { row_dif(x, N, pl, tc, tf); },
-               [&](float2 *x, const float2 *tc, const float2 *tf) { row_dit(x, N, pl, tc, tf); });
-}
-
-// Compile-time plan for one row length (T threads, no padding: N has an odd factor, H staged): the first pass
-// reads S from global memory, the last writes the image, and the last forward pass, the product with H and
-// the first inverse pass run as one step (row_filter_fused): four barriers for 16.15.15.
-// Rows whose staged pair (S and H) would not fit the 200 KB shared-memory cap of the row layouts read H from
-// global memory in the fused step (14400-pulse rows).
-template <int N>
-constexpr bool stage_h_fits() { return filter_row_smem<N, true>() <= 200 * 1024; }
-
-template <int T, int N, int... R>
-__global__ void __launch_bounds__(T, (T <= 256 ? 2 : 1))
-azimuth_fft_fixed_kernel(const float2 *__restrict__ S, const float2 *__restrict__ H, RowMap map,
-                         float2 *__restrict__ out) {
+// Compile-time plan for one row length (T threads, no padding: N has an odd factor): the first pass reads S from
+// global memory, the last writes the image, and the last forward pass, the product with H and the first inverse pass
+// run as one step (row_filter_fused): four barriers for 16.15.15.  H_SMEM: the H row staged by cp.async before S is
+// there; otherwise the fused step reads it from global memory.
+template <typename ROWS, int T, int MINB, int N, bool H_SMEM, int... R>
+__global__ void __launch_bounds__(T, MINB)
+azimuth_fft_fixed_kernel(ROWS rows) {
     extern __shared__ float2 sm[];
-    const size_t row = (size_t)blockIdx.x * N;
-    const size_t hrow = (size_t)(blockIdx.x % map.h_rows) * N;
-    filter_row_cta<T, N, stage_h_fits<N>(), R...>(S + row, H + hrow, map.conj_h != 0, out + row, sm,
-                                                  map.phase ? map.phase + (size_t)(blockIdx.x / map.h_rows) * N : nullptr,
-                                                  map.spec ? map.spec + row : nullptr);
+    const RowRef ref = rows.at(blockIdx.x, N);
+    filter_row_cta<T, N, H_SMEM, R...>(ref.S, ref.H, ref.conj_h, ref.out, sm, ref.phase, ref.spec);
 }
 
 // dl != nullptr: plane blockIdx.y of the range-migration-aware plan, built from the taps of row r whose row
@@ -394,92 +403,100 @@ int azimuth_fft_supported(int n_az) {
     return make_plan(n_az, &pl) ? 1 : 0;
 }
 
-template <int MAXT>
-cudaError_t launch_fft_rows(int g, int t, size_t sm, cudaStream_t s, bool overlap, const float2 *S, const float2 *H,
-                            int N, const RowPlan &pl, const Layout &lay, RowMap map, float2 *out) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g);
-    cfg.blockDim = dim3(t);
-    cfg.dynamicSmemBytes = sm;
-    cfg.stream = s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, azimuth_fft_kernel<MAXT>, S, H, N, pl, lay, map, out);
-}
-
 namespace {
 
-// Launches the compile-time-plan kernel when the run-time planner picks exactly its radices for n_az (so H,
-// made by the run-time plan, is in the same order); returns false to fall back to the run-time plan.
-template <int T, int N, int... R>
-bool try_fixed(int n_az, const RowPlan &pl, int n_rng, RowMap map, bool ov, const float2 *S, const float2 *H,
-               float2 *out, cudaStream_t s, cudaError_t *le, rosar_status *st) {
-    constexpr int rad[] = {R...};
-    if (n_az != N || threads_for(N) != T || pl.pad_shift != pad_shift_for(N) || pad_shift_for(N) != 31 ||
-        pl.npass != (int)sizeof...(R))
-        return false;
-    for (int i = 0; i < pl.npass; ++i)
-        if (pl.rad[i] != rad[i]) return false;
-    static int done[kMaxDevices] = {};
-    const void *k = (const void *)azimuth_fft_fixed_kernel<T, N, R...>;
-    constexpr size_t smem = filter_row_smem<N, stage_h_fits<N>()>();
-    *st = ensure_smem(k, smem, done, "azimuth_fft");
-    if (*st != ROSAR_OK) return true;
+template <typename K, typename... A>
+cudaError_t launch_overlapped(K kernel, int grid, int threads, size_t smem, bool overlap, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_rng);
-    cfg.blockDim = dim3(T);
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = ov ? 1 : 0;
-    *le = cudaLaunchKernelEx(&cfg, azimuth_fft_fixed_kernel<T, N, R...>, S, H, map, out);
-    *st = check_launch("azimuth_fft");
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// One launch of a row filter over n_rng rows; `only_prepare`: set the kernel's shared-memory limit and launch nothing.
+struct RowLaunch {
+    int n_az, n_rng;
+    bool overlap, only_prepare;
+    cudaStream_t s;
+};
+
+template <typename ROWS, int T, int MINB, int N, bool H_SMEM, int... R>
+rosar_status launch_fixed(const RowLaunch &l, const ROWS &rows) {
+    static int done[kMaxDevices] = {};
+    constexpr size_t smem = filter_row_smem<N, H_SMEM>();
+    static_assert(smem <= 200 * 1024, "the staged rows exceed the shared-memory cap");
+    const auto kernel = azimuth_fft_fixed_kernel<ROWS, T, MINB, N, H_SMEM, R...>;
+    rosar_status st = ensure_smem((const void *)kernel, smem, done, "azimuth_fft");
+    if (st != ROSAR_OK || l.only_prepare) return st;
+    const cudaError_t e = launch_overlapped(kernel, l.n_rng, T, smem, l.overlap, l.s, rows);
+    if (e != cudaSuccess) return set_error(ROSAR_ERR_CUDA, "azimuth_fft: launch failed: %s", cudaGetErrorString(e));
+    return check_launch("azimuth_fft");
+}
+
+// Whether the run-time planner picks exactly these radices for n_az (H, made by the run-time plan, is in their order).
+template <int N, int... R>
+bool plan_is(int n_az, const RowPlan &pl) {
+    constexpr int rad[] = {R...};
+    if (n_az != N || pl.pad_shift != 31 || pl.npass != (int)sizeof...(R)) return false;
+    for (int i = 0; i < pl.npass; ++i)
+        if (pl.rad[i] != rad[i]) return false;
     return true;
+}
+
+// Up to two rows an SM, a row's own latency counts: 256 threads and H staged while S is awaited.  With more the SM's
+// rows in flight count: one row of shared memory and at most 64 registers hold 4 CTAs of 3600 pulses (46 % of the
+// warps instead of 30) or 8 of 1800, and H is read in the fused step.  4096 rows of 3600 pulses 82 -> 77 us, 8192 of
+// 1800 97 -> 76; at 256 rows 10.3 and 10.4, 6.4 and 8.2.  7200-pulse rows hold one CTA an SM with H staged: 256 rows
+// 20.5 -> 16.6 us, 2048 rows 141 -> 100.
+constexpr int kFewRows = 304;
+
+template <typename ROWS>
+rosar_status launch_rows_of(const RowLaunch &l, const ROWS &rows) {
+    RowPlan pl;
+    if (!make_plan(l.n_az, &pl))
+        return set_error(ROSAR_ERR_UNSUPPORTED, "azimuth_fft: n_az=%d is not 2^a 3^b 5^c in [2, %d]", l.n_az, AF_MAX_N);
+    const bool few = l.n_rng <= kFewRows;
+    if (plan_is<3600, 16, 15, 15>(l.n_az, pl))
+        return few ? launch_fixed<ROWS, 256, 2, 3600, true, 16, 15, 15>(l, rows)
+                   : launch_fixed<ROWS, 256, 4, 3600, false, 16, 15, 15>(l, rows);
+    if (plan_is<1800, 8, 15, 15>(l.n_az, pl))
+        return few ? launch_fixed<ROWS, 256, 2, 1800, true, 8, 15, 15>(l, rows)
+                   : launch_fixed<ROWS, 128, 8, 1800, false, 8, 15, 15>(l, rows);
+    if (plan_is<7200, 8, 4, 15, 15>(l.n_az, pl)) return launch_fixed<ROWS, 256, 3, 7200, false, 8, 4, 15, 15>(l, rows);
+    if (plan_is<14400, 8, 8, 15, 15>(l.n_az, pl))
+        return launch_fixed<ROWS, 1024, 1, 14400, false, 8, 8, 15, 15>(l, rows);
+    if (plan_is<360, 8, 3, 15>(l.n_az, pl))
+        return few ? launch_fixed<ROWS, 256, 2, 360, true, 8, 3, 15>(l, rows)
+                   : launch_fixed<ROWS, 64, 8, 360, false, 8, 3, 15>(l, rows);
+    const Layout lay = layout_for(l.n_az, true);
+    static int done[3][kMaxDevices] = {};
+    const int T = threads_for(l.n_az), v = T <= 256 ? 0 : T <= 512 ? 1 : 2;
+    const auto kernel = v == 0 ? azimuth_fft_kernel<ROWS, 256> : v == 1 ? azimuth_fft_kernel<ROWS, 512>
+                                                                       : azimuth_fft_kernel<ROWS, 1024>;
+    rosar_status st = ensure_smem((const void *)kernel, lay.bytes, done[v], "azimuth_fft");
+    if (st != ROSAR_OK || l.only_prepare) return st;
+    const cudaError_t e = launch_overlapped(kernel, l.n_rng, T, lay.bytes, l.overlap, l.s, rows, l.n_az, pl, lay);
+    if (e != cudaSuccess) return set_error(ROSAR_ERR_CUDA, "azimuth_fft: launch failed: %s", cudaGetErrorString(e));
+    return check_launch("azimuth_fft");
 }
 
 }  // namespace
 
 rosar_status launch_azimuth_fft(const float2 *S, const float2 *H, int n_rng, int n_az, float2 *out, cudaStream_t s,
                                 bool overlap_predecessor, int h_rows, bool conj_h, const float2 *phase, float2 *spec) {
-    const RowMap map{h_rows > 0 ? h_rows : n_rng, conj_h ? 1 : 0, phase, spec};
-    RowPlan pl;
-    if (!make_plan(n_az, &pl))
-        return set_error(ROSAR_ERR_UNSUPPORTED, "azimuth_fft: n_az=%d is not 2^a 3^b 5^c in [2, %d]", n_az, AF_MAX_N);
-    static int done[4][kMaxDevices] = {};
-    const Layout lay = layout_for(n_az, true);
-    const bool ov = overlap_predecessor;
-    {
-        cudaError_t fle = cudaSuccess;
-        rosar_status fst = ROSAR_OK;
-        if (try_fixed<256, 3600, 16, 15, 15>(n_az, pl, n_rng, map, ov, S, H, out, s, &fle, &fst) ||
-            try_fixed<256, 1800, 8, 15, 15>(n_az, pl, n_rng, map, ov, S, H, out, s, &fle, &fst) ||
-            try_fixed<512, 7200, 8, 4, 15, 15>(n_az, pl, n_rng, map, ov, S, H, out, s, &fle, &fst) ||
-            try_fixed<1024, 14400, 8, 8, 15, 15>(n_az, pl, n_rng, map, ov, S, H, out, s, &fle, &fst) ||
-            try_fixed<256, 360, 8, 3, 15>(n_az, pl, n_rng, map, ov, S, H, out, s, &fle, &fst)) {
-            if (fst == ROSAR_OK && fle != cudaSuccess)
-                return set_error(ROSAR_ERR_CUDA, "azimuth_fft: launch failed: %s", cudaGetErrorString(fle));
-            return fst;
-        }
-    }
-    cudaError_t le = cudaSuccess;
-    static const void *const ks[4] = {(const void *)azimuth_fft_kernel<256>, (const void *)azimuth_fft_kernel<384>,
-                                      (const void *)azimuth_fft_kernel<512>, (const void *)azimuth_fft_kernel<1024>};
-    rosar_status st = launch_rows(
-        n_az, n_rng, lay.bytes,
-        [&](int g, int t, size_t sm) { le = launch_fft_rows<256>(g, t, sm, s, ov, S, H, n_az, pl, lay, map, out); },
-        [&](int g, int t, size_t sm) { le = launch_fft_rows<384>(g, t, sm, s, ov, S, H, n_az, pl, lay, map, out); },
-        [&](int g, int t, size_t sm) { le = launch_fft_rows<512>(g, t, sm, s, ov, S, H, n_az, pl, lay, map, out); },
-        [&](int g, int t, size_t sm) { le = launch_fft_rows<1024>(g, t, sm, s, ov, S, H, n_az, pl, lay, map, out); },
-        ks, done, "azimuth_fft");
-    if (st == ROSAR_OK && le != cudaSuccess)
-        return set_error(ROSAR_ERR_CUDA, "azimuth_fft: launch failed: %s", cudaGetErrorString(le));
-    return st;
+    return launch_rows_of(RowLaunch{n_az, n_rng, overlap_predecessor, false, s},
+                          StackRows{S, H, out, h_rows > 0 ? h_rows : n_rng, conj_h ? 1 : 0, phase, spec});
+}
+
+rosar_status launch_azimuth_group(int n_az, const ScanGroup &g, int total, cudaStream_t s, bool prepare) {
+    return launch_rows_of(RowLaunch{n_az, total, false, prepare, s}, BatchRows{g});
 }
 
 namespace {

@@ -1,6 +1,13 @@
-// Batched form: many uneven scans, one persistent launch inside a CUDA graph.
+// Batched form: many uneven scans bound to one CUDA graph.
 //
-// Work is a list of tiles in ticket order.  A range tile runs the range-FFT tile
+// Scans that all have a plan H, in the default order (every range tile first), run as one launch per range length and
+// one per row length over all scans of that length (ScanGroup): range launches side by side, then row launches.  Each
+// launch is the kernel of a single scan's call with that length's own shared memory, registers and threads.  One
+// kernel for every tile (below) has to hold them all: 80 registers and the shared memory of the longest row, three
+// CTAs an SM, and its tiles ran at half the rate of the kernels made for one length (64 scans, 120 M pixels: 1343 us
+// against the launches' 990).
+//
+// Otherwise one persistent kernel.  Work is a list of tiles in ticket order.  A range tile runs the range-FFT tile
 // (fft_tile.cuh) on P = 4096/L pulses of one scan with the CTA's 256 threads; an
 // azimuth tile runs the gather-MAC tile (azimuth_tile.cuh) on 256*J outputs of one
 // row of one scan, or, for a scan given its frequency-domain plan H, the whole row
@@ -23,27 +30,13 @@
 #include <new>
 
 #include "azimuth_tile.cuh"
+#include "batch_rows.cuh"
 #include "fft_tile.cuh"
-#include "row_fft.cuh"
 
 namespace rosar {
 namespace {
 
 constexpr int BT_THREADS = 256;
-
-struct ScanDev {
-    const float2 *raw;
-    const float *win;
-    const float2 *w;
-    const int32_t *o;
-    float2 *S;
-    float2 *out;
-    const float2 *H;          // frequency-domain plan [L][n_az], or null: gather tiles
-    int o_row_stride, n_az, L, K;
-    int range_tiles, az_tiles_per_row, P, vec_store;
-    int fixed;                // compile-time plan of the row FFT (1: 1800, 2: 3600, 3: 7200 pulses), 0: run-time plan
-    rowfft::RowPlan plan;
-};
 
 struct Segment {
     int first;   // first ticket
@@ -283,6 +276,106 @@ int range_smem_bytes(int L) {
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Launches by length: the scans' indices sorted into groups of one length, and each group's first tile (or row) of
+// every scan.  More lengths than MAX_GROUPS take the persistent kernel.
+constexpr int MAX_GROUPS = 16;
+
+struct Groups {
+    int n = 0;                     // groups
+    int len[MAX_GROUPS], at[MAX_GROUPS], count[MAX_GROUPS], total[MAX_GROUPS];
+};
+
+// order, first: [n_scans] (host); length(s), tiles(s): of scan s.  false: too many lengths or tiles
+template <typename LEN, typename TILES>
+bool group_scans(int n_scans, LEN length, TILES tiles, Groups *g, int *order, int *first) {
+    for (int s = 0; s < n_scans; ++s) {
+        int i = 0;
+        while (i < g->n && g->len[i] != length(s)) ++i;
+        if (i == MAX_GROUPS) return false;
+        if (i == g->n) {
+            g->len[i] = length(s);
+            g->count[i] = 0;
+            ++g->n;
+        }
+        ++g->count[i];
+    }
+    int pos = 0;
+    for (int i = 0; i < g->n; ++i) {
+        long long t = 0;
+        g->at[i] = pos;
+        for (int s = 0; s < n_scans; ++s) {
+            if (length(s) != g->len[i]) continue;
+            order[pos] = s;
+            first[pos++] = (int)t;
+            t += tiles(s);
+            if (t > (1LL << 31) - 1) return false;
+        }
+        g->total[i] = (int)t;
+    }
+    return true;
+}
+
+// Launches of one stage side by side on up to four captured streams, joined on q[0].
+constexpr int GROUP_STREAMS = 4;
+
+template <typename F>
+rosar_status launch_groups(const Groups &g, cudaStream_t *q, cudaEvent_t *ev, F launch) {
+    const int used = g.n < GROUP_STREAMS ? g.n : GROUP_STREAMS;
+    cudaError_t e = cudaEventRecord(ev[0], q[0]);
+    for (int i = 1; i < used && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(q[i], ev[0], 0);
+    rosar_status st = ROSAR_OK;
+    for (int i = 0; i < g.n && e == cudaSuccess && st == ROSAR_OK; ++i) st = launch(i, q[i % GROUP_STREAMS]);
+    for (int i = 1; i < used && e == cudaSuccess; ++i) {
+        e = cudaEventRecord(ev[i], q[i]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(q[0], ev[i], 0);
+    }
+    if (e != cudaSuccess) return set_error(ROSAR_ERR_CUDA, "batch_create: graph capture: %s", cudaGetErrorString(e));
+    return st;
+}
+
+// The whole graph of the launches by length: captures into *graph and instantiates *exec.
+rosar_status capture_groups(const ScanDev *scans, const Groups &rg, const int *r_order, const int *r_first,
+                            const Groups &ag, const int *a_order, const int *a_first, cudaGraph_t *graph,
+                            cudaGraphExec_t *exec) {
+    auto range = [&](int i, cudaStream_t s, bool prepare) {
+        return launch_range_group(rg.len[i], ScanGroup{scans, r_order + rg.at[i], r_first + rg.at[i], rg.count[i]},
+                                  rg.total[i], s, prepare);
+    };
+    auto rows = [&](int i, cudaStream_t s, bool prepare) {
+        return launch_azimuth_group(ag.len[i], ScanGroup{scans, a_order + ag.at[i], a_first + ag.at[i], ag.count[i]},
+                                    ag.total[i], s, prepare);
+    };
+    rosar_status st = ROSAR_OK;
+    for (int i = 0; i < rg.n && st == ROSAR_OK; ++i) st = range(i, nullptr, true);
+    for (int i = 0; i < ag.n && st == ROSAR_OK; ++i) st = rows(i, nullptr, true);
+    if (st != ROSAR_OK) return st;
+    cudaStream_t q[GROUP_STREAMS] = {};
+    cudaEvent_t ev[GROUP_STREAMS] = {};
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < GROUP_STREAMS && e == cudaSuccess; ++i) {
+        e = cudaStreamCreateWithFlags(&q[i], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(q[0], cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        st = launch_groups(rg, q, ev, [&](int i, cudaStream_t s) { return range(i, s, false); });
+        if (st == ROSAR_OK) st = launch_groups(ag, q, ev, [&](int i, cudaStream_t s) { return rows(i, s, false); });
+        e = cudaStreamEndCapture(q[0], graph);
+        if (st != ROSAR_OK && e == cudaSuccess && *graph) cudaGraphDestroy(*graph);
+    }
+    if (st == ROSAR_OK && e == cudaSuccess) {
+        e = cudaGraphInstantiate(exec, *graph, 0);
+        if (e != cudaSuccess) cudaGraphDestroy(*graph);
+    }
+    for (int i = 0; i < GROUP_STREAMS; ++i) {
+        if (ev[i]) cudaEventDestroy(ev[i]);
+        if (q[i]) cudaStreamDestroy(q[i]);
+    }
+    if (st == ROSAR_OK && e != cudaSuccess)
+        st = set_error(ROSAR_ERR_CUDA, "batch_create: graph capture: %s", cudaGetErrorString(e));
+    return st;
+}
+
 }  // namespace
 }  // namespace rosar
 
@@ -345,6 +438,7 @@ rosar_status rosar_batch_create(const rosar_scan *scans, int n_scans, const rosa
         default: break;
     }
     long long total_range = 0, total_az = 0;
+    bool by_length = tn.interleave == 0 && tn.ctas_per_sm == 0 && tn.debug_unmet_scan < 0 && tn.flags == 0;
     rosar_status st = ROSAR_OK;
     for (int s = 0; s < n_scans && st == ROSAR_OK; ++s) {
         const rosar_scan &q = scans[s];
@@ -386,6 +480,7 @@ rosar_status rosar_batch_create(const rosar_scan *scans, int n_scans, const rosa
             const int rs = (int)(sizeof(float2) * (size_t)(rowfft::padded_len(q.n_az) + 64 + rowfft::coarse_len(q.n_az)));
             smem = smem > rs ? smem : rs;
         }
+        by_length = by_length && q.H;
         total_range += d.range_tiles;
         total_az += (long long)d.az_tiles_per_row * q.L;
     }
@@ -395,6 +490,48 @@ rosar_status rosar_batch_create(const rosar_scan *scans, int n_scans, const rosa
         free(hs);
         free(hg);
         return st;
+    }
+    char *ws = static_cast<char *>(workspace);
+    ScanDev *d_scans = reinterpret_cast<ScanDev *>(ws);
+    Segment *d_segs = reinterpret_cast<Segment *>(ws + align256(sizeof(ScanDev) * (size_t)n_scans));
+    int *d_cnt = reinterpret_cast<int *>(ws + align256(sizeof(ScanDev) * (size_t)n_scans) +
+                                         align256(sizeof(Segment) * SEGS_PER_SCAN * (size_t)n_scans));
+    if (by_length) {
+        // the groups' tables take the place of the segments: four ints a scan
+        static_assert(sizeof(Segment) * SEGS_PER_SCAN >= 4 * sizeof(int), "the tables fit the segments");
+        int *tab = reinterpret_cast<int *>(hg), *d_tab = reinterpret_cast<int *>(d_segs);
+        Groups rg, ag;
+        auto range_tiles = [&](int s) {
+            const int P = range_group_pulses(hs[s].L);
+            return (hs[s].n_az + P - 1) / P;
+        };
+        if (group_scans(n_scans, [&](int s) { return hs[s].L; }, range_tiles, &rg, tab, tab + n_scans) &&
+            group_scans(n_scans, [&](int s) { return hs[s].n_az; }, [&](int s) { return hs[s].L; }, &ag, tab + 2 * n_scans,
+                        tab + 3 * n_scans)) {
+            cudaError_t e = cudaMemcpy(d_scans, hs, sizeof(ScanDev) * (size_t)n_scans, cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = cudaMemcpy(d_tab, tab, 4 * sizeof(int) * (size_t)n_scans, cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = cudaMemset(d_cnt, 0, sizeof(int) * CNT_DONE);     // status: nothing here waits
+            free(hs);
+            free(hg);
+            if (e != cudaSuccess)
+                return set_error(ROSAR_ERR_CUDA, "batch_create: descriptor copy: %s", cudaGetErrorString(e));
+            rosar_batch *b = new (std::nothrow) rosar_batch();
+            if (!b) return set_error(ROSAR_ERR_INVALID_ARG, "batch_create: host allocation failed");
+            st = capture_groups(d_scans, rg, d_tab, d_tab + n_scans, ag, d_tab + 2 * n_scans, d_tab + 3 * n_scans,
+                                &b->graph, &b->exec);
+            if (st != ROSAR_OK) {
+                delete b;
+                return st;
+            }
+            b->counters = d_cnt;
+            b->n_scans = n_scans;
+            for (int i = 0; i < rg.n; ++i) b->range_tiles += rg.total[i];
+            b->az_tiles = (int)total_az;
+            b->ctas = b->range_tiles + b->az_tiles;
+            b->smem = smem;
+            *batch = b;
+            return ROSAR_OK;
+        }
     }
     // ticket order.  Azimuth tiles of a scan always come after all of its range tiles, so every range tile an
     // azimuth tile waits for has been handed to a running CTA (which waits on nothing) before it.
@@ -431,11 +568,6 @@ rosar_status rosar_batch_create(const rosar_scan *scans, int n_scans, const rosa
     }
     const int total = first;
 
-    char *ws = static_cast<char *>(workspace);
-    ScanDev *d_scans = reinterpret_cast<ScanDev *>(ws);
-    Segment *d_segs = reinterpret_cast<Segment *>(ws + align256(sizeof(ScanDev) * (size_t)n_scans));
-    int *d_cnt = reinterpret_cast<int *>(ws + align256(sizeof(ScanDev) * (size_t)n_scans) +
-                                         align256(sizeof(Segment) * SEGS_PER_SCAN * (size_t)n_scans));
     cudaError_t e = cudaMemcpy(d_scans, hs, sizeof(ScanDev) * (size_t)n_scans, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(d_segs, hg, sizeof(Segment) * (size_t)ns, cudaMemcpyHostToDevice);
     free(hs);

@@ -15,24 +15,48 @@
 //
 // Memory-bound: 16 algorithmic bytes per sample (8 read, 8 written).
 
+#include "batch_rows.cuh"
 #include "fft_tile.cuh"
 
 namespace rosar {
 namespace {
 
 // Pulses per CTA for the standalone kernel: small tiles give enough CTAs to cover
-// the memory latency at the scan sizes of interest.
+// the memory latency at the scan sizes of interest.  L = 1024 takes 8 pulses (stores of 64 bytes instead of 32) on 512
+// threads at 64 registers, two CTAs an SM: 14400 pulses 65.6 -> 55.6 us (one CTA an SM at 95 registers: 77).
 template <int L>
-struct Plan : fft::Tile<L, (L <= 16 ? 32 : L <= 64 ? 16 : L <= 256 ? 8 : L <= 1024 ? 4 : 2)> {};
+struct Plan : fft::Tile<L, (L <= 16 ? 32 : L <= 64 ? 16 : L <= 256 ? 8 : L == 512 ? 4 : L == 1024 ? 8 : 2)> {
+    static constexpr int MINB = L == 1024 ? 2 : 1;
+};
 
 template <int L>
-__global__ void __launch_bounds__(Plan<L>::THREADS)
+__global__ void __launch_bounds__(Plan<L>::THREADS, Plan<L>::MINB)
 range_compress_kernel(const float2 *__restrict__ raw, const float *__restrict__ win, int n_az, int centred,
                       float2 *__restrict__ S, int vec_store) {
     extern __shared__ float2 smem[];
     const size_t scan = (size_t)blockIdx.y * n_az * L;      // grid.y: scans of a stack
     fft::range_tile<L, Plan<L>::P>(raw + scan, win, n_az, centred != 0, S + scan, blockIdx.x * Plan<L>::P, smem, true,
                                    vec_store != 0);
+}
+
+// The same over the scans of a batch that have this length.
+template <int L>
+__global__ void __launch_bounds__(Plan<L>::THREADS, Plan<L>::MINB)
+range_group_kernel(ScanGroup g) {
+    extern __shared__ float2 smem[];
+    int tile;
+    const ScanDev &sc = g.find(blockIdx.x, tile);
+    fft::range_tile<L, Plan<L>::P>(sc.raw, sc.win, sc.n_az, true, sc.S, tile * Plan<L>::P, smem, true, sc.vec_store != 0);
+}
+
+template <int L>
+rosar_status launch_group_L(const ScanGroup &g, int total, cudaStream_t s, bool prepare) {
+    using PL = Plan<L>;
+    static int done[kMaxDevices] = {};
+    rosar_status st = ensure_smem((const void *)range_group_kernel<L>, PL::SMEM, done, "batch range compression");
+    if (st != ROSAR_OK || prepare) return st;
+    range_group_kernel<L><<<total, PL::THREADS, PL::SMEM, s>>>(g);
+    return check_launch("batch range compression");
 }
 
 template <int L>
@@ -93,6 +117,32 @@ rosar_status launch_range_compress(const float2 *raw, const float *win, int n_az
         case 2048: return launch_L<2048>(raw, win, n_az, centred, S, s, n_scans);
         case 4096: return launch_L<4096>(raw, win, n_az, centred, S, s, n_scans);
         default: return set_error(ROSAR_ERR_UNSUPPORTED, "range_compress: L=%d is not a power of two in [8, 4096]", L);
+    }
+}
+
+int range_group_pulses(int L) {
+    switch (L) {
+        case 16: return Plan<16>::P;
+        case 32: return Plan<32>::P;
+        case 64: return Plan<64>::P;
+        case 128: return Plan<128>::P;
+        case 256: return Plan<256>::P;
+        case 512: return Plan<512>::P;
+        case 1024: return Plan<1024>::P;
+        default: return Plan<2048>::P;
+    }
+}
+
+rosar_status launch_range_group(int L, const ScanGroup &g, int total, cudaStream_t s, bool prepare) {
+    switch (L) {
+        case 16: return launch_group_L<16>(g, total, s, prepare);
+        case 32: return launch_group_L<32>(g, total, s, prepare);
+        case 64: return launch_group_L<64>(g, total, s, prepare);
+        case 128: return launch_group_L<128>(g, total, s, prepare);
+        case 256: return launch_group_L<256>(g, total, s, prepare);
+        case 512: return launch_group_L<512>(g, total, s, prepare);
+        case 1024: return launch_group_L<1024>(g, total, s, prepare);
+        default: return launch_group_L<2048>(g, total, s, prepare);
     }
 }
 

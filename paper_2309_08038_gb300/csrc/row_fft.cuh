@@ -378,7 +378,7 @@ constexpr int last_radix() {
 // phase (optional, [N]): element n is multiplied by phase[n] as it is loaded (the per-pulse phase correction
 // of the differentiable form, S e^{j eps_n}, without a corrected copy of S in memory).
 template <int N, int R, int T, bool WAIT_ASYNC>
-__device__ __forceinline__ void dif_first_global(const float2 *__restrict__ src, float2 *x, const float2 *tc,
+__device__ __forceinline__ void dif_first_global(const float2 *src, float2 *x, const float2 *tc,
                                                  const float2 *tf, bool discard = false,
                                                  const float2 *__restrict__ phase = nullptr) {
     constexpr int s = N / R;
@@ -444,7 +444,7 @@ __device__ __forceinline__ void fused_mid(float2 *x, const float2 *h, float hs, 
 
 // Last DIT pass (M = N) written to global memory with the final conjugation of the inverse.
 template <int N, int R, int T>
-__device__ __forceinline__ void dit_last_global(const float2 *x, float2 *__restrict__ dst, const float2 *tc,
+__device__ __forceinline__ void dit_last_global(const float2 *x, float2 *dst, const float2 *tc,
                                                 const float2 *tf) {
     constexpr int s = N / R;
 #pragma unroll 1
@@ -473,13 +473,14 @@ __device__ __forceinline__ void filter_middle(float2 *x, const float2 *h, float 
     }
 }
 
-// src, dst: the row in global memory (natural order); x: N elements of shared memory (no padding); the
+// src, dst: the row in global memory (natural order), which may be the same row (every element is read before the
+// first barrier, written after the last); x: N elements of shared memory (no padding); the
 // caller has built the twiddle table and synchronised.  With H_SMEM, h may still be arriving by cp.async
 // when this starts (waited for at the end of the first pass).  No barrier at the end.  discard: src is
 // scratch, dropped from L2 once read (dif_first_global).
 template <int N, int T, bool H_SMEM, int R1, int... Rs>
-__device__ __forceinline__ void row_filter_fused(const float2 *__restrict__ src, const float2 *h, float hs, float2 *x,
-                                                 float2 *__restrict__ dst, const float2 *tc, const float2 *tf,
+__device__ __forceinline__ void row_filter_fused(const float2 *src, const float2 *h, float hs, float2 *x,
+                                                 float2 *dst, const float2 *tc, const float2 *tf,
                                                  bool discard = false, const float2 *__restrict__ phase = nullptr,
                                                  float2 *__restrict__ spec = nullptr) {
     static_assert(sizeof...(Rs) >= 1, "at least two passes");
@@ -556,8 +557,8 @@ constexpr size_t filter_row_smem() {
 }
 
 template <int T, int N, bool H_SMEM, int... R>
-__device__ __forceinline__ void filter_row_cta(const float2 *__restrict__ S_row, const float2 *__restrict__ H_row,
-                                               bool conj_h, float2 *__restrict__ out_row, float2 *sm,
+__device__ __forceinline__ void filter_row_cta(const float2 *S_row, const float2 *__restrict__ H_row,
+                                               bool conj_h, float2 *out_row, float2 *sm,
                                                const float2 *__restrict__ phase = nullptr,
                                                float2 *__restrict__ spec = nullptr) {
     static_assert(pad_shift_for(N) == 31, "compile-time filter plans are for rows with an odd factor");

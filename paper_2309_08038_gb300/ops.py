@@ -372,8 +372,8 @@ def image_fft(raw, win, H, workspace=None, out=None, stream=None):
 
 
 def image_fft_scans(raw, win, H, workspace=None, out=None, stream=None):
-    """rosar_image_fft_scans: rosar_image_fft of every scan of raw [n_scans, n_az, L] with one plan H [L, n_az],
-    consecutive scans overlapped where a pipelined plan exists; workspace [2, L, n_az], out [n_scans, L, n_az]."""
+    """rosar_image_fft_scans: rosar_image_fft of every scan of raw [n_scans, n_az, L] with one plan H [L, n_az], two
+    launches for all of them; workspace [2, L, n_az], out [n_scans, L, n_az]."""
     lib = _lib.load()
     require(raw, torch.complex64, "raw", ndim=3)
     n_scans, n_az, L = raw.shape
@@ -392,7 +392,7 @@ def image_fft_scans(raw, win, H, workspace=None, out=None, stream=None):
 
 
 def image_fft_scans_pipelined(L, n_az):
-    """rosar_image_fft_scans_pipelined: True if image_fft_scans overlaps consecutive scans for (L, n_az)."""
+    """rosar_image_fft_scans_pipelined: True for the (L, n_az) that once had a pipelined kernel of their own."""
     return bool(_lib.load().rosar_image_fft_scans_pipelined(int(L), int(n_az)))
 
 
