@@ -46,4 +46,27 @@ __device__ __forceinline__ float2 read_bin(const float2 *__restrict__ S, int l, 
     return (l >= 0 && l < L) ? __ldg(S + (size_t)l * n_az + col) : make_float2(0.f, 0.f);
 }
 
+// Sample at bin x of pulse (n mod n_az): from the staged rows [wlo, wtop) of its column (row pitch `pitch`) where they
+// hold its bins, else through L2.
+template <bool LINEAR>
+__device__ __forceinline__ float2 sample_anywhere(const float2 *__restrict__ S, const float2 *col, int pitch, int wlo,
+                                                  int wtop, float x, int L, int n_az, int n) {
+    if (LINEAR) {
+        const float fl = floorf(x);
+        const int l0 = (int)fl;
+        float2 s0, s1;
+        if (l0 >= wlo && l0 + 1 < wtop) {
+            s0 = col[(l0 - wlo) * pitch];
+            s1 = col[(l0 + 1 - wlo) * pitch];
+        } else {
+            const int m = pmod(n, n_az);
+            s0 = read_bin(S, l0, L, m, n_az);
+            s1 = read_bin(S, l0 + 1, L, m, n_az);
+        }
+        return caxpy(x - fl, csub(s1, s0), s0);
+    }
+    const int l0 = (int)floorf(x + 0.5f);
+    return (l0 >= wlo && l0 < wtop) ? col[(l0 - wlo) * pitch] : read_bin(S, l0, L, pmod(n, n_az), n_az);
+}
+
 }  // namespace rosar
