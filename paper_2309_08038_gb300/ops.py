@@ -128,9 +128,8 @@ def image_fft_host(raw_host, win, H, raw_dev, workspace, out_dev, out_host, stre
     require(raw_dev, torch.complex64, "raw_dev", shape=(n_az, L))
     require(workspace, torch.complex64, "workspace", shape=(L, n_az))
     require(out_dev, torch.complex64, "out_dev", shape=(L, n_az))
-    check(lib.rosar_image_fft_host(ctypes.c_void_p(raw_host.data_ptr()), ptr(win), ptr(H), n_az, L, ptr(raw_dev),
-                                   ptr(workspace), ptr(out_dev), ctypes.c_void_p(out_host.data_ptr()),
-                                   stream_handle(stream)))
+    check(lib.rosar_image_fft_host(ptr(raw_host), ptr(win), ptr(H), n_az, L, ptr(raw_dev), ptr(workspace),
+                                   ptr(out_dev), ptr(out_host), stream_handle(stream)))
     return out_host
 
 
