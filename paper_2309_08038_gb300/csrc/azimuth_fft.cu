@@ -1,29 +1,9 @@
-// K2b: the sparse-aperture azimuth filter of Eq. (43) evaluated exactly as a circular
-// convolution in the azimuth-frequency domain (arXiv 2309.08038, Sec. III-D; the
-// pixel-parallel form of Remark 2, here per range row):
-//
-//   out[r][.] = sum_k w[r][k] * S[r][(. + o_k) mod N] = g_r (*) S[r][.],   g_r[(-o_k) mod N] += w[r][k]
-//            = IFFT_N( FFT_N(g_r)/N . FFT_N(S[r][.]) )
-//
-// The same taps, the same circular modulo; only the summation order differs from the
-// gather form.  Work per pixel is O(log N) instead of O(K), so at K >= 32 the
-// azimuth stage turns from shared-memory/FMA bound to HBM bound (24 B/px: S, H, out).
-//
-// One CTA owns one range row, staged in shared memory (one pad element per 16
-// against bank conflicts).  The forward transform is an in-place mixed-radix
-// decimation-in-frequency FFT (radices 16, 8, 4, 2, 5, 3 and a prime-factor 15; N = 2^a 3^b 5^c <= 16384;
-// a planner picks the sequence with the fewest passes, e.g. 3600 = 16*15*15).
-// Every butterfly reads and writes the same R slots, so only its own R values are
-// live and passes need one barrier each; its twiddles are powers of one table entry.  It leaves the spectrum in digit-reversed
-// order; H is produced by the same transform (so it is stored in that order), the
-// pointwise product needs no reordering, and the inverse is the transposed
-// (decimation-in-time) pass sequence between two conjugations, which restores the
-// natural order.  Twiddles exp(-2*pi*i*q/N) come from a two-level shared table
-// (q >> 6, q & 63) built per CTA with sincospif.
+// Plans and weight gradients of the frequency-domain azimuth filter (azimuth_rows.cu): the transfer functions H
+// of a weight design, and the gradient of the filter in its weights from the rows' cross-spectrum.
 
 #include <cooperative_groups.h>
 
-#include "batch_rows.cuh"
+#include "azimuth_layout.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -32,121 +12,10 @@ namespace {
 
 using namespace rowfft;
 
-// Shared-memory layout of a row: x [padded], then (stage_h) the H row [padded], then the twiddle table.
-struct Layout {
-    int full_tab;
-    int stage_h;
-    size_t bytes;
-};
-
-// What one CTA filters: a row of S through a row of H (conj_h: conj(H), the adjoint filter) into a row of out, which
-// may be the row of S itself.  phase (optional): [N] per-column factors applied as the row is loaded.  spec (optional):
-// [N] receives the row's forward transform (digit-reversed order, before the product with H), for the weight gradient.
-struct RowRef {
-    const float2 *S, *H;
-    float2 *out;
-    bool conj_h;
-    const float2 *phase;
-    float2 *spec;
-};
-
-// Rows of a stack: row b of S and out uses row (b mod h_rows) of H (a stack of scans sharing one plan) and phase row
-// b / h_rows (each scan its own phase correction); phase [n_rows / h_rows][N], spec [n_rows][N].
-struct StackRows {
-    const float2 *S, *H;
-    float2 *out;
-    int h_rows, conj_h;
-    const float2 *phase;
-    float2 *spec;
-
-    __device__ __forceinline__ RowRef at(int b, int N) const {
-        const size_t row = (size_t)b * N;
-        return RowRef{S + row, H + (size_t)(b % h_rows) * N, out + row, conj_h != 0,
-                      phase ? phase + (size_t)(b / h_rows) * N : nullptr, spec ? spec + row : nullptr};
-    }
-};
-
-// Rows of the scans of a batch that have this length, each scan with its own plan.
-struct BatchRows {
-    ScanGroup g;
-
-    __device__ __forceinline__ RowRef at(int b, int N) const {
-        int r;
-        const ScanDev &sc = g.find(b, r);
-        const size_t row = (size_t)r * N;
-        return RowRef{sc.S + row, sc.H + row, sc.out + row, false, nullptr, nullptr};
-    }
-};
-
-// The row filter on one CTA: stage the H row and the twiddle table, wait for S, forward DIF, product with
-// H (digit-reversed order, carries 1/N) between conjugations, DIT, store.
-template <typename ROWS, int MAXT>
-__global__ void __launch_bounds__(MAXT, (MAXT == 384 ? 2 : 1))
-azimuth_fft_kernel(ROWS rows, int N, RowPlan pl, Layout lay) {
-    extern __shared__ float2 sm[];
-    const int pad_shift = pl.pad_shift;
-    float2 *x = sm;
-    float2 *hb = x + padded_len(N);
-    float2 *tw = lay.stage_h ? hb + padded_len(N) : hb;
-    const RowRef ref = rows.at(blockIdx.x, N);
-    const float hs = ref.conj_h ? -1.f : 1.f;
-    // prologue independent of S: the H row and the twiddle table
-    if (lay.stage_h)
-        for (int n = threadIdx.x; n < N; n += blockDim.x) cp_async8(hb + rpad(n, pad_shift), ref.H + n);
-    cp_async_commit();
-    const float2 *tc, *tf;
-    build_twiddles(N, lay.full_tab != 0, tw, &tc, &tf);
-    griddep_wait();                          // S is complete (no-op unless launched to overlap its producer)
-    for (int n = threadIdx.x; n < N; n += blockDim.x) cp_async8(x + rpad(n, pad_shift), ref.S + n);
-    cp_async_commit();
-    cp_async_wait<0>();
-    if (ref.phase)                           // each thread scales the elements it staged
-        for (int n = threadIdx.x; n < N; n += blockDim.x)
-            x[rpad(n, pad_shift)] = cmul(x[rpad(n, pad_shift)], __ldg(ref.phase + n));
-    __syncthreads();
-    row_dif(x, N, pl, tc, tf);
-    if (ref.spec)
-        for (int n = threadIdx.x; n < N; n += blockDim.x) ref.spec[n] = x[rpad(n, pad_shift)];
-    if (lay.stage_h) {
-        for (int n = threadIdx.x; n < N; n += blockDim.x) {   // spectrum times H (same digit-reversed order, carries 1/N), conjugated
-            float2 h = hb[rpad(n, pad_shift)];
-            h.y *= hs;
-            const float2 y = cmul(h, x[rpad(n, pad_shift)]);
-            x[rpad(n, pad_shift)] = make_float2(y.x, -y.y);
-        }
-    } else {
-#pragma unroll 4
-        for (int n = threadIdx.x; n < N; n += blockDim.x) {
-            float2 h = __ldg(ref.H + n);
-            h.y *= hs;
-            const float2 y = cmul(h, x[rpad(n, pad_shift)]);
-            x[rpad(n, pad_shift)] = make_float2(y.x, -y.y);
-        }
-    }
-    __syncthreads();
-    row_dit(x, N, pl, tc, tf);
-    for (int n = threadIdx.x; n < N; n += blockDim.x) {
-        const float2 y = x[rpad(n, pad_shift)];
-        ref.out[n] = make_float2(y.x, -y.y);
-    }
-}
-
-// Compile-time plan for one row length (T threads, no padding: N has an odd factor): the first pass reads S from
-// global memory, the last writes the image, and the last forward pass, the product with H and the first inverse pass
-// run as one step (row_filter_fused): four barriers for 16.15.15.  H_SMEM: the H row staged by cp.async before S is
-// there; otherwise the fused step reads it from global memory.
-template <typename ROWS, int T, int MINB, int N, bool H_SMEM, int... R>
-__global__ void __launch_bounds__(T, MINB)
-azimuth_fft_fixed_kernel(ROWS rows) {
-    extern __shared__ float2 sm[];
-    const RowRef ref = rows.at(blockIdx.x, N);
-    filter_row_cta<T, N, H_SMEM, R...>(ref.S, ref.H, ref.conj_h, ref.out, sm, ref.phase, ref.spec);
-}
-
 // dl != nullptr: plane blockIdx.y of the range-migration-aware plan, built from the taps of row r whose row
 // offset dl[r][k] equals d_lo + blockIdx.y, stored at H[(blockIdx.y * gridDim.x + r) * N].
 template <int MAXT>
-__global__ void __launch_bounds__(MAXT, (MAXT == 384 ? 2 : 1))
+__global__ void __launch_bounds__(MAXT, 1)
 azimuth_plan_kernel(const float2 *__restrict__ w, const int32_t *__restrict__ o, int o_row_stride, int K, int N,
                     RowPlan pl, Layout lay, float2 *__restrict__ H, const int32_t *__restrict__ dl = nullptr,
                     int d_lo = 0) {
@@ -370,28 +239,14 @@ xspec_taps_fixed_kernel(const float2 *__restrict__ P, const int32_t *__restrict_
                    [](float2 *x, const float2 *tc, const float2 *tf) { dit_seq<N, N, false, T, R...>(x, tc, tf); });
 }
 
-constexpr size_t AF_SMEM_CAP = 200 * 1024;
-
-Layout layout_for(int N, bool with_h) {
-    Layout l{};
-    const size_t row = sizeof(float2) * (size_t)padded_len(N);
-    const size_t two = sizeof(float2) * (size_t)(64 + coarse_len(N));
-    l.stage_h = with_h && (2 * row + two <= AF_SMEM_CAP);
-    l.full_tab = 0;      // two-level table: ~N/64 + 64 sincospif per CTA instead of N
-    l.bytes = row * (l.stage_h ? 2 : 1) + two;
-    return l;
-}
-
-template <typename F256, typename F384, typename F512, typename F1024>
-rosar_status launch_rows(int N, int rows, size_t sm, F256 f256, F384 f384, F512 f512, F1024 f1024,
-                         const void *const k[4], int (*done)[kMaxDevices], const char *what) {
+template <typename F256, typename F512, typename F1024>
+rosar_status launch_rows(int N, int rows, size_t sm, F256 f256, F512 f512, F1024 f1024, const void *const k[3], int (*done)[kMaxDevices], const char *what) {
     const int T = threads_for(N);
-    const int v = T <= 256 ? 0 : T <= 384 ? 1 : T <= 512 ? 2 : 3;
+    const int v = T <= 256 ? 0 : T <= 512 ? 1 : 2;
     rosar_status st = ensure_smem(k[v], sm, done[v], what);
     if (st != ROSAR_OK) return st;
     if (v == 0) f256(rows, T, sm);
-    else if (v == 1) f384(rows, T, sm);
-    else if (v == 2) f512(rows, T, sm);
+    else if (v == 1) f512(rows, T, sm);
     else f1024(rows, T, sm);
     return check_launch(what);
 }
@@ -401,102 +256,6 @@ rosar_status launch_rows(int N, int rows, size_t sm, F256 f256, F384 f384, F512 
 int azimuth_fft_supported(int n_az) {
     RowPlan pl;
     return make_plan(n_az, &pl) ? 1 : 0;
-}
-
-namespace {
-
-template <typename K, typename... A>
-cudaError_t launch_overlapped(K kernel, int grid, int threads, size_t smem, bool overlap, cudaStream_t s, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
-// One launch of a row filter over n_rng rows; `only_prepare`: set the kernel's shared-memory limit and launch nothing.
-struct RowLaunch {
-    int n_az, n_rng;
-    bool overlap, only_prepare;
-    cudaStream_t s;
-};
-
-template <typename ROWS, int T, int MINB, int N, bool H_SMEM, int... R>
-rosar_status launch_fixed(const RowLaunch &l, const ROWS &rows) {
-    static int done[kMaxDevices] = {};
-    constexpr size_t smem = filter_row_smem<N, H_SMEM>();
-    static_assert(smem <= 200 * 1024, "the staged rows exceed the shared-memory cap");
-    const auto kernel = azimuth_fft_fixed_kernel<ROWS, T, MINB, N, H_SMEM, R...>;
-    rosar_status st = ensure_smem((const void *)kernel, smem, done, "azimuth_fft");
-    if (st != ROSAR_OK || l.only_prepare) return st;
-    const cudaError_t e = launch_overlapped(kernel, l.n_rng, T, smem, l.overlap, l.s, rows);
-    if (e != cudaSuccess) return set_error(ROSAR_ERR_CUDA, "azimuth_fft: launch failed: %s", cudaGetErrorString(e));
-    return check_launch("azimuth_fft");
-}
-
-// Whether the run-time planner picks exactly these radices for n_az (H, made by the run-time plan, is in their order).
-template <int N, int... R>
-bool plan_is(int n_az, const RowPlan &pl) {
-    constexpr int rad[] = {R...};
-    if (n_az != N || pl.pad_shift != 31 || pl.npass != (int)sizeof...(R)) return false;
-    for (int i = 0; i < pl.npass; ++i)
-        if (pl.rad[i] != rad[i]) return false;
-    return true;
-}
-
-// Up to two rows an SM, a row's own latency counts: 256 threads and H staged while S is awaited.  With more the SM's
-// rows in flight count: one row of shared memory and at most 64 registers hold 4 CTAs of 3600 pulses (46 % of the
-// warps instead of 30) or 8 of 1800, and H is read in the fused step.  4096 rows of 3600 pulses 82 -> 77 us, 8192 of
-// 1800 97 -> 76; at 256 rows 10.3 and 10.4, 6.4 and 8.2.  7200-pulse rows hold one CTA an SM with H staged: 256 rows
-// 20.5 -> 16.6 us, 2048 rows 141 -> 100.
-constexpr int kFewRows = 304;
-
-template <typename ROWS>
-rosar_status launch_rows_of(const RowLaunch &l, const ROWS &rows) {
-    RowPlan pl;
-    if (!make_plan(l.n_az, &pl))
-        return set_error(ROSAR_ERR_UNSUPPORTED, "azimuth_fft: n_az=%d is not 2^a 3^b 5^c in [2, %d]", l.n_az, AF_MAX_N);
-    const bool few = l.n_rng <= kFewRows;
-    if (plan_is<3600, 16, 15, 15>(l.n_az, pl))
-        return few ? launch_fixed<ROWS, 256, 2, 3600, true, 16, 15, 15>(l, rows)
-                   : launch_fixed<ROWS, 256, 4, 3600, false, 16, 15, 15>(l, rows);
-    if (plan_is<1800, 8, 15, 15>(l.n_az, pl))
-        return few ? launch_fixed<ROWS, 256, 2, 1800, true, 8, 15, 15>(l, rows)
-                   : launch_fixed<ROWS, 128, 8, 1800, false, 8, 15, 15>(l, rows);
-    if (plan_is<7200, 8, 4, 15, 15>(l.n_az, pl)) return launch_fixed<ROWS, 256, 3, 7200, false, 8, 4, 15, 15>(l, rows);
-    if (plan_is<14400, 8, 8, 15, 15>(l.n_az, pl))
-        return launch_fixed<ROWS, 1024, 1, 14400, false, 8, 8, 15, 15>(l, rows);
-    if (plan_is<360, 8, 3, 15>(l.n_az, pl))
-        return few ? launch_fixed<ROWS, 256, 2, 360, true, 8, 3, 15>(l, rows)
-                   : launch_fixed<ROWS, 64, 8, 360, false, 8, 3, 15>(l, rows);
-    const Layout lay = layout_for(l.n_az, true);
-    static int done[3][kMaxDevices] = {};
-    const int T = threads_for(l.n_az), v = T <= 256 ? 0 : T <= 512 ? 1 : 2;
-    const auto kernel = v == 0 ? azimuth_fft_kernel<ROWS, 256> : v == 1 ? azimuth_fft_kernel<ROWS, 512>
-                                                                       : azimuth_fft_kernel<ROWS, 1024>;
-    rosar_status st = ensure_smem((const void *)kernel, lay.bytes, done[v], "azimuth_fft");
-    if (st != ROSAR_OK || l.only_prepare) return st;
-    const cudaError_t e = launch_overlapped(kernel, l.n_rng, T, lay.bytes, l.overlap, l.s, rows, l.n_az, pl, lay);
-    if (e != cudaSuccess) return set_error(ROSAR_ERR_CUDA, "azimuth_fft: launch failed: %s", cudaGetErrorString(e));
-    return check_launch("azimuth_fft");
-}
-
-}  // namespace
-
-rosar_status launch_azimuth_fft(const float2 *S, const float2 *H, int n_rng, int n_az, float2 *out, cudaStream_t s,
-                                bool overlap_predecessor, int h_rows, bool conj_h, const float2 *phase, float2 *spec) {
-    return launch_rows_of(RowLaunch{n_az, n_rng, overlap_predecessor, false, s},
-                          StackRows{S, H, out, h_rows > 0 ? h_rows : n_rng, conj_h ? 1 : 0, phase, spec});
-}
-
-rosar_status launch_azimuth_group(int n_az, const ScanGroup &g, int total, cudaStream_t s, bool prepare) {
-    return launch_rows_of(RowLaunch{n_az, total, false, prepare, s}, BatchRows{g});
 }
 
 namespace {
@@ -559,13 +318,12 @@ rosar_status launch_azimuth_weight_grad_fft(const float2 *g, const float2 *S_t, 
     const size_t bytes = sizeof(float2) * (3 * (size_t)padded_len(n_az) + 64 + coarse_len(n_az));
     if (bytes > AF_SMEM_CAP)
         return set_error(ROSAR_ERR_UNSUPPORTED, "weight_grad_fft: n_az=%d needs %zu bytes of shared memory", n_az, bytes);
-    static int done[4][kMaxDevices] = {};
-    static const void *const ks[4] = {(const void *)azimuth_xspec_kernel<256>, (const void *)azimuth_xspec_kernel<384>,
+    static int done[3][kMaxDevices] = {};
+    static const void *const ks[3] = {(const void *)azimuth_xspec_kernel<256>,
                                       (const void *)azimuth_xspec_kernel<512>, (const void *)azimuth_xspec_kernel<1024>};
     return launch_rows(
         n_az, n_rng, bytes,
         [&](int gr, int t, size_t sm) { azimuth_xspec_kernel<256><<<gr, t, sm, s>>>(g, S_t, o, o_row_stride, n_scans, n_rng, K, n_az, pl, grad_w, phase); },
-        [&](int gr, int t, size_t sm) { azimuth_xspec_kernel<384><<<gr, t, sm, s>>>(g, S_t, o, o_row_stride, n_scans, n_rng, K, n_az, pl, grad_w, phase); },
         [&](int gr, int t, size_t sm) { azimuth_xspec_kernel<512><<<gr, t, sm, s>>>(g, S_t, o, o_row_stride, n_scans, n_rng, K, n_az, pl, grad_w, phase); },
         [&](int gr, int t, size_t sm) { azimuth_xspec_kernel<1024><<<gr, t, sm, s>>>(g, S_t, o, o_row_stride, n_scans, n_rng, K, n_az, pl, grad_w, phase); },
         ks, done, "weight_grad_fft");
@@ -606,13 +364,12 @@ rosar_status launch_azimuth_weight_grad_spectra(const float2 *G, const float2 *X
         try_xspec_taps_fixed<256, 360, 8, 3, 15>(n_az, pl, P, o, o_row_stride, n_rng, K, grad_w, s, &st))
         return st;
     const size_t bytes = sizeof(float2) * ((size_t)padded_len(n_az) + 64 + coarse_len(n_az));
-    static int done[4][kMaxDevices] = {};
-    static const void *const ks[4] = {(const void *)xspec_taps_kernel<256>, (const void *)xspec_taps_kernel<384>,
+    static int done[3][kMaxDevices] = {};
+    static const void *const ks[3] = {(const void *)xspec_taps_kernel<256>,
                                       (const void *)xspec_taps_kernel<512>, (const void *)xspec_taps_kernel<1024>};
     return launch_rows(
         n_az, n_rng, bytes,
         [&](int gr, int t, size_t sm) { xspec_taps_kernel<256><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, grad_w); },
-        [&](int gr, int t, size_t sm) { xspec_taps_kernel<384><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, grad_w); },
         [&](int gr, int t, size_t sm) { xspec_taps_kernel<512><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, grad_w); },
         [&](int gr, int t, size_t sm) { xspec_taps_kernel<1024><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, grad_w); },
         ks, done, "weight_grad_spectra");
@@ -623,15 +380,14 @@ rosar_status launch_azimuth_plan(const float2 *w, const int32_t *o, int o_row_st
     RowPlan pl;
     if (!make_plan(n_az, &pl))
         return set_error(ROSAR_ERR_UNSUPPORTED, "azimuth_plan: n_az=%d is not 2^a 3^b 5^c in [2, %d]", n_az, AF_MAX_N);
-    static int done[4][kMaxDevices] = {};
+    static int done[3][kMaxDevices] = {};
     const Layout lay = layout_for(n_az, false);
-    static const void *const ks[4] = {(const void *)azimuth_plan_kernel<256>, (const void *)azimuth_plan_kernel<384>,
+    static const void *const ks[3] = {(const void *)azimuth_plan_kernel<256>,
                                       (const void *)azimuth_plan_kernel<512>, (const void *)azimuth_plan_kernel<1024>};
     const dim3 grid(n_rng, dl ? n_d : 1);
     return launch_rows(
         n_az, n_rng, lay.bytes,
         [&](int, int t, size_t sm) { azimuth_plan_kernel<256><<<grid, t, sm, s>>>(w, o, o_row_stride, K, n_az, pl, lay, H, dl, d_lo); },
-        [&](int, int t, size_t sm) { azimuth_plan_kernel<384><<<grid, t, sm, s>>>(w, o, o_row_stride, K, n_az, pl, lay, H, dl, d_lo); },
         [&](int, int t, size_t sm) { azimuth_plan_kernel<512><<<grid, t, sm, s>>>(w, o, o_row_stride, K, n_az, pl, lay, H, dl, d_lo); },
         [&](int, int t, size_t sm) { azimuth_plan_kernel<1024><<<grid, t, sm, s>>>(w, o, o_row_stride, K, n_az, pl, lay, H, dl, d_lo); },
         ks, done, "azimuth_plan");
