@@ -55,11 +55,12 @@ __device__ __forceinline__ int tap_offset(const int32_t *o, int n) {
     return canon_offset((int)m, n);
 }
 
-// COHERENT: S was written earlier in the same kernel (read through L2, not the non-coherent path).
+// COHERENT: S was written earlier in the same kernel (read through L2).  Otherwise it may have been written by a kernel
+// that this one overlaps: after the grid-dependency wait, but not by the non-coherent path.
 template <bool COHERENT>
 __device__ __forceinline__ float2 load_s(const float2 *p) {
     if (COHERENT) return __ldcg(p);
-    return __ldg(p);
+    return __ldca(p);
 }
 
 // `smem` holds Geo<J>::SMEM_BYTES bytes (GeoMig<J> when MIG); `red` 4*THREADS/32 ints.  Called by all
@@ -141,6 +142,7 @@ __device__ __forceinline__ void azimuth_tile(const float2 *__restrict__ S, const
     const long long nrows = MIG ? (long long)dhi - dlo + 1 : 1;
     const bool staged = MIG ? (span <= SPAN_CAP && nrows <= MIG_ROWS && nrows * wl <= WIN) : span <= SPAN_CAP;
 
+    griddep_wait();    // S is complete (no-op unless launched to overlap its producer, which writes neither o nor w)
     if (staged) {
         const int start = pmod(th0 + lo, n_az);
         for (int q = 0; q < (int)nrows; ++q) {

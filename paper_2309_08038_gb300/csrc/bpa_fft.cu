@@ -120,7 +120,7 @@ bpa_rows_kernel(const float2 *__restrict__ S, BpaParams p, int L, int n_az, int 
                     const int e = j + i * s1;
                     int n = e + off;
                     n += n < 0 ? n_az : n >= n_az ? -n_az : 0;
-                    v[i] = e < len ? __ldg(row + n) : make_float2(0.f, 0.f);
+                    v[i] = e < len ? __ldcg(row + n) : make_float2(0.f, 0.f);
                 }
 #pragma unroll
                 for (int i = 0; i < R1; ++i) bad |= !(fabsf(v[i].x) + fabsf(v[i].y) < kSpreadLimit);

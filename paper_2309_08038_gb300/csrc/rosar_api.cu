@@ -453,7 +453,7 @@ rosar_status rosar_image(const rosar_c32 *raw, const float *win, const rosar_c32
                                reinterpret_cast<float2 *>(workspace), s);
     if (st != ROSAR_OK) return st;
     return launch_sparse_azimuth(reinterpret_cast<const float2 *>(workspace), reinterpret_cast<const float2 *>(w), o,
-                                 o_row_stride, L, n_az, K, reinterpret_cast<float2 *>(out), s);
+                                 o_row_stride, L, n_az, K, reinterpret_cast<float2 *>(out), s, true);
 }
 
 int rosar_azimuth_fft_supported(int n_az) { return azimuth_fft_supported(n_az); }

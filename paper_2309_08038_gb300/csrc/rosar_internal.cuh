@@ -66,8 +66,10 @@ __device__ __forceinline__ int pmod(int a, int n) {
 rosar_status launch_range_compress(const float2 *raw, const float *win, int n_az, int L, int centred,
                                    float2 *S, cudaStream_t s, int n_scans = 1);
 
+// overlap_predecessor: as launch_azimuth_fft's (the kernel before writes S, not w or o).
 rosar_status launch_sparse_azimuth(const float2 *S, const float2 *w, const int32_t *o, int o_row_stride,
-                                   int n_rng, int n_az, int K, float2 *out, cudaStream_t s);
+                                   int n_rng, int n_az, int K, float2 *out, cudaStream_t s,
+                                   bool overlap_predecessor = false);
 
 // Range-migration-aware taps: tap k of row r reads row r + dl[r][k] of S (n_bins rows).
 rosar_status launch_sparse_azimuth_migrating(const float2 *S, int n_bins, const float2 *w, const int32_t *o,

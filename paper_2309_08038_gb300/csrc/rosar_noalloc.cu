@@ -83,5 +83,5 @@ extern "C" rosar_status rosar_image_noalloc(const rosar_c32 *raw, const float *w
     st = launch_range_compress(reinterpret_cast<const float2 *>(raw), win, n_az, L, 1, S, s);
     if (st != ROSAR_OK) return st;
     return launch_sparse_azimuth(S, reinterpret_cast<const float2 *>(w), o, o_row_stride, L, n_az, K,
-                                 reinterpret_cast<float2 *>(out), s);
+                                 reinterpret_cast<float2 *>(out), s, true);
 }

@@ -444,7 +444,7 @@ lr_combine_kernel(const float2 *__restrict__ X, const uint8_t *__restrict__ plan
     for (int q = 0; q < P; ++q) {
         float2 v[16];
 #pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = cmul(x[r], __ldg(W + q * LF + t + r * C::T));
+        for (int r = 0; r < 16; ++r) v[r] = cmul(x[r], __ldca(W + q * LF + t + r * C::T));
         col_dft<LF, 16, 1>(v, t, tw);
         auto exchange = [&](auto R_, auto NS_, auto RN_, bool first) {
             constexpr int R = decltype(R_)::value, NS = decltype(NS_)::value, RN = decltype(RN_)::value;
@@ -496,7 +496,7 @@ __device__ __noinline__ void write_marked(const uint8_t *__restrict__ flags, con
     for (int th = threadIdx.x; th < sh.n_az; th += blockDim.x) {
         int hit = 0;
         for (int k = 0; k < sh.K && !hit; ++k) {
-            const int n = pmod(th + __ldg(offs + k), sh.n_az);
+            const int n = pmod(th + __ldca(offs + k), sh.n_az);
             for (int c = 0; c * TURN_SAMPLES < sh.L; ++c) hit |= flags[(size_t)c * sh.n_az + n];
         }
         if (hit) out_row[th] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
