@@ -17,192 +17,246 @@
 //   kernel 1 X[b] = DIF(S[b]) for every row b of S (the forward transform, same order);
 //   kernel 2 Y_r = sum_d X[r+d] . H_d[r] in increasing d, then conj, DIT, conj (the
 //            inverse, natural order), written to out[r].
-// Rows with a compile-time plan (360, 1800, 3600, 7200 pulses) run the pass sequence with
-// constant strides, the first and last passes of each transform on global memory, the
-// inverse launched to overlap the forward kernel's tail; the others the run-time plan.
+// Every transform's outer pass runs on global memory where it can; the products are formed over consecutive elements
+// (the plans' planes and the spectra are both in digit-reversed order), eight elements a thread and plane in flight.
+// Each kernel is launched to overlap the one before it, and the second asks for its planes of H ahead of the wait,
+// since they come from DRAM.  Bound by latency where the grid is short (256 rows of 3600 pulses are under two CTAs an
+// SM), by the planes of H and the spectra (8 bytes each a plane and pixel) where it is long.  Against products formed
+// per butterfly (strided reads of H and X), staged rows with run-time plans and no overlap of the first kernel: 3600
+// pulses, three planes, 256 rows 20.4 -> 13.0 us, 512 rows 34.8 -> 20.4; 7200 x 256 43.8 -> 28.3; run-time plans 2048
+// x 1024 81 -> 36, 12000 x 128 46.5 -> 32.2, 480 x 256 10.6 -> 9.7.
 
-#include "row_fft.cuh"
+#include "azimuth_layout.cuh"
 
 namespace rosar {
 namespace {
 
 using namespace rowfft;
 
-// One CTA per S row: stage the row (cp.async), build the twiddle table, forward transform, store.
-template <typename FWD>
-__device__ __forceinline__ void spectrum_row(const float2 *__restrict__ S, float2 *__restrict__ X, int N, int pad_shift,
-                                             FWD fwd) {
-    extern __shared__ float2 sm[];
-    float2 *x = sm;
-    float2 *tw = x + padded_len(N);
-    const size_t row = (size_t)blockIdx.x * N;
-    for (int n = threadIdx.x; n < N; n += blockDim.x) cp_async8(x + rpad(n, pad_shift), S + row + n);
-    cp_async_commit();
-    const float2 *tc, *tf;
-    build_twiddles(N, false, tw, &tc, &tf);
-    cp_async_wait<0>();
-    __syncthreads();
-    fwd(x, tc, tf);                                  // ends with a barrier
-    for (int n = threadIdx.x; n < N; n += blockDim.x) X[row + n] = x[rpad(n, pad_shift)];
+// ---- the two halves around the transforms
+
+template <int T>
+__device__ __forceinline__ void store_row(const float2 *x, float2 *__restrict__ X, int N, int pad_shift) {
+    for (int n = threadIdx.x; n < N; n += T) X[n] = x[rpad(n, pad_shift)];
 }
 
-// One CTA per output row r: the planes' products summed in increasing d (each thread owns its frequencies,
-// so no barrier between planes), conjugated, inverse transform, conjugated store.
-template <typename INV>
-__device__ __forceinline__ void combine_row(const float2 *__restrict__ X, const float2 *__restrict__ H, int n_bins,
-                                            int n_rng, int d_lo, int n_d, int N, int pad_shift, float2 *__restrict__ out,
-                                            INV inv) {
-    extern __shared__ float2 sm[];
-    float2 *x = sm;
-    float2 *tw = x + padded_len(N);
-    const int r = blockIdx.x;
-    const float2 *tc, *tf;
-    build_twiddles(N, false, tw, &tc, &tf);
-    for (int n = threadIdx.x; n < N; n += blockDim.x) {
-        float2 acc = make_float2(0.f, 0.f);
-        bool any = false;
-        for (int i = 0; i < n_d; ++i) {
-            const int b = r + d_lo + i;
-            if (b < 0 || b >= n_bins) continue;
-            const float2 p = cmul(__ldg(H + ((size_t)i * n_rng + r) * N + n), __ldg(X + (size_t)b * N + n));
-            acc = any ? cadd(acc, p) : p;
-            any = true;
+// x = conj(sum_d H_d[r] . X[r + d]) over the planes whose rows exist, in increasing d; ends without a barrier.
+struct Planes {
+    const float2 *X, *H;
+    int n_bins, n_rng, d_lo, n_d;
+};
+
+__device__ __forceinline__ void prefetch_planes(const Planes &p, int r, int N, int T) {
+    for (int i = 0; i < p.n_d; ++i) {
+        const char *h = reinterpret_cast<const char *>(p.H + ((size_t)i * p.n_rng + r) * N);
+        for (int b = 128 * threadIdx.x; b < 8 * N; b += 128 * T) asm volatile("prefetch.global.L2 [%0];" ::"l"(h + b));
+    }
+}
+
+__device__ __forceinline__ void sum_planes(const Planes &p, int r, int N, int T, int pad_shift, float2 *x) {
+    constexpr int E = 8;
+    const int i_lo = max(0, -(r + p.d_lo)), i_hi = min(p.n_d, p.n_bins - r - p.d_lo);
+    for (int n0 = threadIdx.x; n0 < N; n0 += E * T) {
+        float2 acc[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[e] = make_float2(0.f, 0.f);
+        for (int i = i_lo; i < i_hi; ++i) {
+            const float2 *Xr = p.X + (size_t)(r + p.d_lo + i) * N, *Hr = p.H + ((size_t)i * p.n_rng + r) * N;
+            float2 h[E], v[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int n = n0 + e * T;
+                h[e] = n < N ? __ldg(Hr + n) : make_float2(0.f, 0.f);
+                v[e] = n < N ? __ldcg(Xr + n) : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int e = 0; e < E; ++e) acc[e] = i == i_lo ? cmul(h[e], v[e]) : cadd(acc[e], cmul(h[e], v[e]));
         }
-        x[rpad(n, pad_shift)] = make_float2(acc.x, -acc.y);
-    }
-    __syncthreads();
-    inv(x, tc, tf);                                  // ends with a barrier
-    const size_t row = (size_t)r * N;
-    for (int n = threadIdx.x; n < N; n += blockDim.x) {
-        const float2 y = x[rpad(n, pad_shift)];
-        out[row + n] = make_float2(y.x, -y.y);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (n0 + e * T < N) x[rpad(n0 + e * T, pad_shift)] = make_float2(acc[e].x, -acc[e].y);
     }
 }
 
-template <int MAXT>
-__global__ void __launch_bounds__(MAXT, 1)
-azimuth_spectrum_kernel(const float2 *__restrict__ S, int N, RowPlan pl, float2 *__restrict__ X) {
-    spectrum_row(S, X, N, pl.pad_shift, [&](float2 *x, const float2 *tc, const float2 *tf) { row_dif(x, N, pl, tc, tf); });
-}
+// ---- compile-time plans
 
-template <int MAXT>
-__global__ void __launch_bounds__(MAXT, 1)
-azimuth_mig_combine_kernel(const float2 *__restrict__ X, const float2 *__restrict__ H, int n_bins, int n_rng, int d_lo,
-                           int n_d, int N, RowPlan pl, float2 *__restrict__ out) {
-    combine_row(X, H, n_bins, n_rng, d_lo, n_d, N, pl.pad_shift, out,
-                [&](float2 *x, const float2 *tc, const float2 *tf) { row_dit(x, N, pl, tc, tf); });
-}
-
-// Compile-time plans (radices R1 .. Rk, no padding).  The forward transform reads S straight into the first DIF
-// pass (dif_first_global) and writes its last pass (blocks of Rk, twiddles 1) straight to X; the inverse reads
-// the planes' products straight into its first DIT pass (blocks of Rk, twiddles 1) and writes its last pass to
-// out (dit_last_global): two shared-memory round trips per transform fewer than staging the rows.
-
-template <int T, int N, int R1, int... Rs>
-__global__ void __launch_bounds__(T, 2)
-azimuth_spectrum_fixed_kernel(const float2 *__restrict__ S, float2 *__restrict__ X) {
-    extern __shared__ float2 sm[];
-    constexpr int RK = last_radix<R1, Rs...>();
-    float2 *x = sm;
-    float2 *tw = x + padded_len(N);
-    const size_t row = (size_t)blockIdx.x * N;
-    const float2 *tc, *tf;
-    build_twiddles(N, false, tw, &tc, &tf);
-    __syncthreads();
-    griddep_launch_dependents();
-    griddep_wait();                                  // S is complete (no-op without a programmatic predecessor)
-    dif_first_global<N, R1, T, false>(S + row, x, tc, tf);
-    dif_middle<N, N / R1, T, WholeCta, Rs...>(x, tc, tf);
+// The pass on blocks of RK (twiddles 1) in place.
+template <int N, int RK, int T>
+__device__ __forceinline__ void inner_pass(float2 *x) {
 #pragma unroll 1
-    for (int b = threadIdx.x; b < N / RK; b += T) {   // last DIF pass: blocks of RK, twiddles 1, to X
+    for (int b = threadIdx.x; b < N / RK; b += T) {
         float2 v[RK];
 #pragma unroll
         for (int q = 0; q < RK; ++q) v[q] = x[b * RK + q];
         small_dft<RK>(v);
 #pragma unroll
-        for (int q = 0; q < RK; ++q) X[row + b * RK + q] = v[q];
-    }
-}
-
-template <int T, int N, int R1, int... Rs>
-__global__ void __launch_bounds__(T, 2)
-azimuth_mig_combine_fixed_kernel(const float2 *__restrict__ X, const float2 *__restrict__ H, int n_bins, int n_rng,
-                                 int d_lo, int n_d, float2 *__restrict__ out) {
-    extern __shared__ float2 sm[];
-    constexpr int RK = last_radix<R1, Rs...>();
-    float2 *x = sm;
-    float2 *tw = x + padded_len(N);
-    const int r = blockIdx.x;
-    const float2 *tc, *tf;
-    build_twiddles(N, false, tw, &tc, &tf);
-    griddep_wait();                                  // X is complete
-#pragma unroll 1
-    for (int b = threadIdx.x; b < N / RK; b += T) {   // first DIT pass on the planes' products: blocks of RK
-        float2 v[RK];
-#pragma unroll
-        for (int q = 0; q < RK; ++q) v[q] = make_float2(0.f, 0.f);
-        bool any = false;
-        for (int i = 0; i < n_d; ++i) {
-            const int bin = r + d_lo + i;
-            if (bin < 0 || bin >= n_bins) continue;
-            const float2 *Xr = X + (size_t)bin * N + b * RK;
-            const float2 *Hr = H + ((size_t)i * n_rng + r) * N + b * RK;
-#pragma unroll
-            for (int q = 0; q < RK; ++q) {
-                const float2 p = cmul(__ldg(Hr + q), __ldg(Xr + q));
-                v[q] = any ? cadd(v[q], p) : p;
-            }
-            any = true;
-        }
-#pragma unroll
-        for (int q = 0; q < RK; ++q) v[q].y = -v[q].y;
-        small_dft<RK>(v);
-#pragma unroll
         for (int q = 0; q < RK; ++q) x[b * RK + q] = v[q];
     }
     __syncthreads();
-    dit_middle<N, N / R1, T, WholeCta, Rs...>(x, tc, tf);
-    dit_last_global<N, R1, T>(x, out + (size_t)r * N, tc, tf);
 }
+
+template <int T, int MINB, int N, int R1, int... Rs>
+__global__ void __launch_bounds__(T, MINB)
+azimuth_spectrum_fixed_kernel(const float2 *__restrict__ S, float2 *__restrict__ X) {
+    extern __shared__ float2 sm[];
+    griddep_launch_dependents();
+    const size_t row = (size_t)blockIdx.x * N;
+    const float2 *tc, *tf;
+    build_twiddles(N, false, sm + N, &tc, &tf);
+    __syncthreads();
+    griddep_wait();                                  // S is complete, X no longer read
+    dif_first_global<N, R1, T, false>(S + row, sm, tc, tf);
+    dif_middle<N, N / R1, T, WholeCta, Rs...>(sm, tc, tf);
+    inner_pass<N, last_radix<R1, Rs...>(), T>(sm);
+    store_row<T>(sm, X + row, N, 31);
+}
+
+template <int T, int MINB, int N, int R1, int... Rs>
+__global__ void __launch_bounds__(T, MINB)
+azimuth_mig_combine_fixed_kernel(Planes p, float2 *__restrict__ out) {
+    extern __shared__ float2 sm[];
+    const int r = blockIdx.x;
+    prefetch_planes(p, r, N, T);
+    const float2 *tc, *tf;
+    build_twiddles(N, false, sm + N, &tc, &tf);
+    griddep_wait();                                  // X is complete
+    sum_planes(p, r, N, T, 31, sm);
+    __syncthreads();
+    inner_pass<N, last_radix<R1, Rs...>(), T>(sm);
+    dit_middle<N, N / R1, T, WholeCta, Rs...>(sm, tc, tf);
+    dit_last_global<N, R1, T>(sm, out + (size_t)r * N, tc, tf);
+}
+
+// ---- run-time plans (blockDim.x threads); a plan of one pass (n_az <= 16) has no outer pass to keep on global memory
+
+template <bool PAD>
+__device__ __forceinline__ void runtime_spectrum(const float2 *src, float2 *x, int N, const RowPlan &pl,
+                                                 const float2 *tc, const float2 *tf) {
+    int M = N;
+    if (pl.npass > 1) {
+#define ROSAR_FIRST(R) rt_first<R, PAD>(src, x, N, tc, tf, nullptr)
+        ROSAR_FOR_RADIX(pl.rad[0], ROSAR_FIRST)
+#undef ROSAR_FIRST
+        M /= pl.rad[0];
+    } else {
+        for (int n = threadIdx.x; n < N; n += blockDim.x) x[cpad<PAD>(n)] = __ldcg(src + n);
+    }
+    __syncthreads();
+    for (int p = pl.npass > 1; p < pl.npass; ++p) {
+        stage<true, PAD>(pl.rad[p], x, N, M, tc, tf);
+        M /= pl.rad[p];
+    }
+}
+
+template <bool PAD>
+__device__ __forceinline__ void runtime_inverse(float2 *x, float2 *dst, int N, const RowPlan &pl, const float2 *tc,
+                                                const float2 *tf) {
+    int M = 1;
+    for (int p = pl.npass - 1; p >= (pl.npass > 1); --p) {
+        M *= pl.rad[p];
+        stage<false, PAD>(pl.rad[p], x, N, M, tc, tf);
+    }
+    if (pl.npass > 1) {
+#define ROSAR_LAST(R) rt_last<R, PAD>(x, dst, N, tc, tf)
+        ROSAR_FOR_RADIX(pl.rad[0], ROSAR_LAST)
+#undef ROSAR_LAST
+    } else {
+        for (int n = threadIdx.x; n < N; n += blockDim.x) {
+            const float2 y = x[cpad<PAD>(n)];
+            dst[n] = make_float2(y.x, -y.y);
+        }
+    }
+}
+
+template <int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB)
+azimuth_spectrum_kernel(const float2 *__restrict__ S, int N, RowPlan pl, float2 *__restrict__ X) {
+    extern __shared__ float2 sm[];
+    griddep_launch_dependents();
+    const size_t row = (size_t)blockIdx.x * N;
+    const float2 *tc, *tf;
+    build_twiddles(N, false, sm + padded_len(N), &tc, &tf);
+    __syncthreads();
+    griddep_wait();
+    if (pl.pad_shift == 4) runtime_spectrum<true>(S + row, sm, N, pl, tc, tf);
+    else runtime_spectrum<false>(S + row, sm, N, pl, tc, tf);      // both end with a barrier
+    for (int n = threadIdx.x; n < N; n += blockDim.x) X[row + n] = sm[rpad(n, pl.pad_shift)];
+}
+
+template <int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB)
+azimuth_mig_combine_kernel(Planes p, int N, RowPlan pl, float2 *__restrict__ out) {
+    extern __shared__ float2 sm[];
+    const int r = blockIdx.x;
+    prefetch_planes(p, r, N, blockDim.x);
+    const float2 *tc, *tf;
+    build_twiddles(N, false, sm + padded_len(N), &tc, &tf);
+    griddep_wait();
+    sum_planes(p, r, N, blockDim.x, pl.pad_shift, sm);
+    __syncthreads();
+    if (pl.pad_shift == 4) runtime_inverse<true>(sm, out + (size_t)r * N, N, pl, tc, tf);
+    else runtime_inverse<false>(sm, out + (size_t)r * N, N, pl, tc, tf);
+}
+
+// ---- launches
 
 size_t row_smem(int N) { return sizeof(float2) * (size_t)(padded_len(N) + 64 + coarse_len(N)); }
 
-// Both kernels with the compile-time plan when the run-time planner picks exactly these radices for n_az (so the
-// spectra and the plans share one order); false to fall back to the run-time plan.
-template <int T, int N, int... R>
-bool try_fixed_mig(int n_az, const RowPlan &pl, const float2 *S, int n_bins, const float2 *H, int d_lo, int n_d,
-                   int n_rng, float2 *X, float2 *out, cudaStream_t s, rosar_status *st) {
-    constexpr int rad[] = {R...};
-    if (n_az != N || threads_for(N) != T || pl.pad_shift != 31 || pad_shift_for(N) != 31 || pl.npass != (int)sizeof...(R))
-        return false;
-    for (int i = 0; i < pl.npass; ++i)
-        if (pl.rad[i] != rad[i]) return false;
-    static int done_a[kMaxDevices] = {}, done_b[kMaxDevices] = {};
-    const size_t sm = row_smem(N);
-    *st = ensure_smem((const void *)azimuth_spectrum_fixed_kernel<T, N, R...>, sm, done_a, "sparse_azimuth_migrating_fft");
-    if (*st == ROSAR_OK)
-        *st = ensure_smem((const void *)azimuth_mig_combine_fixed_kernel<T, N, R...>, sm, done_b,
-                          "sparse_azimuth_migrating_fft");
-    if (*st != ROSAR_OK) return true;
-    azimuth_spectrum_fixed_kernel<T, N, R...><<<n_bins, T, sm, s>>>(S, X);
-    // the combine kernel's twiddle table overlaps the spectrum kernel's tail (programmatic dependent launch)
+struct MigCall {
+    const float2 *S;
+    Planes p;
+    float2 *X, *out;
+    int N;
+    cudaStream_t s;
+};
+
+template <typename KA, typename KB, typename... A>
+rosar_status launch_pair(const MigCall &c, KA spectrum, KB combine, int T, int (*done)[kMaxDevices], A... plan) {
+    const char *what = "sparse_azimuth_migrating_fft";
+    const size_t sm = row_smem(c.N);
+    rosar_status st = ensure_smem((const void *)spectrum, sm, done[0], what);
+    if (st == ROSAR_OK) st = ensure_smem((const void *)combine, sm, done[1], what);
+    if (st != ROSAR_OK) return st;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_rng);
+    cfg.gridDim = dim3(c.p.n_bins);
     cfg.blockDim = dim3(T);
     cfg.dynamicSmemBytes = sm;
-    cfg.stream = s;
+    cfg.stream = c.s;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, azimuth_mig_combine_fixed_kernel<T, N, R...>, (const float2 *)X, H,
-                                             n_bins, n_rng, d_lo, n_d, out);
-    *st = e != cudaSuccess ? set_error(ROSAR_ERR_CUDA, "sparse_azimuth_migrating_fft: launch failed: %s",
-                                       cudaGetErrorString(e))
-                           : check_launch("sparse_azimuth_migrating_fft");
+    cudaError_t e = cudaLaunchKernelEx(&cfg, spectrum, c.S, plan..., c.X);
+    cfg.gridDim = dim3(c.p.n_rng);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, combine, c.p, plan..., c.out);
+    if (e != cudaSuccess) return set_error(ROSAR_ERR_CUDA, "%s: launch failed: %s", what, cudaGetErrorString(e));
+    return check_launch(what);
+}
+
+template <int T, int MINB, int N, int... R>
+rosar_status launch_fixed(const MigCall &c) {
+    static int done[2][kMaxDevices] = {};
+    return launch_pair(c, azimuth_spectrum_fixed_kernel<T, MINB, N, R...>, azimuth_mig_combine_fixed_kernel<T, MINB, N, R...>,
+                       T, done);
+}
+
+template <int MAXT, int MINB>
+rosar_status launch_runtime(const MigCall &c, const RowPlan &pl, int T) {
+    static int done[2][kMaxDevices] = {};
+    return launch_pair(c, azimuth_spectrum_kernel<MAXT, MINB>, azimuth_mig_combine_kernel<MAXT, MINB>, T, done, c.N, pl);
+}
+
+template <int N, int... R>
+bool plan_is(int n_az, const RowPlan &pl) {
+    constexpr int rad[] = {R...};
+    if (n_az != N || pl.pad_shift != 31 || pl.npass != (int)sizeof...(R)) return false;
+    for (int i = 0; i < pl.npass; ++i)
+        if (pl.rad[i] != rad[i]) return false;
     return true;
 }
+
+constexpr int kFewRows = 304;      // as the row filter: up to two rows an SM a row's own latency counts
 
 }  // namespace
 
@@ -212,32 +266,17 @@ rosar_status launch_sparse_azimuth_migrating_fft(const float2 *S, int n_bins, co
     if (!make_plan(n_az, &pl))
         return set_error(ROSAR_ERR_UNSUPPORTED, "sparse_azimuth_migrating_fft: n_az=%d is not 2^a 3^b 5^c in [2, %d]",
                          n_az, AF_MAX_N);
-    {
-        rosar_status st = ROSAR_OK;
-        if (try_fixed_mig<256, 3600, 16, 15, 15>(n_az, pl, S, n_bins, H, d_lo, n_d, n_rng, X, out, s, &st) ||
-            try_fixed_mig<256, 1800, 8, 15, 15>(n_az, pl, S, n_bins, H, d_lo, n_d, n_rng, X, out, s, &st) ||
-            try_fixed_mig<512, 7200, 8, 4, 15, 15>(n_az, pl, S, n_bins, H, d_lo, n_d, n_rng, X, out, s, &st) ||
-            try_fixed_mig<256, 360, 8, 3, 15>(n_az, pl, S, n_bins, H, d_lo, n_d, n_rng, X, out, s, &st))
-            return st;
-    }
-    const size_t sm = row_smem(n_az);
-    if (sm > 200 * 1024)
-        return set_error(ROSAR_ERR_UNSUPPORTED, "sparse_azimuth_migrating_fft: n_az=%d needs %zu bytes of shared memory",
-                         n_az, sm);
-    const int T = threads_for(n_az);
-    static int done[8][kMaxDevices] = {};
-    auto go = [&](auto ka, auto kb, int v) -> rosar_status {
-        rosar_status st = ensure_smem((const void *)ka, sm, done[2 * v], "sparse_azimuth_migrating_fft");
-        if (st == ROSAR_OK) st = ensure_smem((const void *)kb, sm, done[2 * v + 1], "sparse_azimuth_migrating_fft");
-        if (st != ROSAR_OK) return st;
-        ka<<<n_bins, T, sm, s>>>(S, n_az, pl, X);
-        kb<<<n_rng, T, sm, s>>>(X, H, n_bins, n_rng, d_lo, n_d, n_az, pl, out);
-        return check_launch("sparse_azimuth_migrating_fft");
-    };
-    if (T <= 256) return go(azimuth_spectrum_kernel<256>, azimuth_mig_combine_kernel<256>, 0);
-    if (T <= 384) return go(azimuth_spectrum_kernel<384>, azimuth_mig_combine_kernel<384>, 1);
-    if (T <= 512) return go(azimuth_spectrum_kernel<512>, azimuth_mig_combine_kernel<512>, 2);
-    return go(azimuth_spectrum_kernel<1024>, azimuth_mig_combine_kernel<1024>, 3);
+    const MigCall c{S, Planes{X, H, n_bins, n_rng, d_lo, n_d}, X, out, n_az, s};
+    const bool few = n_rng <= kFewRows;
+    if (plan_is<3600, 16, 15, 15>(n_az, pl)) return launch_fixed<256, 4, 3600, 16, 15, 15>(c);
+    if (plan_is<1800, 8, 15, 15>(n_az, pl))
+        return few ? launch_fixed<256, 4, 1800, 8, 15, 15>(c) : launch_fixed<128, 8, 1800, 8, 15, 15>(c);
+    if (plan_is<7200, 8, 4, 15, 15>(n_az, pl)) return launch_fixed<256, 3, 7200, 8, 4, 15, 15>(c);
+    if (plan_is<360, 8, 3, 15>(n_az, pl)) return launch_fixed<128, 8, 360, 8, 3, 15>(c);
+    // 128 threads up to 2048: 480 x 256 9.7 us against 12.2 on 256, 1024 x 256 10.1 against 12.3, 1125 x 512 17.0 each.
+    if (n_az <= 4096) return launch_runtime<256, 3>(c, pl, n_az <= 2048 ? 128 : 256);
+    if (n_az <= 8192 && !few) return launch_runtime<256, 3>(c, pl, 256);
+    return launch_runtime<512, 1>(c, pl, 512);
 }
 
 }  // namespace rosar

@@ -93,3 +93,21 @@ def test_batch_by_length_equals_single_scans(rosar, lengths):
         for i, (out, sc) in enumerate(zip(b.outs, scans)):
             assert torch.equal(out, rosar.image_fft(sc["raw"], sc["win"], sc["H"])), i
     b.close()
+
+
+# the migrating filter's plans of one, two and more passes, padded and odd, at the lines between its thread counts and
+# (n_rng 305) between few and many rows; the gather form's bar is 2e-6 and the filter's 5e-6, each against FP64
+@pytest.mark.parametrize("n_az,n_rng", [(2, 7), (16, 305), (30, 7), (81, 305), (360, 9), (675, 5), (1024, 305), (1800, 9),
+                                        (1800, 305), (2048, 5), (2250, 305), (3600, 6), (4096, 3), (4500, 3), (7200, 4),
+                                        (8192, 3), (8640, 305), (14400, 2), (16384, 2)])
+def test_migrating_filter_equals_gather_form(rosar, n_az, n_rng):
+    import torch
+    rng = np.random.default_rng(n_az + n_rng)
+    K = 6
+    S, w = torch.from_numpy(_c(rng, n_rng + 2, n_az)).cuda(), torch.from_numpy(_c(rng, n_rng, K)).cuda()
+    o = torch.from_numpy(rng.integers(-n_az // 2, n_az // 2 + 1, K).astype(np.int32)).cuda()
+    dl = torch.from_numpy(rng.integers(-2, 5, (n_rng, K)).astype(np.int32)).cuda()     # rows on both sides are missing
+    plan = rosar.azimuth_plan_migrating(w, o, dl, n_az)
+    got = rosar.sparse_azimuth_migrating_fft(S, plan)
+    ref = rosar.sparse_azimuth_migrating(S, w, o, dl)
+    assert torch.linalg.norm(got - ref) <= (TOL_FFT_FILTER + 2e-6) * torch.linalg.norm(ref)
