@@ -188,6 +188,24 @@ __device__ __forceinline__ float2 twiddle(int q, const float2 *tc, const float2 
 
 using fft::twiddle_powers;
 
+// Row lengths of which two CTAs (1 KB of shared memory each besides their own) fit the 228 KB of an SM without the
+// twiddle table and not with it: their compile-time plans compute each butterfly's twiddle instead.
+__host__ __device__ constexpr bool direct_twiddles(int n) {
+    return 2 * (8 * n + 1024) <= 228 * 1024 && 2 * (8 * (n + 64 + coarse_len(n)) + 1024) > 228 * 1024;
+}
+
+// exp(-2 pi i q/N) for a compile-time plan.
+template <int N>
+__device__ __forceinline__ float2 twiddle_of(int q, const float2 *tc, const float2 *tf) {
+    if constexpr (direct_twiddles(N)) {
+        float s, c;
+        sincospif((float)q * (2.f / (float)N), &s, &c);
+        return make_float2(c, -s);
+    } else {
+        return twiddle(q, tc, tf);
+    }
+}
+
 // One in-place decimation-in-frequency stage: radix R on blocks of length M (stride s = M/R):
 // v = DFT_R(x[base + r*s]); x[base + q*s] = v[q] * W_M^(j*q).
 template <int R, bool PAD>
@@ -310,7 +328,7 @@ __device__ __forceinline__ void dif_pass_c(float2 *x, const float2 *tc, const fl
         small_dft<R>(v);
         x[cpad<PAD>(base)] = v[0];
         float2 wq[R];
-        twiddle_powers<R>(twiddle(j * tstep, tc, tf), wq);
+        twiddle_powers<R>(twiddle_of<N>(j * tstep, tc, tf), wq);
 #pragma unroll
         for (int q = 1; q < R; ++q) x[cpad<PAD>(base + q * s)] = cmul(v[q], wq[q]);
     }
@@ -327,7 +345,7 @@ __device__ __forceinline__ void dit_pass_c(float2 *x, const float2 *tc, const fl
         const int base = blk * M + j;
         float2 v[R];
         float2 wq[R];
-        twiddle_powers<R>(twiddle(j * tstep, tc, tf), wq);
+        twiddle_powers<R>(twiddle_of<N>(j * tstep, tc, tf), wq);
         v[0] = x[cpad<PAD>(base)];
 #pragma unroll
         for (int q = 1; q < R; ++q) v[q] = cmul(x[cpad<PAD>(base + q * s)], wq[q]);
@@ -405,7 +423,7 @@ __device__ __forceinline__ void dif_first_global(const float2 *__restrict__ src,
         small_dft<R>(v);
         x[j] = v[0];
         float2 wq[R];
-        twiddle_powers<R>(twiddle(j, tc, tf), wq);
+        twiddle_powers<R>(twiddle_of<N>(j, tc, tf), wq);
 #pragma unroll
         for (int q = 1; q < R; ++q) x[j + q * s] = cmul(v[q], wq[q]);
     }
@@ -418,6 +436,10 @@ __device__ __forceinline__ void dif_first_global(const float2 *__restrict__ src,
             asm volatile("discard.global.L2 [%0], 128;" ::"l"(l) : "memory");
     }
 }
+
+// Where the product with H reads it: the fused step from global memory, the fused step from shared memory, or a step
+// of its own from global memory.
+enum HSource { kFused = 0, kStaged = 1, kStreamed = 2 };
 
 // Last forward pass (blocks of R, stride 1), y = conj(H . X) (conj(H) . X conjugated when hs = -1), and the
 // first pass of the inverse on the same block.  H is in the forward transform's digit-reversed order; h is
@@ -453,6 +475,48 @@ __device__ __forceinline__ void fused_mid(float2 *x, const float2 *h, float hs, 
     __syncthreads();
 }
 
+// The same with the product over consecutive elements between the two passes (kStreamed): a shared-memory round trip
+// more, and H read once in full lines, where the fused step's reads of R elements a thread outgrow the L1 that the
+// rows leave (two rows of 14400: 26 KB left, 61 KB of lines a row).
+template <int N, int R, int T>
+__device__ __forceinline__ void streamed_mid(float2 *x, const float2 *__restrict__ h, float hs,
+                                             float2 *__restrict__ spec) {
+    constexpr int nb = N / R, E = 8;
+#pragma unroll 1
+    for (int inverse = 0; inverse < 2; ++inverse) {
+#pragma unroll 1
+        for (int b = threadIdx.x; b < nb; b += T) {
+            const int base = b * R;
+            float2 v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = x[base + r];
+            small_dft<R>(v);
+            if (spec && !inverse) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) spec[r * nb + b] = v[r];
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) x[base + r] = v[r];
+        }
+        __syncthreads();
+        if (inverse) break;
+#pragma unroll 1
+        for (int n0 = threadIdx.x; n0 < N; n0 += E * T) {
+            float2 hv[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) hv[e] = n0 + e * T < N ? __ldg(h + n0 + e * T) : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (n0 + e * T < N) {
+                    hv[e].y *= hs;
+                    const float2 y = cmul(hv[e], x[n0 + e * T]);
+                    x[n0 + e * T] = make_float2(y.x, -y.y);
+                }
+        }
+        __syncthreads();
+    }
+}
+
 // Last DIT pass (M = N) written to global memory with the final conjugation of the inverse.
 template <int N, int R, int T>
 __device__ __forceinline__ void dit_last_global(const float2 *x, float2 *__restrict__ dst, const float2 *tc,
@@ -461,7 +525,7 @@ __device__ __forceinline__ void dit_last_global(const float2 *x, float2 *__restr
 #pragma unroll 1
     for (int j = threadIdx.x; j < s; j += T) {
         float2 v[R], wq[R];
-        twiddle_powers<R>(twiddle(j, tc, tf), wq);
+        twiddle_powers<R>(twiddle_of<N>(j, tc, tf), wq);
         v[0] = x[j];
 #pragma unroll
         for (int q = 1; q < R; ++q) v[q] = cmul(x[j + q * s], wq[q]);
@@ -471,32 +535,33 @@ __device__ __forceinline__ void dit_last_global(const float2 *x, float2 *__restr
     }
 }
 
-template <int N, int M, int T, bool H_SMEM, int R, int... Rest>
+template <int N, int M, int T, int H_FROM, int R, int... Rest>
 __device__ __forceinline__ void filter_middle(float2 *x, const float2 *h, float hs, const float2 *tc, const float2 *tf,
                                               float2 *__restrict__ spec = nullptr) {
     if constexpr (sizeof...(Rest) == 0) {
         static_assert(M == R, "the last radix spans the last block");
-        fused_mid<N, R, T, H_SMEM>(x, h, hs, spec);
+        if constexpr (H_FROM == kStreamed) streamed_mid<N, R, T>(x, h, hs, spec);
+        else fused_mid<N, R, T, H_FROM == kStaged>(x, h, hs, spec);
     } else {
         dif_pass_c<N, M, R, false, T>(x, tc, tf);
-        filter_middle<N, M / R, T, H_SMEM, Rest...>(x, h, hs, tc, tf, spec);
+        filter_middle<N, M / R, T, H_FROM, Rest...>(x, h, hs, tc, tf, spec);
         dit_pass_c<N, M, R, false, T>(x, tc, tf);
     }
 }
 
 // src, dst: the row in global memory (natural order), which may be the same row (every element is read before the
 // first barrier, written after the last); x: N elements of shared memory (no padding); the
-// caller has built the twiddle table and synchronised.  With H_SMEM, h may still be arriving by cp.async
+// caller has built the twiddle table and synchronised.  With kStaged, h may still be arriving by cp.async
 // when this starts (waited for at the end of the first pass).  No barrier at the end.  discard: src is
 // scratch, dropped from L2 once read (dif_first_global).
-template <int N, int T, bool H_SMEM, int R1, int... Rs>
+template <int N, int T, int H_FROM, int R1, int... Rs>
 __device__ __forceinline__ void row_filter_fused(const float2 *src, const float2 *h, float hs, float2 *x,
                                                  float2 *dst, const float2 *tc, const float2 *tf,
                                                  bool discard = false, const float2 *__restrict__ phase = nullptr,
                                                  float2 *__restrict__ spec = nullptr) {
     static_assert(sizeof...(Rs) >= 1, "at least two passes");
-    dif_first_global<N, R1, T, H_SMEM>(src, x, tc, tf, discard, phase);
-    filter_middle<N, N / R1, T, H_SMEM, Rs...>(x, h, hs, tc, tf, spec);
+    dif_first_global<N, R1, T, H_FROM == kStaged>(src, x, tc, tf, discard, phase);
+    filter_middle<N, N / R1, T, H_FROM, Rs...>(x, h, hs, tc, tf, spec);
     dit_last_global<N, R1, T>(x, dst, tc, tf);
 }
 
@@ -660,33 +725,36 @@ __device__ __forceinline__ void build_twiddles(int N, bool full, float2 *tw, con
 
 
 // One row of the azimuth filter on one CTA of T threads with a compile-time plan (N with an odd factor):
-// stage the H row (cp.async; H_SMEM) and the twiddle table, wait for the predecessor grid (S is complete), run
-// row_filter_fused.  sm: (H_SMEM ? 2 : 1) (N + 1) + 64 + coarse_len(N) float2 of shared memory
-// (filter_row_smem); without H_SMEM the fused middle step reads H from global memory (rows too long to
-// stage two of them).
-template <int N, bool H_SMEM = true>
+// stage the H row (cp.async; kStaged) and the twiddle table, wait for the predecessor grid (S is complete), run
+// row_filter_fused.  sm: (H_FROM == kStaged ? 2 : 1) (N + 1) + 64 + coarse_len(N) float2 of shared memory, N with direct_twiddles
+// (filter_row_smem); otherwise H is read from global memory.
+template <int N, int H_FROM = kStaged>
 constexpr size_t filter_row_smem() {
-    return sizeof(float2) * (size_t)((H_SMEM ? 2 : 1) * padded_len(N) + 64 + coarse_len(N));
+    if (direct_twiddles(N)) return sizeof(float2) * (size_t)((H_FROM == kStaged ? 2 : 1) * N);
+    return sizeof(float2) * (size_t)((H_FROM == kStaged ? 2 : 1) * padded_len(N) + 64 + coarse_len(N));
 }
 
-template <int T, int N, bool H_SMEM, int... R>
+template <int T, int N, int H_FROM, int... R>
 __device__ __forceinline__ void filter_row_cta(const float2 *S_row, const float2 *__restrict__ H_row,
                                                bool conj_h, float2 *out_row, float2 *sm,
                                                const float2 *__restrict__ phase = nullptr,
                                                float2 *__restrict__ spec = nullptr) {
     static_assert(pad_shift_for(N) == 31, "compile-time filter plans are for rows with an odd factor");
+    constexpr int row = direct_twiddles(N) ? N : padded_len(N);
     float2 *x = sm;
-    float2 *hb = x + padded_len(N);
-    float2 *tw = H_SMEM ? hb + padded_len(N) : hb;
-    if (H_SMEM) {
+    float2 *hb = x + row;
+    float2 *tw = H_FROM == kStaged ? hb + row : hb;
+    if (H_FROM == kStaged) {
         for (int n = threadIdx.x; n < N; n += T) cp_async8(hb + n, H_row + n);   // waited for after the first pass
         cp_async_commit();
     }
-    const float2 *tc, *tf;
-    build_twiddles(N, false, tw, &tc, &tf);
-    __syncthreads();
+    const float2 *tc = nullptr, *tf = nullptr;
+    if constexpr (!direct_twiddles(N)) {
+        build_twiddles(N, false, tw, &tc, &tf);
+        __syncthreads();
+    }
     griddep_wait();                          // S is complete (no-op unless launched to overlap its producer)
-    row_filter_fused<N, T, H_SMEM, R...>(S_row, H_SMEM ? hb : H_row, conj_h ? -1.f : 1.f, x, out_row, tc, tf, false,
+    row_filter_fused<N, T, H_FROM, R...>(S_row, H_FROM == kStaged ? hb : H_row, conj_h ? -1.f : 1.f, x, out_row, tc, tf, false,
                                          phase, spec);
 }
 
