@@ -1,4 +1,4 @@
-// Shared memory of the run-time-plan row kernels (azimuth_rows.cu, azimuth_fft.cu).
+// Shared memory of the run-time-plan row kernels (azimuth_rows.cu, azimuth_mig_fft.cu).
 #pragma once
 
 #include "row_fft.cuh"

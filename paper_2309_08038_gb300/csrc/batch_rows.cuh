@@ -1,5 +1,5 @@
 // Scans of a batch as the kernels read them, and groups of scans that one launch covers: the range compression of all
-// scans of one length L, the azimuth rows of all scans of one n_az (batch.cu, range_compress.cu, azimuth_fft.cu).
+// scans of one length L, the azimuth rows of all scans of one n_az (batch.cu, range_compress.cu, azimuth_rows.cu).
 #pragma once
 
 #include "rosar_internal.cuh"

@@ -263,50 +263,105 @@ __device__ __forceinline__ void range_tile(const float2 *__restrict__ raw, const
 // Adjoint of range_tile for pulses n0 .. n0+P-1 (Eq. (38) transposed, conjugate-Wirtinger convention):
 //   grad_raw[n][m] = win[m] * sum_l conj(c_l) * exp(+j*2*pi*l*m/L) * g[l][n]
 //                  = win[m] * conj( DFT_l{ c_l * conj(g[l][n]) }[m] ).
-// Reads the range-major gradient g [L][n_az] with loads coalesced along azimuth, runs the same
-// Stockham passes with every result kept in the per-pulse buffer (natural order), and writes
-// grad_raw [n_az][L] pulse-major.  blockDim.x == T*P; `smem` holds Tile<L, P>::SMEM_ELEMS elements.
+// The lanes of a warp run over the tile's pulses first: a thread's 16 bins of the range-major gradient g [L][n_az]
+// come straight into registers (P pulses of a bin are one segment), the passes exchange through a buffer [bin][pulse]
+// (one bin of padding in 16: neighbouring threads of a pulse fall on the other half of the banks), and the last pass
+// stores grad_raw [n_az][L] from registers, 32 / P consecutive samples a pulse (L of 16 and 32: through the buffer).
+
+// One pass of radix R (sub-transform size NS before it).  FIRST: v holds the bins t + r*T.  LAST: v is left with sample
+// b*T + t + r*NS of the transform at v[b*R + brev(r)].
+template <int L, int P, int R, int NS, bool FIRST, bool LAST>
+__device__ __forceinline__ void column_pass(float2 (&v)[Tile<L, P>::RM], int t, int p, float2 *buf, const float2 *tab) {
+    constexpr int RM = Tile<L, P>::RM, T = Tile<L, P>::T, NB = RM / R;
+    if (!FIRST) {
+        __syncthreads();
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[b * R + r] = buf[pad16(t + b * T + r * (L / R)) * P + p];
+        if (!LAST) __syncthreads();          // read before the next exchange overwrites it
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        const int j = t + b * T, k = j & (NS - 1);
+        if (NS > 1) {
+            float2 wq[R];
+            twiddle_powers<R>(half_twiddle(tab, 2 * k * (L / (NS * R))), wq);
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[b * R + r] = cmul(v[b * R + r], wq[r]);
+        }
+        dft_dif<R>(v + b * R);
+        if (!LAST) {
+            const int base = (j - k) * R + k;
+#pragma unroll
+            for (int r = 0; r < R; ++r) buf[pad16(base + r * NS) * P + p] = v[b * R + brev(r, ilog2(R))];
+        }
+    }
+}
+
+// blockDim.x == T*P; `smem` holds Tile<L, P>::TAB + P*LP elements.
 template <int L, int P>
 __device__ __forceinline__ void range_adjoint_tile(const float2 *__restrict__ g, const float *__restrict__ win,
                                                    int n_az, bool centred, float2 *__restrict__ grad_raw, int n0,
                                                    float2 *smem) {
     using PL = Tile<L, P>;
-    constexpr int RM = PL::RM, T = PL::T;
+    constexpr int RM = PL::RM, T = PL::T, NF = PL::NF, RR = PL::RR;
     float2 *tab = smem;
     float2 *buf = smem + PL::TAB;
-    const int t = threadIdx.x % T;
-    const int p = threadIdx.x / T;
-    const int np = min(P, n_az - n0);
+    const int p = threadIdx.x % P, t = threadIdx.x / P;
+    const int n = n0 + p;
+    const bool live = n < n_az;
+    float2 v[RM];
+#pragma unroll
+    for (int r = 0; r < RM; ++r) v[r] = live ? ld_stream(g + (size_t)(t + r * T) * n_az + n) : make_float2(0.f, 0.f);
     build_half_twiddles<L>(tab, PL::THREADS);
     __syncthreads();
-    for (int idx = threadIdx.x; idx < L * P; idx += PL::THREADS) {
-        const int l = idx / P, q = idx % P;
-        float2 x = q < np ? cconj(__ldg(g + (size_t)l * n_az + n0 + q)) : make_float2(0.f, 0.f);
-        if (centred) {
-            const float2 c = half_twiddle(tab, l);
-            x = cmul(x, (l & 1) ? make_float2(-c.x, -c.y) : c);
+#pragma unroll
+    for (int r = 0; r < RM; ++r) v[r].y = -v[r].y;
+    if (centred) {
+        // c_l = (-1)^l exp(-j*pi*l/L), l = t + r*T (T even: one sign a thread; T = 1: r's)
+        float2 sp[RM];
+        twiddle_powers<RM>(half_twiddle(tab, T), sp);
+        const float2 ct = half_twiddle(tab, t);
+#pragma unroll
+        for (int r = 0; r < RM; ++r) {
+            const float2 c = r == 0 ? ct : cmul(ct, sp[r]);
+            v[r] = cmul(v[r], ((t + r * T) & 1) ? make_float2(-c.x, -c.y) : c);
         }
-        buf[q * PL::LP + pad16(l)] = x;
     }
-    __syncthreads();
-    float2 v[RM];
-    float2 *pb = buf + p * PL::LP;
-    constexpr int NF = PL::NF, RR = PL::RR;
+    constexpr int RL = L < 16 ? L : RR > 1 ? RR : 16;        // the last pass's radix
     if constexpr (L < 16) {
-        stockham_pass<L, P, L, 1, false, false>(v, t, p, pb, buf, tab, false);
+        column_pass<L, P, L, 1, true, true>(v, t, p, buf, tab);
     } else {
-        stockham_pass<L, P, 16, 1, false, false>(v, t, p, pb, buf, tab, false);
-        if constexpr (NF >= 2) stockham_pass<L, P, 16, 16, false, false>(v, t, p, pb, buf, tab, false);
-        if constexpr (NF >= 3) stockham_pass<L, P, 16, 256, false, false>(v, t, p, pb, buf, tab, false);
-        if constexpr (RR > 1) stockham_pass<L, P, RR, (L / RR), false, false>(v, t, p, pb, buf, tab, false);
+        column_pass<L, P, 16, 1, true, (NF == 1 && RR == 1)>(v, t, p, buf, tab);
+        if constexpr (NF >= 2) column_pass<L, P, 16, 16, false, (NF == 2 && RR == 1)>(v, t, p, buf, tab);
+        if constexpr (NF >= 3) column_pass<L, P, 16, 256, false, (NF == 3 && RR == 1)>(v, t, p, buf, tab);
+        if constexpr (RR > 1) column_pass<L, P, RR, (L / RR), false, true>(v, t, p, buf, tab);
     }
-    for (int idx = threadIdx.x; idx < P * L; idx += PL::THREADS) {
-        const int q = idx / L, m = idx % L;
-        if (q < np) {
-            const float wm = win ? __ldg(win + m) : 1.f;
-            grad_raw[(size_t)(n0 + q) * L + m] = cscale(cconj(buf[q * PL::LP + pad16(m)]), wm);
+    if constexpr (L >= 16 && T < 4) {
+        // fewer than 4 samples of a pulse side by side: through the buffer, [pulse][sample] with an odd stride
+        __syncthreads();
+#pragma unroll
+        for (int b = 0; b < RM / RL; ++b)
+#pragma unroll
+            for (int r = 0; r < RL; ++r) buf[p * (L + 1) + t + b * T + r * (L / RL)] = v[b * RL + brev(r, ilog2(RL))];
+        __syncthreads();
+        const int np = min(P, n_az - n0);
+        for (int idx = threadIdx.x; idx < np * L; idx += PL::THREADS) {
+            const int q = idx / L, m = idx % L;
+            grad_raw[(size_t)n0 * L + idx] = cscale(cconj(buf[q * (L + 1) + m]), win ? __ldg(win + m) : 1.f);
         }
+        return;
     }
+    if (!live) return;
+#pragma unroll
+    for (int b = 0; b < RM / RL; ++b)
+#pragma unroll
+        for (int r = 0; r < RL; ++r) {
+            const int m = t + b * T + r * (L / RL);
+            const float wm = win ? __ldg(win + m) : 1.f;
+            grad_raw[(size_t)n * L + m] = cscale(cconj(v[b * RL + brev(r, ilog2(RL))]), wm);
+        }
 }
 
 }  // namespace fft

@@ -59,20 +59,31 @@ rosar_status launch_group_L(const ScanGroup &g, int total, cudaStream_t s, bool 
     return check_launch("batch range compression");
 }
 
+// Pulses a CTA of the adjoint: 8 are a 64-byte segment of a bin's row, and 4 consecutive samples of a pulse's are a
+// sector.  Bound by memory: 16 scans of 3600 x 256 80 -> 53 us (of 35 at the copy rate), x 128 48 -> 27, 8 scans of
+// x 512 110 -> 65 (75 on two CTAs an SM), 4 of x 1024 103 -> 76 (93 on one), against bins staged pulse by pulse in shared memory
+// before the first pass and after the last.
 template <int L>
-__global__ void __launch_bounds__(Plan<L>::THREADS)
+struct AdjointPlan : fft::Tile<L, (L <= 16 ? 32 : L <= 32 ? 16 : L <= 1024 ? 8 : L == 2048 ? 4 : 2)> {
+    using Base = fft::Tile<L, (L <= 16 ? 32 : L <= 32 ? 16 : L <= 1024 ? 8 : L == 2048 ? 4 : 2)>;
+    static constexpr size_t SMEM = sizeof(float2) * (size_t)(Base::TAB + Base::P * Base::LP);
+};
+
+template <int L>
+__global__ void __launch_bounds__(AdjointPlan<L>::THREADS, L == 1024 ? 2 : L == 512 ? 3 : 1)
 range_adjoint_kernel(const float2 *__restrict__ g, const float *__restrict__ win, int n_az, int centred,
                      float2 *__restrict__ grad_raw) {
     extern __shared__ float2 smem[];
     const size_t scan = (size_t)blockIdx.y * n_az * L;      // grid.y: scans of a stack
-    fft::range_adjoint_tile<L, Plan<L>::P>(g + scan, win, n_az, centred != 0, grad_raw + scan, blockIdx.x * Plan<L>::P,
-                                           smem);
+    constexpr int P = AdjointPlan<L>::P;
+    fft::range_adjoint_tile<L, P>(g + scan, win, n_az, centred != 0, grad_raw + scan, blockIdx.x * P, smem);
 }
 
 template <int L>
 rosar_status launch_adjoint_L(const float2 *g, const float *win, int n_az, int centred, float2 *grad_raw,
                               cudaStream_t s, int n_scans) {
-    using PL = Plan<L>;
+    using PL = AdjointPlan<L>;
+    static_assert(PL::SMEM <= 227 * 1024, "range-adjoint tile exceeds shared memory");
     if (PL::SMEM > 48 * 1024) {
         static int done[kMaxDevices] = {};
         rosar_status st = ensure_smem((const void *)range_adjoint_kernel<L>, PL::SMEM, done, "range_compress_adjoint");

@@ -95,7 +95,7 @@ rosar_status launch_phasors(const float *eps, long long n, float2 *P, cudaStream
 rosar_status launch_range_compress_adjoint(const float2 *g, const float *win, int n_az, int L, int centred,
                                            float2 *grad_raw, cudaStream_t s, int n_scans = 1);
 
-// Azimuth filter in the frequency domain (azimuth_fft.cu).
+// Azimuth filter in the frequency domain (plans: azimuth_fft.cu, rows: azimuth_rows.cu).
 int azimuth_fft_supported(int n_az);
 
 // Image loss of the differentiable form (image_loss.cu): partial sums per call = image_loss_partials().

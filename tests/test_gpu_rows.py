@@ -111,3 +111,20 @@ def test_migrating_filter_equals_gather_form(rosar, n_az, n_rng):
     got = rosar.sparse_azimuth_migrating_fft(S, plan)
     ref = rosar.sparse_azimuth_migrating(S, w, o, dl)
     assert torch.linalg.norm(got - ref) <= (TOL_FFT_FILTER + 2e-6) * torch.linalg.norm(ref)
+
+
+# every length (and so every number and radix of passes), pulse counts around the tiles of 4, 8, 16 and 32 pulses; the
+# bar of the adjoint's parity test
+@pytest.mark.parametrize("L", [8, 16, 32, 64, 128, 256, 512, 1024, 2048, 4096])
+@pytest.mark.parametrize("n_az", [1, 15, 33])
+def test_range_adjoint_tiles_match_oracle(rosar, L, n_az):
+    import torch
+    rng = np.random.default_rng(L + n_az)
+    g = _c(rng, L, n_az)
+    win = synth.hann_window(L)
+    for w in (win, None):
+        for centred in (True, False):
+            got = rosar.range_compress_adjoint(torch.from_numpy(g).cuda(), None if w is None else torch.from_numpy(w).cuda(),
+                                               centred=centred).cpu().numpy()
+            ref = O.range_compress_adjoint(g, np.ones(L, np.float32) if w is None else w, centred)
+            assert np.linalg.norm(got - ref) <= 2e-6 * np.linalg.norm(ref), centred
