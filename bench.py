@@ -3,7 +3,7 @@
 
 Headline workload: the batched form, 256 scans of uneven size (n_az in {1800, 3600, 7200} pulses,
 L in {128, 256, 512, 1024} ADC samples, K in {32, 64, 128} taps of M = n_az/6), 480,844,800 image
-pixels, imaged by ONE persistent kernel launch replayed from a CUDA graph (rosar_batch_launch):
+pixels, imaged by ONE graph launch (rosar_batch_launch):
 range compression of every pulse and the sparse azimuth filter of every row.  One step = the whole
 batch.  Metric: image px/s.
 
@@ -635,11 +635,20 @@ def run_reference(args):
 
 # ------------------------------------------------------------------- ours --
 
-BATCH_SOURCES = ("batch.cu", "fft_tile.cuh", "row_fft.cuh", "azimuth_tile.cuh", "rosar_internal.cuh")
+BATCH_SOURCES = ("batch.cu", "batch_rows.cuh", "azimuth_rows.cu", "range_compress.cu", "fft_tile.cuh", "row_fft.cuh",
+                 "azimuth_tile.cuh", "rosar_internal.cuh")
+
+
+def batch_launches(tuning, cfgs):
+    """Kernels of one rosar_batch_launch of scans that all have a plan H: the default tuning takes one range launch per
+    pulse length and one azimuth launch per row length, any other the one persistent kernel."""
+    if tuning.interleave == 0 and tuning.ctas_per_sm == 0 and tuning.flags == 0:
+        return len({c.L for c in cfgs}) + len({c.n_az for c in cfgs})
+    return 1
 
 
 def headline_batched(torch, rosar, args, device, world, stream, peaks, peak_src, clk_gpu):
-    """The batched workload through one persistent graph launch per step (the timed steps of the headline)."""
+    """The batched workload through one graph launch per step (the timed steps of the headline)."""
     wl = BatchedWorkload(torch, rosar, device, args.batch_scans)
     tuned = rosar.autotune.tune_batch(wl.scans)
     b = rosar.Batch(wl.scans, tuned["tuning"])
@@ -653,8 +662,11 @@ def headline_batched(torch, rosar, args, device, world, stream, peaks, peak_src,
     px = wl.px
     hbm = float(peaks["hbm_gbs"])
     info = b.info()
-    kname = f"batch_kernel<{b.tuning.az_tile // 256}>"
-    traffic = recorded_traffic("batch_kernel", f"batched{len(wl.cfgs)}", source_hash(*BATCH_SOURCES))
+    launches = batch_launches(b.tuning, wl.cfgs)
+    kname = (f"batch_kernel<{b.tuning.az_tile // 256}>" if launches == 1 else
+             f"range_group_kernel<L> and azimuth_fft_fixed_kernel<BatchRows, ...>, {launches} launches")
+    traffic = recorded_traffic("batch_kernel" if launches == 1 else "batch_by_length", f"batched{len(wl.cfgs)}",
+                               source_hash(*BATCH_SOURCES))
     roofline = {"kernel": kname, "bound": "hbm", "achieved": 16.0 * px / t / 1e9, "peak": hbm, "unit": "GB/s",
                 "frac": 16.0 * px / t / 1e9 / hbm, "traffic": traffic,
                 "peak_note": f"HBM copy bandwidth of {peak_src} peaks",
@@ -665,7 +677,7 @@ def headline_batched(torch, rosar, args, device, world, stream, peaks, peak_src,
                               "reported beside it",
                 "frac_32B_per_px": 32.0 * px / t / 1e9 / hbm,
                 "plan_bytes_per_px": 8, "frac_with_plan_24B_per_px": 24.0 * px / t / 1e9 / hbm,
-                "us_per_launch": t * 1e6, "launches_per_step": 1}
+                "us_per_launch": t / launches * 1e6, "launches_per_step": launches}
     head = {"ms": ms, "t": t, "wall": wall, "px": px, "clocks": clk.summary(), "roofline": roofline,
             "tuning": vars(b.tuning), "autotune_ms": tuned["ms"], "autotune_cached": tuned.get("cached", False),
             "tiles": info}
@@ -822,12 +834,12 @@ def highres_bench(torch, rosar, device, world, hbm):
     return {"workload": "14400 pulses x 1024 samples, 1024 rows of K=128 taps (per-row weights), complex64",
             "image_fft_px_s": world * px / t_img, "ms_per_image": t_img * 1e3,
             "range_compress_kernel<1024>": {"us_per_launch": t_k1 * 1e6, "hbm_frac": 16.0 * px / t_k1 / 1e9 / hbm},
-            "azimuth_fft_fixed_kernel<1024, 14400, 8, 8, 15, 15>": {"us_per_launch": t_k2 * 1e6,
-                                                                      "hbm_frac": 24.0 * px / t_k2 / 1e9 / hbm}}
+            "azimuth_fft_fixed_kernel<512, 14400, 8, 8, 15, 15>": {"us_per_launch": t_k2 * 1e6,
+                                                                     "hbm_frac": 24.0 * px / t_k2 / 1e9 / hbm}}
 
 
 def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_src, compare_on):
-    """The indoor scan (3600 pulses x 256 samples, K=64 of M=600): the pipelined multi-scan call, the per-scan
+    """The indoor scan (3600 pulses x 256 samples, K=64 of M=600): the multi-scan call, the per-scan
     calls and the kernels alone, on 16 rotating scan buffers (354 MB), plus the paper's four methods on it."""
     import numpy as np
     cfg, sc, raw_stack, raws, w, o, win = indoor_inputs(torch, device, rank)
@@ -899,7 +911,6 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
     fp32_peak = sm_count * 128 * 2 * sm_mhz * 1e6 / 1e12
     sfu_peak = sm_count * 16 * sm_mhz * 1e6 / 1e12             # T SFU ops/s (16 per SM per clock)
     hbm = float(peaks["hbm_gbs"])
-    bf16_peak = float(peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops", 1700.0)))
     k1_bytes = 16.0 * px
     k2_bytes = 16.0 * px + 8.0 * cfg.L * K + 4.0 * K
     k2_flops = 8.0 * K * px
@@ -927,7 +938,7 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
             "us_per_launch": t_k2f * 1e6, "algorithmic_bytes": k2f_bytes, "gbs": k2f_bytes / t_k2f / 1e9,
             "hbm_frac": k2f_bytes / t_k2f / 1e9 / hbm,
             "traffic": recorded_traffic("azimuth_fft_fixed_kernel<3600>", "indoor",
-                                        source_hash("azimuth_fft.cu", "row_fft.cuh", "fft_tile.cuh")),
+                                        source_hash("azimuth_rows.cu", "row_fft.cuh", "fft_tile.cuh")),
             "plan_us_once": t_plan * 1e6},
         "fp32_peak_tflops": fp32_peak,
         "fp32_peak_note": f"FFMA: {sm_count} SMs x 128 lanes x 2 flop x {sm_mhz:.0f} MHz (sm_max_mhz of {peak_src} peaks)",
@@ -942,17 +953,14 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
         def call_ms(n, reps_=64):
             m_, _ = graph_loop(torch, lambda i: scans_call(n), reps_, 3, 1, stream, world, device)
             return m_ / reps_
-        t_stage = (call_ms(N_BUF) - call_ms(N_BUF // 2)) / (N_BUF - N_BUF // 2) * 1e-3
-        stage_name = "image_stage_kernel<256, 3600, 16, 15, 15>"
-        res["stage_kernel"] = {
-            "kernel": stage_name, "us_per_launch": t_stage * 1e6,
-            "frac_16B_per_px": 16.0 * px / t_stage / 1e9 / hbm, "frac_32B_per_px": 32.0 * px / t_stage / 1e9 / hbm,
-            "frac_40B_per_px": 40.0 * px / t_stage / 1e9 / hbm,
-            "traffic": recorded_traffic("image_stage_kernel<256,3600>", "indoor",
-                                        source_hash("image_pipeline.cu", "row_fft.cuh", "fft_tile.cuh")),
-            "note": "steady-state launch = (16-scan call - 8-scan call)/8; one launch range-compresses one scan "
-                    "and filters the previous one: 16 B/px minimum, 32 B/px with the S round trip, 40 B/px with "
-                    "the plan H"}
+        t_scan = (call_ms(N_BUF) - call_ms(N_BUF // 2)) / (N_BUF - N_BUF // 2) * 1e-3
+        res["scans_call"] = {
+            "kernels": "range_compress_kernel<256>, azimuth_fft_fixed_kernel<256, 3600, 16, 15, 15>",
+            "us_per_scan": t_scan * 1e6,
+            "frac_16B_per_px": 16.0 * px / t_scan / 1e9 / hbm, "frac_32B_per_px": 32.0 * px / t_scan / 1e9 / hbm,
+            "frac_40B_per_px": 40.0 * px / t_scan / 1e9 / hbm,
+            "note": "(16-scan call - 8-scan call)/8; two launches for the whole sequence, S written into the images and "
+                    "filtered in place: 16 B/px minimum, 32 B/px with the S round trip, 40 B/px with the plan H"}
         m, _ = graph_loop(torch, lambda i: image_step(i % N_BUF), max(512, steps // 4), 16, N_BUF, stream, world,
                           device)
         res["image_fft_per_scan_px_s"] = world * px / (m / max(512, steps // 4) * 1e-3)
@@ -983,8 +991,8 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
                 "img_fft_bpa": rosar.bpa(S_bufs[0], radar, cfg.L, cfg.M_ap).cpu().numpy(),
                 "img_bpa_time": rosar.bpa_time(raws[0], win, radar, cfg.L, cfg.M_ap).cpu().numpy(),
                 "img_sas_time": rosar.sas_time(raws[0], win, w, o, radar).cpu().numpy()}
-        # planned forms: the B operand (coefficient x window x phasor) computed once per weight design; a plan
-        # build is timed on its second call (the first loads the kernels and allocates the plan's memory)
+        # planned forms: the taps' transforms computed once per weight design; a plan build is timed on its second call
+        # (the first loads the kernels and allocates the plan's memory)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         splan = rosar.sas_time_plan(win, w, o, radar, cfg.n_az, cfg.L)
         torch.cuda.synchronize()
@@ -1011,52 +1019,38 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
         del bplan
         t_bj, t_bn = ms_bj / 20 * 1e-3, ms_bn / 20 * 1e-3
         t_bt, t_st = ms_bt / 3 * 1e-3, ms_st / 20 * 1e-3
-        f_bt = 8.0 * cfg.M_ap * cfg.L * px
-        f_st = 8.0 * cfg.K * cfg.L * px
+
+        def frac16(t):
+            return 16.0 * px / t / 1e9 / hbm
         pp = float(cfg.M_ap) * px                              # pixel-pulses of one BPA image
         res["compare"] = {
             "fft_bpa_px_s": world * px / (t_bj + t_k1), "fft_bpa_nominal_px_s": world * px / (t_bn + t_k1),
-            "bpa_kernel<0,1> (supplied errors)": dict(bpa_entry(t_bj, pp, BPA_FLOPS_ERR, 4, fp32_peak, sfu_peak),
-                                  traffic=recorded_traffic("bpa_kernel<0,1>", "indoor", source_hash("bpa.cu"))),
-            "bpa_kernel<1,1> (nominal)": dict(bpa_entry(t_bn, pp, BPA_FLOPS_NOM, 0, fp32_peak, sfu_peak),
-                                  traffic=recorded_traffic("bpa_kernel<1,1>", "indoor", source_hash("bpa.cu"))),
-            "bpa_note": "bpa_kernel<NOMINAL, LINEAR>, linear interpolation; algorithmic work per "
-                        "pixel-pulse: nominal 12 flop (linear interpolation 4, complex MAC 8), supplied errors "
-                        "34 flop and 4 SFU ops (rsqrt, reciprocal, sine, cosine); peaks derived at the measured "
-                        "SM clock: FP32 152 SMs x 128 lanes x 2 flop, SFU 152 SMs x 16 ops per clock; both "
-                        "variants are bound by instruction issue (ncu: 76-86 % issue active)",
+            "bpa_errors2_kernel<1> (supplied errors)": bpa_entry(t_bj, pp, BPA_FLOPS_ERR, 4, fp32_peak, sfu_peak),
+            "bpa_rows_kernel (nominal)": {"us_per_call": t_bn * 1e6, "hbm_frac_16B_per_px": frac16(t_bn)},
+            "bpa_note": "linear interpolation; supplied errors: algorithmic work per pixel-pulse 34 flop and 4 SFU ops "
+                        "(rsqrt, reciprocal, sine, cosine), peaks derived at the measured SM clock: FP32 152 SMs x 128 "
+                        "lanes x 2 flop, SFU 152 SMs x 16 ops per clock; nominal: per range row circular correlations "
+                        "in the azimuth-frequency domain (S in, image out: 16 B/px)",
             "bpa_time_px_s": world * px / t_bt, "sas_time_px_s": world * px / t_st,
-            "td_tcg_kernel<BPA>": {"us_per_launch": t_bt * 1e6, "tflops": f_bt / t_bt / 1e12,
-                                  "tensor_frac": 3 * f_bt / t_bt / 1e12 / bf16_peak,
-                                  "traffic": recorded_traffic("td_tcg_kernel<1>", "indoor", source_hash("time_domain.cu"))},
-            "td_tcg_kernel<SAS>": {"us_per_launch": t_st * 1e6, "tflops": f_st / t_st / 1e12,
-                                  "tensor_frac": 3 * f_st / t_st / 1e12 / bf16_peak,
-                                  "traffic": recorded_traffic("td_tcg_kernel<0>", "indoor", source_hash("time_domain.cu"))},
+            "time-domain BPA": {"us_per_call": t_bt * 1e6, "hbm_frac_16B_per_px": frac16(t_bt)},
+            "time-domain SAS": {"us_per_call": t_st * 1e6, "hbm_frac_16B_per_px": frac16(t_st)},
             "planned": {
-                "td_tcw_kernel<SAS>": {"us_per_launch": t_stp * 1e6, "tflops": f_st / t_stp / 1e12,
-                                       "tensor_frac": 3 * f_st / t_stp / 1e12 / bf16_peak,
-                                       "plan_us_once": t_splan * 1e6, "plan_MB": plan_mb[0],
-                                       "traffic": recorded_traffic("td_tcw_kernel<0>", "indoor",
-                                                                   source_hash("time_domain.cu"))},
-                "td_tcw_kernel<BPA>": {"us_per_launch": t_btp * 1e6, "tflops": f_bt / t_btp / 1e12,
-                                       "tensor_frac": 3 * f_bt / t_btp / 1e12 / bf16_peak,
-                                       "plan_us_once": t_bplan * 1e6, "plan_MB": plan_mb[1],
-                                       "traffic": recorded_traffic("td_tcw_kernel<1>", "indoor",
-                                                                   source_hash("time_domain.cu"))},
-                "note": "B operand (coefficient x window x phasor, bf16 hi/lo, tiled as the tensor cores read it) "
-                        "computed once per weight design; per scan the kernel stages one window of raw pulses per "
-                        "16-sample chunk shared by all taps within 120 pulses, and streams the B tiles by bulk copy; "
-                        "plan_us_once is one plan build (the paper's W_BP / W_SA, computed per image there)"},
+                "time-domain SAS": {"us_per_call": t_stp * 1e6, "hbm_frac_16B_per_px": frac16(t_stp),
+                                    "plan_us_once": t_splan * 1e6, "plan_MB": plan_mb[0]},
+                "time-domain BPA": {"us_per_call": t_btp * 1e6, "hbm_frac_16B_per_px": frac16(t_btp),
+                                    "plan_us_once": t_bplan * 1e6, "plan_MB": plan_mb[1]},
+                "note": "azimuth transforms of the taps' low-rank planes computed once per weight design; per scan the "
+                        "pulses are transformed, combined with the planes and transformed back; plan_us_once is one "
+                        "plan build (the paper's W_BP / W_SA, computed per image there)"},
             "paper_table_ms_per_image": {"BPA": t_bt * 1e3, "SAS": t_st * 1e3,
-                                         "BPA (B built per image + planned kernel)": (t_bplan + t_btp) * 1e3,
-                                         "SAS (B built per image + planned kernel)": (t_splan + t_stp) * 1e3,
+                                         "BPA (plan built per image)": (t_bplan + t_btp) * 1e3,
+                                         "SAS (plan built per image)": (t_splan + t_stp) * 1e3,
                                          "FFT+BPA": (t_bn + t_k1) * 1e3,
                                          "FFT+SAS": ms / steps, "FFT+SAS (per-pulse peak bins)": t_migf_img * 1e3},
             "note": "FFT+BPA = range compression + back-projection over M=600 pulses (nominal geometry; the "
                     "supplied-error variant is timed beside it); BPA / SAS = time-domain forms (Eq. (14); "
-                    "Algorithm 2 with W_SA) on the tensor cores, unplanned (B generated in the kernel) and with B "
-                    "built per image by the plan kernels then the planned kernel; tensor_frac of the measured "
-                    "sustained bf16 peak executed (3 split-bf16 products per term); FFT+SAS = the timed indoor path"}
+                    "Algorithm 2 with W_SA) evaluated by transforms, the plan built within the call, and with a kept plan; "
+                    "FFT+SAS = the timed indoor path"}
         res["highres"] = highres_bench(torch, rosar, device, world, hbm)
     return res, indoor_img, (cfg, sc, w, o, win)
 
@@ -1209,7 +1203,7 @@ def run_ours(args):
     peaks, peak_src = measured_peaks()
     hbm = float(peaks["hbm_gbs"])
 
-    # ---- headline: the batched workload, one persistent graph launch per step
+    # ---- headline: the batched workload, one graph launch per step
     wl, b, head = headline_batched(torch, rosar, args, device, world, stream, peaks, peak_src, local)
     value = world * head["px"] / head["t"]
     batched = {"scans": len(wl.cfgs), "pixels": wl.px, "px_s": value, "ms_per_batch": head["t"] * 1e3,
@@ -1278,11 +1272,12 @@ def run_ours(args):
                                "each scan's plan H, computed once from its weights outside the timed region)",
                        "l2": "inputs larger than L2: every step reads 3.85 GB of raw cubes and writes 3.85 GB of "
                              "images (129 MB L2)",
-                       "launch": "one CUDA graph per step: counter reset + one persistent kernel (tiles from an "
-                                 "atomic ticket counter), no host work between steps",
+                       "launch": "one CUDA graph per step: one range launch per pulse length and one azimuth launch per "
+                                 "row length (or, if the tuner finds it faster, one persistent kernel), no host work "
+                                 "between steps",
                        "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
             "clocks": head["clocks"],
-            "gpu_launches": args.steps,
+            "gpu_launches": args.steps * head["roofline"]["launches_per_step"],
             "roofline": head["roofline"],
             "e2e": e2e,
             "cpu_baseline": cpu,
@@ -1332,8 +1327,8 @@ def kernel_cases(args):
         ("range_compress_kernel", lambda: rosar.range_compress(raws[0], win, out=S)),
         ("sparse_azimuth_kernel", lambda: rosar.sparse_azimuth(S, w, o)),
         ("azimuth_fft_fixed_kernel", lambda: rosar.sparse_azimuth_fft(S, H)),
-        ("bpa_kernel<nominal>", lambda: rosar.bpa(S, radar, cfg.L, cfg.M_ap)),
-        ("bpa_kernel<supplied errors>", lambda: rosar.bpa(S, radar, cfg.L, cfg.M_ap, dphi=dphi, dr=dr)),
+        ("bpa nominal", lambda: rosar.bpa(S, radar, cfg.L, cfg.M_ap)),
+        ("bpa supplied errors", lambda: rosar.bpa(S, radar, cfg.L, cfg.M_ap, dphi=dphi, dr=dr)),
         ("migrating spectrum + combine", lambda: rosar.sparse_azimuth_migrating_fft(S, mplan)),
         ("diff forward filter", lambda: rosar.sparse_azimuth_fft_scans_ex(stack, H, P=P, spectrum=X)),
         ("loss partial + final", lambda: rosar.image_l2_loss(stack, ref)),
@@ -1341,12 +1336,12 @@ def kernel_cases(args):
         ("diff adjoint filter", lambda: rosar.sparse_azimuth_fft_scans_ex(g, H, adjoint=True, spectrum=G)),
         ("weight grad (accumulate + taps)", lambda: rosar.azimuth_weight_grad_spectra(G, X, o, cfg.K)),
         ("phase grad", lambda: rosar.phase_grad_phasor(stack, P, g)),
-        ("image_stage_kernel (3 scans)", lambda: rosar.image_fft_scans(raw_stack[:3], win, H, workspace=ws2)),
-        (f"batch_kernel ({args.kernel_cases} scans)", lambda: b.launch()),
-        ("td_tcg_kernel<BPA> (unplanned call)", lambda: rosar.bpa_time(raws[0], win, radar, cfg.L, cfg.M_ap)),
-        ("td_tcg_kernel<SAS> (unplanned call)", lambda: rosar.sas_time(raws[0], win, w, o, radar)),
-        ("td_tcw_kernel<BPA>", lambda: rosar.bpa_time_planned(raws[0], bplan)),
-        ("td_tcw_kernel<SAS>", lambda: rosar.sas_time_planned(raws[0], splan)),
+        ("scans call (3 scans)", lambda: rosar.image_fft_scans(raw_stack[:3], win, H, workspace=ws2)),
+        (f"batch ({args.kernel_cases} scans)", lambda: b.launch()),
+        ("time-domain BPA (unplanned call)", lambda: rosar.bpa_time(raws[0], win, radar, cfg.L, cfg.M_ap)),
+        ("time-domain SAS (unplanned call)", lambda: rosar.sas_time(raws[0], win, w, o, radar)),
+        ("time-domain BPA (planned)", lambda: rosar.bpa_time_planned(raws[0], bplan)),
+        ("time-domain SAS (planned)", lambda: rosar.sas_time_planned(raws[0], splan)),
     ]
     for _ in range(2):
         for _, c in calls:
