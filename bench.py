@@ -1025,8 +1025,13 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
         pp = float(cfg.M_ap) * px                              # pixel-pulses of one BPA image
         res["compare"] = {
             "fft_bpa_px_s": world * px / (t_bj + t_k1), "fft_bpa_nominal_px_s": world * px / (t_bn + t_k1),
-            "bpa_errors2_kernel<1> (supplied errors)": bpa_entry(t_bj, pp, BPA_FLOPS_ERR, 4, fp32_peak, sfu_peak),
-            "bpa_rows_kernel (nominal)": {"us_per_call": t_bn * 1e6, "hbm_frac_16B_per_px": frac16(t_bn)},
+            "bpa_errors2_kernel<1> (supplied errors)": dict(
+                bpa_entry(t_bj, pp, BPA_FLOPS_ERR, 4, fp32_peak, sfu_peak),
+                traffic=recorded_traffic("bpa_errors2_kernel<1>", "indoor", source_hash("bpa.cu"))),
+            "bpa_rows_kernel (nominal)": {
+                "us_per_call": t_bn * 1e6, "hbm_frac_16B_per_px": frac16(t_bn),
+                "traffic": recorded_traffic("bpa_rows_kernel", "indoor",
+                                            source_hash("bpa_fft.cu", "bpa_geometry.cuh", "row_fft.cuh", "fft_tile.cuh"))},
             "bpa_note": "linear interpolation; supplied errors: algorithmic work per pixel-pulse 34 flop and 4 SFU ops "
                         "(rsqrt, reciprocal, sine, cosine), peaks derived at the measured SM clock: FP32 152 SMs x 128 "
                         "lanes x 2 flop, SFU 152 SMs x 16 ops per clock; nominal: per range row circular correlations "
