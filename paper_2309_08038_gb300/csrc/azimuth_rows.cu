@@ -217,18 +217,6 @@ rosar_status launch_rows_of(const RowLaunch &l, const ROWS &rows) {
     if (plan_is<14400, 8, 8, 15, 15>(l.n_az, pl))
         return l.n_rng <= 152 ? launch_fixed<ROWS, 1024, 1, 14400, kFused, 8, 8, 15, 15>(l, rows)
                               : launch_fixed<ROWS, 512, 2, 14400, kStreamed, 8, 8, 15, 15>(l, rows);
-    if (plan_is<3600, 16, 15, 15>(l.n_az, pl))
-        return few ? launch_fixed<ROWS, 256, 2, 3600, kStaged, 16, 15, 15>(l, rows)
-                   : launch_fixed<ROWS, 256, 4, 3600, kFused, 16, 15, 15>(l, rows);
-    if (plan_is<1800, 8, 15, 15>(l.n_az, pl))
-        return few ? launch_fixed<ROWS, 256, 2, 1800, kStaged, 8, 15, 15>(l, rows)
-                   : launch_fixed<ROWS, 128, 8, 1800, kFused, 8, 15, 15>(l, rows);
-    if (plan_is<7200, 8, 4, 15, 15>(l.n_az, pl))
-        return l.n_rng <= 152 ? launch_fixed<ROWS, 512, 1, 7200, kStaged, 8, 4, 15, 15>(l, rows)
-                              : launch_fixed<ROWS, 256, 3, 7200, kFused, 8, 4, 15, 15>(l, rows);
-    if (plan_is<14400, 8, 8, 15, 15>(l.n_az, pl))
-        return l.n_rng <= 152 ? launch_fixed<ROWS, 1024, 1, 14400, false, 8, 8, 15, 15>(l, rows)
-                              : launch_fixed<ROWS, 512, 2, 14400, false, 8, 8, 15, 15>(l, rows);
     if (plan_is<360, 8, 3, 15>(l.n_az, pl))
         return few ? launch_fixed<ROWS, 256, 2, 360, kStaged, 8, 3, 15>(l, rows)
                    : launch_fixed<ROWS, 64, 8, 360, kFused, 8, 3, 15>(l, rows);
