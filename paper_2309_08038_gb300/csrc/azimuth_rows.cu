@@ -121,13 +121,14 @@ azimuth_fft_kernel(ROWS rows, int N, RowPlan pl, Layout lay) {
 
 // Compile-time plan for one row length (T threads, no padding: N has an odd factor): the first pass reads S from
 // global memory, the last writes the image, and the last forward pass, the product with H and the first inverse pass
-// run as one step (row_filter_fused): four barriers for 16.15.15.  H_FROM: where H is read (HSource).
-template <typename ROWS, int T, int MINB, int N, int H_FROM, int... R>
+// run as one step (row_filter_fused): four barriers for 16.15.15.  H_FROM: where H is read (HSource).  PAIRED:
+// the two outermost passes of each transform in registers (row_filter_paired).
+template <typename ROWS, int T, int MINB, int N, int H_FROM, bool PAIRED, int... R>
 __global__ void __launch_bounds__(T, MINB)
 azimuth_fft_fixed_kernel(ROWS rows) {
     extern __shared__ float2 sm[];
     const RowRef ref = rows.at(blockIdx.x, N);
-    filter_row_cta<T, N, H_FROM, R...>(ref.S, ref.H, ref.conj_h, ref.out, sm, ref.phase, ref.spec);
+    filter_row_cta<T, N, H_FROM, PAIRED, R...>(ref.S, ref.H, ref.conj_h, ref.out, sm, ref.phase, ref.spec);
 }
 
 }  // namespace
@@ -156,12 +157,12 @@ struct RowLaunch {
     cudaStream_t s;
 };
 
-template <typename ROWS, int T, int MINB, int N, int H_FROM, int... R>
+template <typename ROWS, int T, int MINB, int N, int H_FROM, bool PAIRED, int... R>
 rosar_status launch_fixed(const RowLaunch &l, const ROWS &rows) {
     static int done[kMaxDevices] = {};
     constexpr size_t smem = filter_row_smem<N, H_FROM>();
     static_assert(smem <= 200 * 1024, "the staged rows exceed the shared-memory cap");
-    const auto kernel = azimuth_fft_fixed_kernel<ROWS, T, MINB, N, H_FROM, R...>;
+    const auto kernel = azimuth_fft_fixed_kernel<ROWS, T, MINB, N, H_FROM, PAIRED, R...>;
     rosar_status st = ensure_smem((const void *)kernel, smem, done, "azimuth_fft");
     if (st != ROSAR_OK || l.only_prepare) return st;
     const cudaError_t e = launch_overlapped(kernel, l.n_rng, T, smem, l.overlap, l.s, rows);
@@ -194,7 +195,8 @@ bool plan_is(int n_az, const RowPlan &pl) {
 // rows in flight count: one row of shared memory and at most 64 registers hold 4 CTAs of 3600 pulses (46 % of the
 // warps instead of 30) or 8 of 1800, and H is read in the fused step.  4096 rows of 3600 pulses 82 -> 77 us, 8192 of
 // 1800 97 -> 76; at 256 rows 10.3 and 10.4, 6.4 and 8.2.  7200-pulse rows hold one CTA an SM with H staged: 152 rows
-// 10.2 us (11.3 not staged), 256 rows 18.4 -> 15.8, 1024 rows 72 -> 54.
+// 10.2 us (11.3 not staged).  With more rows three CTAs an SM and the passes of radix 8 and 4 together in registers
+// (PAIRED): 256 rows 18.4 -> 15.8 -> 13.8, 1024 rows 72 -> 54 -> 47, 4096 rows 271 -> 186 -> 159 (176 on two CTAs).
 constexpr int kFewRows = 304;
 
 template <typename ROWS>
@@ -204,22 +206,22 @@ rosar_status launch_rows_of(const RowLaunch &l, const ROWS &rows) {
         return set_error(ROSAR_ERR_UNSUPPORTED, "azimuth_fft: n_az=%d is not 2^a 3^b 5^c in [2, %d]", l.n_az, AF_MAX_N);
     const bool few = l.n_rng <= kFewRows;
     if (plan_is<3600, 16, 15, 15>(l.n_az, pl))
-        return few ? launch_fixed<ROWS, 256, 2, 3600, kStaged, 16, 15, 15>(l, rows)
-                   : launch_fixed<ROWS, 256, 4, 3600, kFused, 16, 15, 15>(l, rows);
+        return few ? launch_fixed<ROWS, 256, 2, 3600, kStaged, false, 16, 15, 15>(l, rows)
+                   : launch_fixed<ROWS, 256, 4, 3600, kFused, false, 16, 15, 15>(l, rows);
     if (plan_is<1800, 8, 15, 15>(l.n_az, pl))
-        return few ? launch_fixed<ROWS, 256, 2, 1800, kStaged, 8, 15, 15>(l, rows)
-                   : launch_fixed<ROWS, 128, 8, 1800, kFused, 8, 15, 15>(l, rows);
+        return few ? launch_fixed<ROWS, 256, 2, 1800, kStaged, false, 8, 15, 15>(l, rows)
+                   : launch_fixed<ROWS, 128, 8, 1800, kFused, false, 8, 15, 15>(l, rows);
     if (plan_is<7200, 8, 4, 15, 15>(l.n_az, pl))
-        return l.n_rng <= 152 ? launch_fixed<ROWS, 512, 1, 7200, kStaged, 8, 4, 15, 15>(l, rows)
-                              : launch_fixed<ROWS, 256, 3, 7200, kFused, 8, 4, 15, 15>(l, rows);
+        return l.n_rng <= 152 ? launch_fixed<ROWS, 512, 1, 7200, kStaged, false, 8, 4, 15, 15>(l, rows)
+                              : launch_fixed<ROWS, 256, 3, 7200, kFused, true, 8, 4, 15, 15>(l, rows);
     // 14400: one row an SM on 1024 threads, or two on 512 each.  152 rows 15.8 us (17.0 streamed); 256 rows 32.8 -> 28.9,
     // 1024 rows 130 -> 115 (two rows an SM with the fused step 133, one with the streamed step 140).
     if (plan_is<14400, 8, 8, 15, 15>(l.n_az, pl))
-        return l.n_rng <= 152 ? launch_fixed<ROWS, 1024, 1, 14400, kFused, 8, 8, 15, 15>(l, rows)
-                              : launch_fixed<ROWS, 512, 2, 14400, kStreamed, 8, 8, 15, 15>(l, rows);
+        return l.n_rng <= 152 ? launch_fixed<ROWS, 1024, 1, 14400, kFused, false, 8, 8, 15, 15>(l, rows)
+                              : launch_fixed<ROWS, 512, 2, 14400, kStreamed, false, 8, 8, 15, 15>(l, rows);
     if (plan_is<360, 8, 3, 15>(l.n_az, pl))
-        return few ? launch_fixed<ROWS, 256, 2, 360, kStaged, 8, 3, 15>(l, rows)
-                   : launch_fixed<ROWS, 64, 8, 360, kFused, 8, 3, 15>(l, rows);
+        return few ? launch_fixed<ROWS, 256, 2, 360, kStaged, false, 8, 3, 15>(l, rows)
+                   : launch_fixed<ROWS, 64, 8, 360, kFused, false, 8, 3, 15>(l, rows);
     // The run-time plan: the staged H row pays where a row's own latency counts.  Against loading the row, the passes,
     // the product and the store as steps of their own: 800 pulses, 256 rows 8.3 -> 7.1 us, 2048 rows 47 -> 22; 4500:
     // 23.9 -> 19.7 and 165 -> 89; 16384: 76 -> 51 (256 rows).

@@ -535,6 +535,82 @@ __device__ __forceinline__ void dit_last_global(const float2 *x, float2 *__restr
     }
 }
 
+// The first two DIF passes (radices R1 and R2) of one element in N/(R1 R2) together in registers, read from global
+// memory, and their transposes written to it: the same products in the same order as dif_first_global and dif_pass_c,
+// dit_pass_c and dit_last_global, with a trip of the row through shared memory and a barrier fewer each way.
+template <int N, int R1, int R2, int T, bool WAIT_ASYNC>
+__device__ __forceinline__ void dif_first_two_global(const float2 *__restrict__ src, float2 *x, const float2 *tc,
+                                                     const float2 *tf, const float2 *__restrict__ phase) {
+    constexpr int s1 = N / R1, s2 = s1 / R2;
+#pragma unroll 1
+    for (int j = threadIdx.x; j < s2; j += T) {
+        float2 v[R2][R1];
+#pragma unroll
+        for (int t = 0; t < R2; ++t)
+#pragma unroll
+            for (int r = 0; r < R1; ++r) v[t][r] = __ldcg(src + j + t * s2 + r * s1);
+        if (phase) {
+#pragma unroll
+            for (int t = 0; t < R2; ++t)
+#pragma unroll
+                for (int r = 0; r < R1; ++r) v[t][r] = cmul(v[t][r], __ldg(phase + j + t * s2 + r * s1));
+        }
+#pragma unroll
+        for (int t = 0; t < R2; ++t) {
+            small_dft<R1>(v[t]);
+            float2 wq[R1];
+            twiddle_powers<R1>(twiddle_of<N>(j + t * s2, tc, tf), wq);
+#pragma unroll
+            for (int q = 1; q < R1; ++q) v[t][q] = cmul(v[t][q], wq[q]);
+        }
+        float2 wp[R2];
+        twiddle_powers<R2>(twiddle_of<N>(j * R1, tc, tf), wp);
+#pragma unroll
+        for (int q = 0; q < R1; ++q) {
+            float2 u[R2];
+#pragma unroll
+            for (int t = 0; t < R2; ++t) u[t] = v[t][q];
+            small_dft<R2>(u);
+            x[q * s1 + j] = u[0];
+#pragma unroll
+            for (int p = 1; p < R2; ++p) x[q * s1 + p * s2 + j] = cmul(u[p], wp[p]);
+        }
+    }
+    if (WAIT_ASYNC) cp_async_wait<0>();
+    __syncthreads();
+}
+
+template <int N, int R1, int R2, int T>
+__device__ __forceinline__ void dit_last_two_global(const float2 *x, float2 *__restrict__ dst, const float2 *tc,
+                                                    const float2 *tf) {
+    constexpr int s1 = N / R1, s2 = s1 / R2;
+#pragma unroll 1
+    for (int j = threadIdx.x; j < s2; j += T) {
+        float2 v[R2][R1], wp[R2];
+        twiddle_powers<R2>(twiddle_of<N>(j * R1, tc, tf), wp);
+#pragma unroll
+        for (int q = 0; q < R1; ++q) {
+            float2 u[R2];
+            u[0] = x[q * s1 + j];
+#pragma unroll
+            for (int p = 1; p < R2; ++p) u[p] = cmul(x[q * s1 + p * s2 + j], wp[p]);
+            small_dft<R2>(u);
+#pragma unroll
+            for (int t = 0; t < R2; ++t) v[t][q] = u[t];
+        }
+#pragma unroll
+        for (int t = 0; t < R2; ++t) {
+            float2 wq[R1];
+            twiddle_powers<R1>(twiddle_of<N>(j + t * s2, tc, tf), wq);
+#pragma unroll
+            for (int q = 1; q < R1; ++q) v[t][q] = cmul(v[t][q], wq[q]);
+            small_dft<R1>(v[t]);
+#pragma unroll
+            for (int r = 0; r < R1; ++r) dst[j + t * s2 + r * s1] = make_float2(v[t][r].x, -v[t][r].y);
+        }
+    }
+}
+
 template <int N, int M, int T, int H_FROM, int R, int... Rest>
 __device__ __forceinline__ void filter_middle(float2 *x, const float2 *h, float hs, const float2 *tc, const float2 *tf,
                                               float2 *__restrict__ spec = nullptr) {
@@ -563,6 +639,16 @@ __device__ __forceinline__ void row_filter_fused(const float2 *src, const float2
     dif_first_global<N, R1, T, H_FROM == kStaged>(src, x, tc, tf, discard, phase);
     filter_middle<N, N / R1, T, H_FROM, Rs...>(x, h, hs, tc, tf, spec);
     dit_last_global<N, R1, T>(x, dst, tc, tf);
+}
+
+// row_filter_fused with the two outermost passes of each transform in registers.
+template <int N, int T, int H_FROM, int R1, int R2, int... Rs>
+__device__ __forceinline__ void row_filter_paired(const float2 *src, const float2 *h, float hs, float2 *x, float2 *dst,
+                                                  const float2 *tc, const float2 *tf, const float2 *__restrict__ phase,
+                                                  float2 *__restrict__ spec) {
+    dif_first_two_global<N, R1, R2, T, H_FROM == kStaged>(src, x, tc, tf, phase);
+    filter_middle<N, N / (R1 * R2), T, H_FROM, Rs...>(x, h, hs, tc, tf, spec);
+    dit_last_two_global<N, R1, R2, T>(x, dst, tc, tf);
 }
 
 // Forward DFT of the row, output in digit-reversed order.
@@ -734,7 +820,7 @@ constexpr size_t filter_row_smem() {
     return sizeof(float2) * (size_t)((H_FROM == kStaged ? 2 : 1) * padded_len(N) + 64 + coarse_len(N));
 }
 
-template <int T, int N, int H_FROM, int... R>
+template <int T, int N, int H_FROM, bool PAIRED, int... R>
 __device__ __forceinline__ void filter_row_cta(const float2 *S_row, const float2 *__restrict__ H_row,
                                                bool conj_h, float2 *out_row, float2 *sm,
                                                const float2 *__restrict__ phase = nullptr,
@@ -754,8 +840,10 @@ __device__ __forceinline__ void filter_row_cta(const float2 *S_row, const float2
         __syncthreads();
     }
     griddep_wait();                          // S is complete (no-op unless launched to overlap its producer)
-    row_filter_fused<N, T, H_FROM, R...>(S_row, H_FROM == kStaged ? hb : H_row, conj_h ? -1.f : 1.f, x, out_row, tc, tf, false,
-                                         phase, spec);
+    const float2 *h = H_FROM == kStaged ? hb : H_row;
+    const float hs = conj_h ? -1.f : 1.f;
+    if constexpr (PAIRED) row_filter_paired<N, T, H_FROM, R...>(S_row, h, hs, x, out_row, tc, tf, phase, spec);
+    else row_filter_fused<N, T, H_FROM, R...>(S_row, h, hs, x, out_row, tc, tf, false, phase, spec);
 }
 
 inline int threads_for(int N) { return N <= 4096 ? 256 : N <= 8192 ? 512 : 1024; }
