@@ -606,8 +606,8 @@ rosar_status rosar_image_fft_scans(const rosar_c32 *raw, const float *win, const
         return set_error(ROSAR_ERR_UNSUPPORTED, "image_fft_scans: n_az=%d is not 2^a 3^b 5^c <= 16384", n_az);
     // Range compression of a group of scans straight into their images' place, then their rows filtered where they lie:
     // two launches for the whole sequence, each of many waves.  One launch per scan overlapped with the next scan's
-    // range tiles was 148 us for 16 scans of 3600 x 256 (9.3 us a scan); the two launches take 118.  Smaller groups, whose
-    // S would still lie in L2, are slower: 8 scans 120, 4 scans 132 us.
+    // range tiles was 148 us for 16 scans of 3600 x 256 (9.3 us a scan); the two launches take 113.  Smaller groups, whose
+    // S would still lie in L2, are slower: where all scans took 118, groups of 8 took 120, of 4 132 us.
     const size_t elems = (size_t)n_az * L;
     const long long by_rows = (1LL << 30) / L;
     const int group = by_rows < 65535 ? (int)by_rows : 65535;
