@@ -145,9 +145,11 @@ def _up256(n):
     return (n + 255) & ~255
 
 
-def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None):
-    """rosar_bpa_time: time-domain back-projection (Eq. (14)) of the raw cube [n_az, L] onto rows 0..n_rng-1; by
-    transforms (rosar_bpa_time_fft, plan and workspace allocated here) where the library offers that for the sizes."""
+def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None, transforms=False):
+    """rosar_bpa_time: time-domain back-projection (Eq. (14)) of the raw cube [n_az, L] onto rows 0..n_rng-1.
+    transforms=True: by transforms (rosar_bpa_time_fft, plan and workspace allocated here) where the library offers that
+    for the sizes.  Single pixels of the two forms differ by up to 1.1e-3 of the larger of the pixel and the image's rms
+    (beside strong targets, by the tensor cores' rounding), so the caller chooses."""
     lib = _lib.load()
     require(raw, torch.complex64, "raw", ndim=2)
     n_az, L = raw.shape
@@ -157,7 +159,7 @@ def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None):
         out = torch.empty((n_rng, n_az), dtype=torch.complex64, device=raw.device)
     require(out, torch.complex64, "out", shape=(n_rng, n_az))
     st = radar.as_struct()
-    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 1, n_az, L, n_rng, M_ap)
+    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 1, n_az, L, n_rng, M_ap) if transforms else 0
     if nbytes and raw.data_ptr() % 16 == 0:
         at, ws = _up256(nbytes), lib.rosar_time_domain_fft_workspace_bytes(1, n_az, L, n_rng, M_ap)
         scratch = _scratch(at + ws, raw.device, stream)
@@ -204,7 +206,7 @@ def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
 @dataclass(frozen=True)
 class TimeDomainPlan:
     """What the time-domain forms compute once per weight design, with the shape it was made for: a uint8 device
-    tensor, either the transform form's plan (rosar_*_time_fft_plan, where the library offers it for the sizes) or the
+    tensor, either the transform form's plan (rosar_*_time_fft_plan, for BPA where the caller asked for it) or the
     precomputed B operand of the tensor-core forms (rosar_*_time_plan: rosar_time_domain_plan_bytes(n_rng, L, K)
     bytes, which the other's size never equals)."""
 
@@ -260,14 +262,15 @@ def sas_time_planned(raw, plan: TimeDomainPlan, out=None, stream=None):
     return _planned(raw, plan, 0, lib.rosar_sas_time_planned, lib.rosar_sas_time_fft, out, stream)
 
 
-def bpa_time_plan(win, radar: Radar, n_az, L, n_rng, M_ap, device=None, stream=None):
-    """rosar_bpa_time_plan or rosar_bpa_time_fft_plan: the plan of rosar_bpa_time (M_ap taps of the nominal geometry)."""
+def bpa_time_plan(win, radar: Radar, n_az, L, n_rng, M_ap, device=None, stream=None, transforms=False):
+    """rosar_bpa_time_plan: the B operand of rosar_bpa_time (M_ap taps of the nominal geometry).  transforms=True: the
+    plan of rosar_bpa_time_fft (rosar_bpa_time_fft_plan) where the library offers that form (see bpa_time)."""
     lib = _lib.load()
     if win is not None:
         require(win, torch.float32, "win", shape=(L,))
     device = win.device if win is not None else (device or torch.device("cuda"))
     st = radar.as_struct()
-    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 1, n_az, L, n_rng, M_ap)
+    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 1, n_az, L, n_rng, M_ap) if transforms else 0
     data = torch.empty(nbytes, dtype=torch.uint8, device=device) if nbytes else _plan_tensor(n_rng, L, M_ap, device)
     make = lib.rosar_bpa_time_fft_plan if nbytes else lib.rosar_bpa_time_plan
     check(make(ptr(win), ctypes.byref(st), n_az, L, n_rng, M_ap, ptr(data), data.numel(), stream_handle(stream)))
