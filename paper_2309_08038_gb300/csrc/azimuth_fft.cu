@@ -196,8 +196,7 @@ xspec_accumulate_kernel(const float2 *__restrict__ G, const float2 *__restrict__
     P[i] = p;
 }
 
-// rk > 0: the spectra came from the compile-time-plan filter, stored radix-major for its last radix rk (element
-// i = q*(N/rk) + b holds digit-reversed position b*rk + q); rk == 0: stored in digit-reversed order.
+// rk: the order of the spectra, stored_radix of the row length.
 template <typename INV>
 __device__ __forceinline__ void xspec_taps_row(const float2 *__restrict__ Pg, const int32_t *__restrict__ o,
                                                int o_row_stride, int K, int N, int pad_shift, int rk,
@@ -226,8 +225,8 @@ __device__ __forceinline__ void xspec_taps_row(const float2 *__restrict__ Pg, co
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
 xspec_taps_kernel(const float2 *__restrict__ P, const int32_t *__restrict__ o, int o_row_stride, int K, int N,
-                  RowPlan pl, float2 *__restrict__ grad_w) {
-    xspec_taps_row(P, o, o_row_stride, K, N, pl.pad_shift, 0, grad_w,
+                  RowPlan pl, int rk, float2 *__restrict__ grad_w) {
+    xspec_taps_row(P, o, o_row_stride, K, N, pl.pad_shift, rk, grad_w,
                    [&](float2 *x, const float2 *tc, const float2 *tf) { row_dit(x, N, pl, tc, tf); });
 }
 
@@ -333,10 +332,8 @@ namespace {
 template <int T, int N, int... R>
 bool try_xspec_taps_fixed(int n_az, const RowPlan &pl, const float2 *P, const int32_t *o, int o_row_stride, int n_rng,
                           int K, float2 *grad_w, cudaStream_t s, rosar_status *st) {
-    constexpr int rad[] = {R...};
-    if (n_az != N || threads_for(N) != T || pl.pad_shift != 31 || pl.npass != (int)sizeof...(R)) return false;
-    for (int i = 0; i < pl.npass; ++i)
-        if (pl.rad[i] != rad[i]) return false;
+    if (threads_for(N) != T || !FixedRadices<N, R...>::is(n_az, pl) || stored_radix(n_az, pl) != last_radix<R...>())
+        return false;
     static int done[kMaxDevices] = {};
     const size_t smem = sizeof(float2) * ((size_t)padded_len(N) + 64 + coarse_len(N));
     *st = ensure_smem((const void *)xspec_taps_fixed_kernel<T, N, R...>, smem, done, "weight_grad_spectra");
@@ -364,14 +361,15 @@ rosar_status launch_azimuth_weight_grad_spectra(const float2 *G, const float2 *X
         try_xspec_taps_fixed<256, 360, 8, 3, 15>(n_az, pl, P, o, o_row_stride, n_rng, K, grad_w, s, &st))
         return st;
     const size_t bytes = sizeof(float2) * ((size_t)padded_len(n_az) + 64 + coarse_len(n_az));
+    const int rk = stored_radix(n_az, pl);
     static int done[3][kMaxDevices] = {};
     static const void *const ks[3] = {(const void *)xspec_taps_kernel<256>,
                                       (const void *)xspec_taps_kernel<512>, (const void *)xspec_taps_kernel<1024>};
     return launch_rows(
         n_az, n_rng, bytes,
-        [&](int gr, int t, size_t sm) { xspec_taps_kernel<256><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, grad_w); },
-        [&](int gr, int t, size_t sm) { xspec_taps_kernel<512><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, grad_w); },
-        [&](int gr, int t, size_t sm) { xspec_taps_kernel<1024><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, grad_w); },
+        [&](int gr, int t, size_t sm) { xspec_taps_kernel<256><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, rk, grad_w); },
+        [&](int gr, int t, size_t sm) { xspec_taps_kernel<512><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, rk, grad_w); },
+        [&](int gr, int t, size_t sm) { xspec_taps_kernel<1024><<<gr, t, sm, s>>>(P, o, o_row_stride, K, n_az, pl, rk, grad_w); },
         ks, done, "weight_grad_spectra");
 }
 

@@ -247,15 +247,6 @@ rosar_status launch_runtime(const MigCall &c, const RowPlan &pl, int T) {
     return launch_pair(c, azimuth_spectrum_kernel<MAXT, MINB>, azimuth_mig_combine_kernel<MAXT, MINB>, T, done, c.N, pl);
 }
 
-template <int N, int... R>
-bool plan_is(int n_az, const RowPlan &pl) {
-    constexpr int rad[] = {R...};
-    if (n_az != N || pl.pad_shift != 31 || pl.npass != (int)sizeof...(R)) return false;
-    for (int i = 0; i < pl.npass; ++i)
-        if (pl.rad[i] != rad[i]) return false;
-    return true;
-}
-
 constexpr int kFewRows = 304;      // as the row filter: up to two rows an SM a row's own latency counts
 
 }  // namespace
@@ -268,11 +259,11 @@ rosar_status launch_sparse_azimuth_migrating_fft(const float2 *S, int n_bins, co
                          n_az, AF_MAX_N);
     const MigCall c{S, Planes{X, H, n_bins, n_rng, d_lo, n_d}, X, out, n_az, s};
     const bool few = n_rng <= kFewRows;
-    if (plan_is<3600, 16, 15, 15>(n_az, pl)) return launch_fixed<256, 4, 3600, 16, 15, 15>(c);
-    if (plan_is<1800, 8, 15, 15>(n_az, pl))
+    if (Row3600::is(n_az, pl)) return launch_fixed<256, 4, 3600, 16, 15, 15>(c);
+    if (Row1800::is(n_az, pl))
         return few ? launch_fixed<256, 4, 1800, 8, 15, 15>(c) : launch_fixed<128, 8, 1800, 8, 15, 15>(c);
-    if (plan_is<7200, 8, 4, 15, 15>(n_az, pl)) return launch_fixed<256, 3, 7200, 8, 4, 15, 15>(c);
-    if (plan_is<360, 8, 3, 15>(n_az, pl)) return launch_fixed<128, 8, 360, 8, 3, 15>(c);
+    if (Row7200::is(n_az, pl)) return launch_fixed<256, 3, 7200, 8, 4, 15, 15>(c);
+    if (Row360::is(n_az, pl)) return launch_fixed<128, 8, 360, 8, 3, 15>(c);
     // 128 threads up to 2048: 480 x 256 9.7 us against 12.2 on 256, 1024 x 256 10.1 against 12.3, 1125 x 512 17.0 each.
     if (n_az <= 4096) return launch_runtime<256, 3>(c, pl, n_az <= 2048 ? 128 : 256);
     if (n_az <= 8192 && !few) return launch_runtime<256, 3>(c, pl, 256);

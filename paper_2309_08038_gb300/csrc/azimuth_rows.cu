@@ -181,14 +181,17 @@ rosar_status launch_runtime(const RowLaunch &l, const ROWS &rows, const RowPlan 
     return check_launch("azimuth_fft");
 }
 
-// Whether the run-time planner picks exactly these radices for n_az (H, made by the run-time plan, is in their order).
-template <int N, int... R>
-bool plan_is(int n_az, const RowPlan &pl) {
-    constexpr int rad[] = {R...};
-    if (n_az != N || pl.pad_shift != 31 || pl.npass != (int)sizeof...(R)) return false;
-    for (int i = 0; i < pl.npass; ++i)
-        if (pl.rad[i] != rad[i]) return false;
-    return true;
+// The run-time plan: the staged H row pays where a row's own latency counts.  Against loading the row, the passes,
+// the product and the store as steps of their own: 800 pulses, 256 rows 8.3 -> 7.1 us, 2048 rows 47 -> 22; 4500:
+// 23.9 -> 19.7 and 165 -> 89; 16384: 76 -> 51 (256 rows).
+template <typename ROWS>
+rosar_status launch_rows_runtime(const RowLaunch &l, const ROWS &rows, const RowPlan &pl, bool few) {
+    const Layout lay = layout_for(l.n_az, few);
+    if (l.n_az <= 4096) return launch_runtime<ROWS, 256, 3>(l, rows, pl, lay, !few && l.n_az <= 2048 ? 128 : 256);
+    if (l.n_az <= 8192 && !few) return launch_runtime<ROWS, 256, 3>(l, rows, pl, lay, 256);
+    // two rows an SM up to about 14200: 1024 rows of 9000 120 -> 92 us, of 12000 152 -> 121, of 13500 158 -> 156
+    if (!few && 2 * (lay.bytes + 1024) <= 228 * 1024) return launch_runtime<ROWS, 512, 2>(l, rows, pl, lay, 512);
+    return launch_runtime<ROWS, 512, 1>(l, rows, pl, lay, 512);
 }
 
 // Up to two rows an SM, a row's own latency counts: 256 threads and H staged while S is awaited.  With more the SM's
@@ -205,32 +208,23 @@ rosar_status launch_rows_of(const RowLaunch &l, const ROWS &rows) {
     if (!make_plan(l.n_az, &pl))
         return set_error(ROSAR_ERR_UNSUPPORTED, "azimuth_fft: n_az=%d is not 2^a 3^b 5^c in [2, %d]", l.n_az, AF_MAX_N);
     const bool few = l.n_rng <= kFewRows;
-    if (plan_is<3600, 16, 15, 15>(l.n_az, pl))
+    if (stored_radix(l.n_az, pl) == 0) return launch_rows_runtime<ROWS>(l, rows, pl, few);
+    if (Row3600::is(l.n_az, pl))
         return few ? launch_fixed<ROWS, 256, 2, 3600, kStaged, false, 16, 15, 15>(l, rows)
                    : launch_fixed<ROWS, 256, 4, 3600, kFused, false, 16, 15, 15>(l, rows);
-    if (plan_is<1800, 8, 15, 15>(l.n_az, pl))
+    if (Row1800::is(l.n_az, pl))
         return few ? launch_fixed<ROWS, 256, 2, 1800, kStaged, false, 8, 15, 15>(l, rows)
                    : launch_fixed<ROWS, 128, 8, 1800, kFused, false, 8, 15, 15>(l, rows);
-    if (plan_is<7200, 8, 4, 15, 15>(l.n_az, pl))
+    if (Row7200::is(l.n_az, pl))
         return l.n_rng <= 152 ? launch_fixed<ROWS, 512, 1, 7200, kStaged, false, 8, 4, 15, 15>(l, rows)
                               : launch_fixed<ROWS, 256, 3, 7200, kFused, true, 8, 4, 15, 15>(l, rows);
     // 14400: one row an SM on 1024 threads, or two on 512 each.  152 rows 15.8 us (17.0 streamed); 256 rows 32.8 -> 28.9,
     // 1024 rows 130 -> 115 (two rows an SM with the fused step 133, one with the streamed step 140).
-    if (plan_is<14400, 8, 8, 15, 15>(l.n_az, pl))
+    if (Row14400::is(l.n_az, pl))
         return l.n_rng <= 152 ? launch_fixed<ROWS, 1024, 1, 14400, kFused, false, 8, 8, 15, 15>(l, rows)
                               : launch_fixed<ROWS, 512, 2, 14400, kStreamed, false, 8, 8, 15, 15>(l, rows);
-    if (plan_is<360, 8, 3, 15>(l.n_az, pl))
-        return few ? launch_fixed<ROWS, 256, 2, 360, kStaged, false, 8, 3, 15>(l, rows)
-                   : launch_fixed<ROWS, 64, 8, 360, kFused, false, 8, 3, 15>(l, rows);
-    // The run-time plan: the staged H row pays where a row's own latency counts.  Against loading the row, the passes,
-    // the product and the store as steps of their own: 800 pulses, 256 rows 8.3 -> 7.1 us, 2048 rows 47 -> 22; 4500:
-    // 23.9 -> 19.7 and 165 -> 89; 16384: 76 -> 51 (256 rows).
-    const Layout lay = layout_for(l.n_az, few);
-    if (l.n_az <= 4096) return launch_runtime<ROWS, 256, 3>(l, rows, pl, lay, !few && l.n_az <= 2048 ? 128 : 256);
-    if (l.n_az <= 8192 && !few) return launch_runtime<ROWS, 256, 3>(l, rows, pl, lay, 256);
-    // two rows an SM up to about 14200: 1024 rows of 9000 120 -> 92 us, of 12000 152 -> 121, of 13500 158 -> 156
-    if (!few && 2 * (lay.bytes + 1024) <= 228 * 1024) return launch_runtime<ROWS, 512, 2>(l, rows, pl, lay, 512);
-    return launch_runtime<ROWS, 512, 1>(l, rows, pl, lay, 512);
+    return few ? launch_fixed<ROWS, 256, 2, 360, kStaged, false, 8, 3, 15>(l, rows)
+               : launch_fixed<ROWS, 64, 8, 360, kFused, false, 8, 3, 15>(l, rows);
 }
 
 }  // namespace
