@@ -133,12 +133,20 @@ def image_fft_host(raw_host, win, H, raw_dev, workspace, out_dev, out_host, stre
     return out_host
 
 
+def _empty(shape, dtype, device, stream):
+    """A tensor of one call on `stream`, from that stream's own memory: what the block held before was given back in that
+    stream's order, so the call's kernels overwrite nothing that another stream still uses, and once freed the block is
+    handed out again in the same order."""
+    if stream is None:
+        return torch.empty(shape, dtype=dtype, device=device)
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(stream.cuda_stream, device=device)
+    with torch.cuda.stream(stream):
+        return torch.empty(shape, dtype=dtype, device=device)
+
+
 def _scratch(nbytes, device, stream):
-    """Device scratch of one call: allocated on the current stream, kept until `stream` has passed the call."""
-    t = torch.empty(nbytes, dtype=torch.uint8, device=device)
-    if stream is not None:
-        t.record_stream(stream)
-    return t
+    return _empty(nbytes, torch.uint8, device, stream)
 
 
 def _up256(n):
@@ -156,7 +164,7 @@ def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None, transfo
     if win is not None:
         require(win, torch.float32, "win", shape=(L,))
     if out is None:
-        out = torch.empty((n_rng, n_az), dtype=torch.complex64, device=raw.device)
+        out = _empty((n_rng, n_az), torch.complex64, raw.device, stream)
     require(out, torch.complex64, "out", shape=(n_rng, n_az))
     st = radar.as_struct()
     nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 1, n_az, L, n_rng, M_ap) if transforms else 0
@@ -185,7 +193,7 @@ def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
     n_rng, K = w.shape
     stride = _offsets(o, n_rng, K)
     if out is None:
-        out = torch.empty((n_rng, n_az), dtype=torch.complex64, device=raw.device)
+        out = _empty((n_rng, n_az), torch.complex64, raw.device, stream)
     require(out, torch.complex64, "out", shape=(n_rng, n_az))
     st = radar.as_struct()
     nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, n_az, L, n_rng, K) if stride == 0 else 0
@@ -217,9 +225,9 @@ class TimeDomainPlan:
     K: int
 
 
-def _plan_tensor(n_rng, L, K, device):
-    nbytes = int(_lib.load().rosar_time_domain_plan_bytes(n_rng, L, K))
-    return torch.empty(nbytes, dtype=torch.uint8, device=device)
+def _plan_tensor(nbytes, n_rng, L, K, device, stream):
+    """nbytes, or 0 for the tensor-core plan's size."""
+    return _scratch(nbytes or int(_lib.load().rosar_time_domain_plan_bytes(n_rng, L, K)), device, stream)
 
 
 def sas_time_plan(win, w, o, radar: Radar, n_az, L, centred=True, stream=None):
@@ -232,7 +240,7 @@ def sas_time_plan(win, w, o, radar: Radar, n_az, L, centred=True, stream=None):
         require(win, torch.float32, "win", shape=(L,))
     st = radar.as_struct()
     nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, n_az, L, n_rng, K)
-    data = torch.empty(nbytes, dtype=torch.uint8, device=w.device) if nbytes else _plan_tensor(n_rng, L, K, w.device)
+    data = _plan_tensor(nbytes, n_rng, L, K, w.device, stream)
     make = lib.rosar_sas_time_fft_plan if nbytes else lib.rosar_sas_time_plan
     check(make(ptr(win), ptr(w), ptr(o), ctypes.byref(st), n_az, L, n_rng, K, 1 if centred else 0, ptr(data),
                data.numel(), stream_handle(stream)))
@@ -243,7 +251,7 @@ def _planned(raw, plan, bpa, direct, transforms, out, stream):
     lib = _lib.load()
     require(raw, torch.complex64, "raw", shape=(plan.n_az, plan.L))
     if out is None:
-        out = torch.empty((plan.n_rng, plan.n_az), dtype=torch.complex64, device=raw.device)
+        out = _empty((plan.n_rng, plan.n_az), torch.complex64, raw.device, stream)
     require(out, torch.complex64, "out", shape=(plan.n_rng, plan.n_az))
     sizes = (plan.n_az, plan.L, plan.n_rng, plan.K)
     if plan.data.numel() == lib.rosar_time_domain_plan_bytes(plan.n_rng, plan.L, plan.K):
@@ -271,7 +279,7 @@ def bpa_time_plan(win, radar: Radar, n_az, L, n_rng, M_ap, device=None, stream=N
     device = win.device if win is not None else (device or torch.device("cuda"))
     st = radar.as_struct()
     nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 1, n_az, L, n_rng, M_ap) if transforms else 0
-    data = torch.empty(nbytes, dtype=torch.uint8, device=device) if nbytes else _plan_tensor(n_rng, L, M_ap, device)
+    data = _plan_tensor(nbytes, n_rng, L, M_ap, device, stream)
     make = lib.rosar_bpa_time_fft_plan if nbytes else lib.rosar_bpa_time_plan
     check(make(ptr(win), ctypes.byref(st), n_az, L, n_rng, M_ap, ptr(data), data.numel(), stream_handle(stream)))
     return TimeDomainPlan(data, n_az, L, n_rng, M_ap)
