@@ -34,6 +34,7 @@
 // lr_inverse_* writes the NaNs.
 
 #include <math.h>
+#include <stddef.h>
 
 #include "row_fft.cuh"
 #include "time_domain_lr.cuh"
@@ -62,6 +63,15 @@ __device__ __forceinline__ float2 turns(double q) {
     float s, c;
     sincospif(2.f * (float)q, &s, &c);
     return make_float2(c, s);
+}
+
+// Planes of the plan, or 0 where it was not made for a call of this shape; after the grid-dependency wait, and not by the
+// non-coherent path (the kernel may overlap the one that writes the plan).
+__device__ __forceinline__ int plan_planes(const uint8_t *plan, const Shape &sh) {
+    const int4 a = __ldcg(reinterpret_cast<const int4 *>(plan)), b = __ldcg(reinterpret_cast<const int4 *>(plan) + 1);
+    static_assert(offsetof(Header, K) == 16 && offsetof(Header, planes) == 20 && sizeof(Header) == 32, "two vectors");
+    const bool same = a.x == lr::kPlanTag + sh.bpa && a.y == sh.n_az && a.z == sh.L && a.w == sh.n_rng && b.x == sh.K;
+    return same && b.y >= 0 && b.y <= MAX_PLANES ? b.y : 0;
 }
 
 __device__ __forceinline__ float cheb_node(int q, int P) { return cospif((float)(2 * q + 1) / (float)(2 * P)); }
@@ -115,7 +125,7 @@ lr_taps_kernel(const float *__restrict__ win, const float2 *__restrict__ w, cons
         row_q[tid] = (double)(((long long)l * (L - 1)) % (2LL * Lf)) / (2.0 * Lf);
         row_t[tid] = ((double)l + iv.mid) / iv.half;
     }
-    if (cta == 0 && tid == 32) *reinterpret_cast<Header *>(plan) = Header{P, sh.N};
+    if (cta == 0 && tid == 32) *reinterpret_cast<Header *>(plan) = Header{lr::kPlanTag + sh.bpa, n_az, L, sh.n_rng, K, P, {0, 0}};
     float2 *W = reinterpret_cast<float2 *>(plan + sh.w_at);
     const double inv_lf = 1.0 / Lf;               // exact: a power of two
     for (int i = cta * TAPS_THREADS + tid; i < P * Lf; i += gridDim.x * gridDim.y * TAPS_THREADS) {
@@ -165,7 +175,7 @@ template <typename FWD>
 __device__ __forceinline__ void lr_plan_row(const Shape &sh, uint8_t *plan, float2 *x, int x_len, int pad_shift, FWD fwd) {
     __shared__ float node[MAX_PLANES];
     griddep_wait();                           // the taps are complete
-    const int P = reinterpret_cast<const Header *>(plan)->planes;
+    const int P = plan_planes(plan, sh);
     if (threadIdx.x < P) node[threadIdx.x] = cheb_node(threadIdx.x, P);
     const float4 *taps = reinterpret_cast<const float4 *>(plan + sh.taps_at) + (size_t)blockIdx.x * sh.K;
     for (int q = blockIdx.y; q < P; q += gridDim.y) {
@@ -414,7 +424,7 @@ lr_combine_kernel(const float2 *__restrict__ X, const uint8_t *__restrict__ plan
     for (int i = threadIdx.x; i < 2 * C::HT; i += C::THREADS) hs[i] = make_float2(0.f, 0.f);
     __syncthreads();
     griddep_wait();
-    const int P = reinterpret_cast<const Header *>(plan)->planes;
+    const int P = plan_planes(plan, sh);
     const float2 *W = reinterpret_cast<const float2 *>(plan + sh.w_at);
     // H_q's tile: 16 bytes (two frequencies) a copy, 8 a thread; bins without a row stay zero
     int at[8];
@@ -432,7 +442,7 @@ lr_combine_kernel(const float2 *__restrict__ X, const uint8_t *__restrict__ plan
             if (at[i] >= 0) cp_async16(dst + 2 * i * C::THREADS, H + at[i]);
         cp_async_commit();
     };
-    stage(0);
+    if (P > 0) stage(0);
     float2 x[16], acc[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
@@ -484,6 +494,10 @@ lr_combine_kernel(const float2 *__restrict__ X, const uint8_t *__restrict__ plan
     }
 }
 
+__device__ __forceinline__ void fill_nan(float2 *__restrict__ out_row, int n) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out_row[i] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
+}
+
 // Whether any pulse is marked, and NaN for the pixels of a row whose aperture holds a marked pulse.
 __device__ __forceinline__ bool any_marked(const uint8_t *__restrict__ flags, const Shape &sh) {
     int any = 0;
@@ -513,6 +527,8 @@ lr_inverse_fixed_kernel(const float2 *__restrict__ Y, Shape sh, const uint8_t *_
     build_twiddles(N, false, sm + N, &tc, &tf);
     griddep_wait();
     const float2 *row = Y + (size_t)blockIdx.x * sh.pitch;
+    float2 *out_row = out + (size_t)blockIdx.x * sh.n_az;
+    if (plan_planes(plan, sh) == 0) return fill_nan(out_row, sh.n_az);
     const bool marked = any_marked(flags, sh);
 #pragma unroll 1
     for (int b = threadIdx.x; b < NB; b += T) {
@@ -528,7 +544,6 @@ lr_inverse_fixed_kernel(const float2 *__restrict__ Y, Shape sh, const uint8_t *_
     }
     __syncthreads();
     dit_middle<N, s1, T, WholeCta, Rs...>(sm, tc, tf);
-    float2 *out_row = out + (size_t)blockIdx.x * sh.n_az;
 #pragma unroll 1
     for (int j = threadIdx.x; j < s1; j += T) {
         float2 v[R1], wq[R1];
@@ -553,6 +568,8 @@ lr_inverse_runtime_kernel(const float2 *__restrict__ Y, Shape sh, RowPlan pl, co
     build_twiddles(sh.N, false, sm + padded_len(sh.N), &tc, &tf);
     griddep_wait();
     const float2 *row = Y + (size_t)blockIdx.x * sh.pitch;
+    float2 *out_row = out + (size_t)blockIdx.x * sh.n_az;
+    if (plan_planes(plan, sh) == 0) return fill_nan(out_row, sh.n_az);
     const bool marked = any_marked(flags, sh);
     for (int n = threadIdx.x; n < sh.N; n += T) {
         const float2 v = __ldcg(row + n);
@@ -560,7 +577,6 @@ lr_inverse_runtime_kernel(const float2 *__restrict__ Y, Shape sh, RowPlan pl, co
     }
     __syncthreads();
     row_dit(sm, sh.N, pl, tc, tf);
-    float2 *out_row = out + (size_t)blockIdx.x * sh.n_az;
     for (int n = threadIdx.x; n < sh.n_az; n += T) {
         const float2 v = sm[rpad(n, pl.pad_shift)];
         out_row[n] = make_float2(v.x, -v.y);
@@ -646,6 +662,7 @@ namespace lr {
 
 Shape shape_of(bool bpa, int n_az, int L, int n_rng, int K) {
     Shape sh = {};
+    sh.bpa = bpa ? 1 : 0;
     sh.n_az = n_az;
     sh.L = L;
     sh.n_rng = n_rng;

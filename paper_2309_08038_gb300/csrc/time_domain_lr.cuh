@@ -41,6 +41,7 @@ __host__ __device__ inline Interval residuals(float r0_over_dR, float s_max, int
 // Shape of one call; valid = 0 where the form does not apply.
 struct Shape {
     int valid;
+    int bpa;         // taps of back-projection, else of SAS
     int n_az, L, n_rng, K;
     int Lf;          // range transform length, a power of two >= L
     int N;           // azimuth transform length
@@ -56,9 +57,16 @@ struct Shape {
     size_t h_plane;  // bytes of one plane of H
 };
 
-struct Header {
-    int planes, N;
+// First bytes of a plan: what it was made for.  The kernels of an image call compare it with the call's own shape, on
+// which every address they form in the plan depends (a BPA plan's rows are padded otherwise than a SAS plan's): a plan
+// of another kind or size, or something else, is not read any further and gives an image of NaN.
+struct alignas(16) Header {
+    int kind;        // kPlanTag + bpa
+    int n_az, L, n_rng, K;
+    int planes;
+    int unused[2];
 };
+constexpr int kPlanTag = 0x6c725000;
 
 Shape shape_of(bool bpa, int n_az, int L, int n_rng, int K);
 // Planes a plan must have room for: one more than the host counts, whose float operations may round otherwise than

@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 from dataclasses import dataclass
+from typing import Optional
 
 import torch
 
@@ -223,6 +224,7 @@ class TimeDomainPlan:
     L: int
     n_rng: int
     K: int
+    bpa: Optional[bool] = None      # back-projection's or SAS's taps; None (built by hand): those of the call it is given to
 
 
 def _plan_tensor(nbytes, n_rng, L, K, device, stream):
@@ -244,20 +246,24 @@ def sas_time_plan(win, w, o, radar: Radar, n_az, L, centred=True, stream=None):
     make = lib.rosar_sas_time_fft_plan if nbytes else lib.rosar_sas_time_plan
     check(make(ptr(win), ptr(w), ptr(o), ctypes.byref(st), n_az, L, n_rng, K, 1 if centred else 0, ptr(data),
                data.numel(), stream_handle(stream)))
-    return TimeDomainPlan(data, n_az, L, n_rng, K)
+    return TimeDomainPlan(data, n_az, L, n_rng, K, False)
 
 
-def _planned(raw, plan, bpa, direct, transforms, out, stream):
+def _planned(raw, plan, bpa, out, stream):
+    """A plan of either kind holds its taps, and either call images with it (`bpa`: the call's kind, whose limits hold)."""
     lib = _lib.load()
     require(raw, torch.complex64, "raw", shape=(plan.n_az, plan.L))
     if out is None:
         out = _empty((plan.n_rng, plan.n_az), torch.complex64, raw.device, stream)
     require(out, torch.complex64, "out", shape=(plan.n_rng, plan.n_az))
     sizes = (plan.n_az, plan.L, plan.n_rng, plan.K)
-    if plan.data.numel() == lib.rosar_time_domain_plan_bytes(plan.n_rng, plan.L, plan.K):
+    if plan.data.numel() == lib.rosar_time_domain_plan_bytes(plan.n_rng, plan.L, plan.K) or (bpa and plan.K > plan.n_az):
+        direct = lib.rosar_bpa_time_planned if bpa else lib.rosar_sas_time_planned
         check(direct(ptr(raw), ptr(plan.data), *sizes, ptr(out), stream_handle(stream)))
     else:
-        ws = lib.rosar_time_domain_fft_workspace_bytes(bpa, *sizes)
+        kind = bpa if plan.bpa is None else plan.bpa
+        transforms = lib.rosar_bpa_time_fft if kind else lib.rosar_sas_time_fft
+        ws = lib.rosar_time_domain_fft_workspace_bytes(int(kind), *sizes)
         scratch = _scratch(ws, raw.device, stream)
         check(transforms(ptr(raw), ptr(plan.data), *sizes, ptr(scratch), ws, ptr(out), stream_handle(stream)))
     return out
@@ -266,8 +272,7 @@ def _planned(raw, plan, bpa, direct, transforms, out, stream):
 def sas_time_planned(raw, plan: TimeDomainPlan, out=None, stream=None):
     """rosar_sas_time_planned or rosar_sas_time_fft: rosar_sas_time of raw [n_az, L] with a plan from sas_time_plan
     (which holds the offsets)."""
-    lib = _lib.load()
-    return _planned(raw, plan, 0, lib.rosar_sas_time_planned, lib.rosar_sas_time_fft, out, stream)
+    return _planned(raw, plan, False, out, stream)
 
 
 def bpa_time_plan(win, radar: Radar, n_az, L, n_rng, M_ap, device=None, stream=None, transforms=False):
@@ -282,13 +287,12 @@ def bpa_time_plan(win, radar: Radar, n_az, L, n_rng, M_ap, device=None, stream=N
     data = _plan_tensor(nbytes, n_rng, L, M_ap, device, stream)
     make = lib.rosar_bpa_time_fft_plan if nbytes else lib.rosar_bpa_time_plan
     check(make(ptr(win), ctypes.byref(st), n_az, L, n_rng, M_ap, ptr(data), data.numel(), stream_handle(stream)))
-    return TimeDomainPlan(data, n_az, L, n_rng, M_ap)
+    return TimeDomainPlan(data, n_az, L, n_rng, M_ap, True)
 
 
 def bpa_time_planned(raw, plan: TimeDomainPlan, out=None, stream=None):
     """rosar_bpa_time_planned or rosar_bpa_time_fft: rosar_bpa_time of raw [n_az, L] with a plan from bpa_time_plan."""
-    lib = _lib.load()
-    return _planned(raw, plan, 1, lib.rosar_bpa_time_planned, lib.rosar_bpa_time_fft, out, stream)
+    return _planned(raw, plan, True, out, stream)
 
 
 def image(raw, win, w, o, workspace=None, out=None, stream=None):
