@@ -498,7 +498,8 @@ __device__ __forceinline__ void fill_nan(float2 *__restrict__ out_row, int n) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) out_row[i] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
 }
 
-// Whether any pulse is marked, and NaN for the pixels of a row whose aperture holds a marked pulse.
+// Whether any pulse is marked, and NaN for the pixels of a row whose aperture holds a marked pulse.  (The kernel overlaps
+// the one before it, so nothing that this call wrote is read by the non-coherent path.)
 __device__ __forceinline__ bool any_marked(const uint8_t *__restrict__ flags, const Shape &sh) {
     int any = 0;
     for (int n = threadIdx.x; n < sh.flag_bytes / 4; n += blockDim.x) any |= __ldcg(reinterpret_cast<const int *>(flags) + n);
@@ -511,7 +512,7 @@ __device__ __noinline__ void write_marked(const uint8_t *__restrict__ flags, con
         int hit = 0;
         for (int k = 0; k < sh.K && !hit; ++k) {
             const int n = pmod(th + __ldca(offs + k), sh.n_az);
-            for (int c = 0; c * TURN_SAMPLES < sh.L; ++c) hit |= flags[(size_t)c * sh.n_az + n];
+            for (int c = 0; c * TURN_SAMPLES < sh.L; ++c) hit |= __ldcg(flags + (size_t)c * sh.n_az + n);
         }
         if (hit) out_row[th] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
     }
