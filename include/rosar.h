@@ -121,6 +121,9 @@ ROSAR_API rosar_status rosar_sparse_azimuth(const rosar_c32 *S, const rosar_c32 
  * R_n = 0.  S(x, n) is linear interpolation between bins floor(x) and floor(x)+1
  * (interp = 1) or the nearest bin floor(x + 0.5) (interp = 0, the paper's l*_n of
  * Eq. (40)); bins outside 0..L-1 read zero.  S must be the centred range compression.
+ * With nominal positions most sizes are imaged row by row by transforms: a value of S that is not finite or above 1e30
+ * reaches the pixels that read it only; below that the float32 rounding (about 1e-7 of the rms of the rows read) lies in
+ * every pixel of the row.
  *   S           [L][n_az] complex                                         (in)
  *   radar       host pointer                                              (in)
  *   pulse_dphi  [n_az] float angle errors in radians, or NULL (all zero)  (in)
@@ -268,7 +271,9 @@ ROSAR_API rosar_status rosar_bpa_time_planned(const rosar_c32 *raw, const void *
  * float32 accuracy; the image is then P range transforms and one azimuth transform each way instead of K*L
  * multiply-adds a pixel.  Same sums as rosar_bpa_time / rosar_sas_time (shared offsets), closer to them than the
  * tensor-core forms (about 1e-6 relative L2 against 1e-5).  A pulse with a sample that is not finite makes the
- * pixels whose taps read it NaN, as there.
+ * pixels whose taps read it NaN, as there, and samples of 1e20 and more reach those pixels only.  Below that the
+ * float32 rounding of the transforms (about 1e-7 of the scan's rms) lies in every pixel: where one pulse is far above the
+ * rest, the pixels that do not read it lose the digits that it is above.
  *   rosar_time_domain_fft_plan_bytes: size of the plan (bpa = 1: rosar_bpa_time's taps, K = M_ap; 0: SAS), or 0
  *     where this form is not offered: sizes it does not exist for (n_rng > L, L > 2048, pulse counts without a long
  *     enough transform, an arm of very many range bins), sizes too small for it to pay, or invalid arguments.  Never

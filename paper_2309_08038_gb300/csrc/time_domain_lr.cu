@@ -29,9 +29,10 @@
 // and 95 (630).  Of the 48: turn 4, forward 6, combine 26, inverse 8, the rest hand-overs.  The relative L2 error is
 // 8e-7 where the bf16-split contraction has 1.5e-5.
 //
-// A pulse with a sample that is not finite makes every pixel whose aperture holds the pulse NaN, as in the direct
-// sums; a transform would spread it over the image, so lr_turn_kernel zeroes such samples and marks the pulse, and
-// lr_inverse_* writes the NaNs.
+// A transform would spread a sample that is not finite, or so large that its rounding is, over the image.  The direct
+// sums keep it to the pixels that read the pulse, and so does this: lr_turn_kernel zeroes such samples and marks their
+// pulse, and lr_inverse_* adds their terms to the pixels whose aperture holds it (NaN where one is not finite).  Smaller
+// samples go through the transforms: each leaves float32 rounding of its own size in every pixel.
 
 #include <math.h>
 #include <stddef.h>
@@ -125,7 +126,7 @@ lr_taps_kernel(const float *__restrict__ win, const float2 *__restrict__ w, cons
         row_q[tid] = (double)(((long long)l * (L - 1)) % (2LL * Lf)) / (2.0 * Lf);
         row_t[tid] = ((double)l + iv.mid) / iv.half;
     }
-    if (cta == 0 && tid == 32) *reinterpret_cast<Header *>(plan) = Header{lr::kPlanTag + sh.bpa, n_az, L, sh.n_rng, K, P, {0, 0}};
+    if (cta == 0 && tid == 32) *reinterpret_cast<Header *>(plan) = Header{lr::kPlanTag + sh.bpa, n_az, L, sh.n_rng, K, P, iv.half, 0};
     float2 *W = reinterpret_cast<float2 *>(plan + sh.w_at);
     const double inv_lf = 1.0 / Lf;               // exact: a power of two
     for (int i = cta * TAPS_THREADS + tid; i < P * Lf; i += gridDim.x * gridDim.y * TAPS_THREADS) {
@@ -248,10 +249,14 @@ lr_plan_runtime_kernel(Shape sh, RowPlan pl, uint8_t *__restrict__ plan) {
 
 // ---------------------------------------------------------------------------------------- per scan --
 
+// Samples up to this pass the transforms: sums of 16384 pulses, 2048 samples and the taps stay far inside float32.
+constexpr float kSpreadLimit = 1e20f;
+__device__ __forceinline__ bool passes(float2 v) { return fabsf(v.x) + fabsf(v.y) < kSpreadLimit; }   // false for NaN
+
 constexpr int TURN_PULSES = 16, TURN_SAMPLES = 64, TURN_THREADS = 256;
 
 // raw [n_az][L] -> turned [L][t_pitch], a tile of 16 pulses x 64 samples per CTA: rows of 64 samples in, runs of 16
-// pulses out.  A value that is not finite is stored as zero and marks its pulse, flags [sample tiles][n_az].
+// pulses out.  A value that may not pass is stored as zero and marks its pulse, flags [sample tiles][n_az].
 __global__ void __launch_bounds__(TURN_THREADS)
 lr_turn_kernel(const float2 *__restrict__ raw, Shape sh, int t_pitch, float2 *__restrict__ turned,
                uint8_t *__restrict__ flags) {
@@ -273,7 +278,7 @@ lr_turn_kernel(const float2 *__restrict__ raw, Shape sh, int t_pitch, float2 *__
 #pragma unroll
     for (int i = 0; i < IT; ++i) {
         const int e = threadIdx.x + i * TURN_THREADS, p = e / TURN_SAMPLES, m = e % TURN_SAMPLES;
-        if (!(isfinite(v[i].x) && isfinite(v[i].y))) {
+        if (!passes(v[i])) {
             bad[p] = 1;
             v[i] = make_float2(0.f, 0.f);
         }
@@ -498,30 +503,57 @@ __device__ __forceinline__ void fill_nan(float2 *__restrict__ out_row, int n) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) out_row[i] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
 }
 
-// Whether any pulse is marked, and NaN for the pixels of a row whose aperture holds a marked pulse.  (The kernel overlaps
-// the one before it, so nothing that this call wrote is read by the non-coherent path.)
+// Whether any pulse is marked, and the terms of the marked pulses' zeroed samples for the pixels of row r whose aperture
+// holds one: the tap's phasor is the first node's window turned by the tap's distance from that node.  (The kernel
+// overlaps the one before it, so nothing that this call wrote is read by the non-coherent path.)
 __device__ __forceinline__ bool any_marked(const uint8_t *__restrict__ flags, const Shape &sh) {
     int any = 0;
     for (int n = threadIdx.x; n < sh.flag_bytes / 4; n += blockDim.x) any |= __ldcg(reinterpret_cast<const int *>(flags) + n);
     return __syncthreads_or(any) != 0;
 }
-__device__ __noinline__ void write_marked(const uint8_t *__restrict__ flags, const int32_t *__restrict__ offs,
-                                          const Shape &sh, float2 *__restrict__ out_row) {
+__device__ __noinline__ void add_marked(const float2 *__restrict__ raw, const uint8_t *__restrict__ flags,
+                                        const uint8_t *__restrict__ plan, const Shape &sh, int r,
+                                        float2 *__restrict__ out_row) {
+    const float half = __ldcg(reinterpret_cast<const float *>(plan + offsetof(Header, half)));
+    const float node = cheb_node(0, plan_planes(plan, sh)), inv_lf = 1.f / (float)sh.Lf, mid = 0.5f * (float)(sh.L - 1);
+    const float2 *W = reinterpret_cast<const float2 *>(plan + sh.w_at);
+    const int32_t *offs = reinterpret_cast<const int32_t *>(plan + sh.offs_at);
+    const float4 *taps = reinterpret_cast<const float4 *>(plan + sh.taps_at) + (size_t)r * sh.K;
+    const int l = (int)((2LL * r * sh.Lf + sh.L) / (2LL * sh.L));
     __syncthreads();                          // after the row's own stores
     for (int th = threadIdx.x; th < sh.n_az; th += blockDim.x) {
-        int hit = 0;
-        for (int k = 0; k < sh.K && !hit; ++k) {
-            const int n = pmod(th + __ldca(offs + k), sh.n_az);
-            for (int c = 0; c * TURN_SAMPLES < sh.L; ++c) hit |= __ldcg(flags + (size_t)c * sh.n_az + n);
+        float2 add = make_float2(0.f, 0.f);
+        bool hit = false, finite = true;
+        for (int k = 0; k < sh.K; ++k) {
+            const int n = pmod(th + __ldcg(offs + k), sh.n_az);
+            for (int m0 = 0; m0 < sh.L; m0 += TURN_SAMPLES) {
+                if (!__ldcg(flags + (size_t)(m0 / TURN_SAMPLES) * sh.n_az + n)) continue;
+                hit = true;
+                const float4 t = __ldcg(taps + k);
+                const float per_m = half * (t.z - node) * inv_lf;
+                float2 sum = make_float2(0.f, 0.f);
+                for (int m = m0; m < min(m0 + TURN_SAMPLES, sh.L); ++m) {
+                    const float2 v = __ldcg(raw + (size_t)n * sh.L + m);
+                    if (passes(v)) continue;
+                    finite = finite && isfinite(v.x) && isfinite(v.y);
+                    float s, c;
+                    sincospif(2.f * fmaf(per_m, (float)m - mid, (float)((l * m) & (sh.Lf - 1)) * inv_lf), &s, &c);
+                    cmac(sum, cmul(__ldcg(W + m), make_float2(c, -s)), v);
+                }
+                cmac(add, make_float2(t.x * (float)sh.N, t.y * (float)sh.N), sum);
+            }
         }
-        if (hit) out_row[th] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
+        if (hit) {
+            const float nan = __int_as_float(0x7fc00000);
+            out_row[th] = finite ? cadd(out_row[th], add) : make_float2(nan, nan);
+        }
     }
 }
 
 template <int T, int N, int R1, int... Rs>
 __global__ void __launch_bounds__(T)
 lr_inverse_fixed_kernel(const float2 *__restrict__ Y, Shape sh, const uint8_t *__restrict__ plan,
-                        const uint8_t *__restrict__ flags, float2 *__restrict__ out) {
+                        const uint8_t *__restrict__ flags, const float2 *__restrict__ raw, float2 *__restrict__ out) {
     extern __shared__ float2 sm[];
     constexpr int s1 = N / R1, RK = last_radix<R1, Rs...>(), NB = N / RK;
     const float2 *tc, *tf;
@@ -557,13 +589,13 @@ lr_inverse_fixed_kernel(const float2 *__restrict__ Y, Shape sh, const uint8_t *_
         for (int i = 0; i < R1; ++i)
             if (j + i * s1 < sh.n_az) out_row[j + i * s1] = make_float2(v[i].x, -v[i].y);
     }
-    if (marked) write_marked(flags, reinterpret_cast<const int32_t *>(plan + sh.offs_at), sh, out_row);
+    if (marked) add_marked(raw, flags, plan, sh, blockIdx.x, out_row);
 }
 
 template <int T>
 __global__ void __launch_bounds__(T)
 lr_inverse_runtime_kernel(const float2 *__restrict__ Y, Shape sh, RowPlan pl, const uint8_t *__restrict__ plan,
-                          const uint8_t *__restrict__ flags, float2 *__restrict__ out) {
+                          const uint8_t *__restrict__ flags, const float2 *__restrict__ raw, float2 *__restrict__ out) {
     extern __shared__ float2 sm[];
     const float2 *tc, *tf;
     build_twiddles(sh.N, false, sm + padded_len(sh.N), &tc, &tf);
@@ -582,7 +614,7 @@ lr_inverse_runtime_kernel(const float2 *__restrict__ Y, Shape sh, RowPlan pl, co
         const float2 v = sm[rpad(n, pl.pad_shift)];
         out_row[n] = make_float2(v.x, -v.y);
     }
-    if (marked) write_marked(flags, reinterpret_cast<const int32_t *>(plan + sh.offs_at), sh, out_row);
+    if (marked) add_marked(raw, flags, plan, sh, blockIdx.x, out_row);
 }
 
 // -------------------------------------------------------------------------------------------- host --
@@ -816,14 +848,14 @@ rosar_status launch_time_domain_lr(const float2 *raw, int n_az, int L, int n_rng
         st = ensure_smem(f->inverse, smem, f->done[2], what);
         if (st != ROSAR_OK) return st;
         return go(what,
-                  reinterpret_cast<void (*)(const float2 *, Shape, const uint8_t *, const uint8_t *, float2 *)>(
+                  reinterpret_cast<void (*)(const float2 *, Shape, const uint8_t *, const uint8_t *, const float2 *, float2 *)>(
                       const_cast<void *>(f->inverse)),
-                  dim3(n_rng), T, smem, true, s, Y, sh, pb, flags, out);
+                  dim3(n_rng), T, smem, true, s, Y, sh, pb, flags, raw, out);
     }
     auto fn = T == 256 ? lr_inverse_runtime_kernel<256> : lr_inverse_runtime_kernel<512>;
     st = ensure_smem((const void *)fn, smem, done[2 + (T == 512)], what);
     if (st != ROSAR_OK) return st;
-    return go(what, fn, dim3(n_rng), T, smem, true, s, Y, sh, pl, pb, flags, out);
+    return go(what, fn, dim3(n_rng), T, smem, true, s, Y, sh, pl, pb, flags, raw, out);
 }
 
 }  // namespace rosar

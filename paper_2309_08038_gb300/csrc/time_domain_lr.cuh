@@ -64,7 +64,8 @@ struct alignas(16) Header {
     int kind;        // kPlanTag + bpa
     int n_az, L, n_rng, K;
     int planes;
-    int unused[2];
+    float half;      // of the interval of eta
+    int unused;
 };
 constexpr int kPlanTag = 0x6c725000;
 
