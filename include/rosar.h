@@ -277,7 +277,8 @@ ROSAR_API rosar_status rosar_bpa_time_planned(const rosar_c32 *raw, const void *
  *   rosar_time_domain_fft_plan_bytes: size of the plan (bpa = 1: rosar_bpa_time's taps, K = M_ap; 0: SAS), or 0
  *     where this form is not offered: sizes it does not exist for (n_rng > L, L > 2048, pulse counts without a long
  *     enough transform, an arm of very many range bins), sizes too small for it to pay, or invalid arguments.  Never
- *     equal to rosar_time_domain_plan_bytes.
+ *     equal to rosar_time_domain_plan_bytes.  P n_rng rows of the padded pulse count, 8 bytes a value: for SAS, whose
+ *     offsets may reach half a turn, P is near 30 for an arm of 4 bins (0.2 GB for 3600 x 256), so large scans take GBs.
  *   rosar_time_domain_fft_workspace_bytes: scratch of one image call.
  *   rosar_*_time_fft_plan: writes the plan (device, 256-byte aligned); arguments as rosar_*_time_plan.
  *   rosar_*_time_fft: the image from raw (as rosar_*_time_planned), the plan and a workspace (device, 256-byte

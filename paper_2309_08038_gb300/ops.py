@@ -154,6 +154,21 @@ def _up256(n):
     return (n + 255) & ~255
 
 
+# Scratch that sas_time may take for itself.  Its plan has planes for offsets up to half a turn, about 30 (n_rng, n_az)
+# planes at the arms and bins of these radars: 0.2 GB at 3600 x 256, 0.7 GB at 4501 x 320, 6.6 GB at 14400 x 2048.
+SCRATCH_LIMIT = 1 << 30
+
+
+def _optional_scratch(nbytes, device, stream):
+    """Scratch for a call that has another way: None above SCRATCH_LIMIT or where the device has no room for it."""
+    if nbytes > SCRATCH_LIMIT:
+        return None
+    try:
+        return _scratch(nbytes, device, stream)
+    except torch.cuda.OutOfMemoryError:
+        return None
+
+
 def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None, transforms=False):
     """rosar_bpa_time: time-domain back-projection (Eq. (14)) of the raw cube [n_az, L] onto rows 0..n_rng-1.
     transforms=True: by transforms (rosar_bpa_time_fft, plan and workspace allocated here) where the library offers that
@@ -184,7 +199,8 @@ def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None, transfo
 
 def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
     """rosar_sas_time: time-domain sparse-aperture imaging (Algorithm 2) of the raw cube [n_az, L]; one output
-    row per row of w [n_rng, K].  Shared offsets by transforms (rosar_sas_time_fft) where the library offers that."""
+    row per row of w [n_rng, K].  Shared offsets by transforms (rosar_sas_time_fft) where the library offers that
+    and the plan and workspace, taken for the call, fit SCRATCH_LIMIT and the device."""
     lib = _lib.load()
     require(raw, torch.complex64, "raw", ndim=2)
     n_az, L = raw.shape
@@ -198,9 +214,11 @@ def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
     require(out, torch.complex64, "out", shape=(n_rng, n_az))
     st = radar.as_struct()
     nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, n_az, L, n_rng, K) if stride == 0 else 0
+    scratch = None
     if nbytes and raw.data_ptr() % 16 == 0:
         at, ws = _up256(nbytes), lib.rosar_time_domain_fft_workspace_bytes(0, n_az, L, n_rng, K)
-        scratch = _scratch(at + ws, raw.device, stream)
+        scratch = _optional_scratch(at + ws, raw.device, stream)
+    if scratch is not None:
         h = stream_handle(stream)
         check(lib.rosar_sas_time_fft_plan(ptr(win), ptr(w), ptr(o), ctypes.byref(st), n_az, L, n_rng, K,
                                           1 if centred else 0, scratch.data_ptr(), nbytes, h))
@@ -233,7 +251,8 @@ def _plan_tensor(nbytes, n_rng, L, K, device, stream):
 
 
 def sas_time_plan(win, w, o, radar: Radar, n_az, L, centred=True, stream=None):
-    """rosar_sas_time_plan or rosar_sas_time_fft_plan for the weights w [n_rng, K] and shared offsets o [K]."""
+    """rosar_sas_time_fft_plan, where the library offers that form and the device has room for its plan (about 240 bytes a
+    pixel, see SCRATCH_LIMIT), else rosar_sas_time_plan, for the weights w [n_rng, K] and shared offsets o [K]."""
     lib = _lib.load()
     require(w, torch.complex64, "w", ndim=2)
     n_rng, K = w.shape
@@ -242,7 +261,13 @@ def sas_time_plan(win, w, o, radar: Radar, n_az, L, centred=True, stream=None):
         require(win, torch.float32, "win", shape=(L,))
     st = radar.as_struct()
     nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, n_az, L, n_rng, K)
-    data = _plan_tensor(nbytes, n_rng, L, K, w.device, stream)
+    try:
+        data = _plan_tensor(nbytes, n_rng, L, K, w.device, stream)
+    except torch.cuda.OutOfMemoryError:
+        if not nbytes:
+            raise
+        nbytes = 0
+        data = _plan_tensor(0, n_rng, L, K, w.device, stream)
     make = lib.rosar_sas_time_fft_plan if nbytes else lib.rosar_sas_time_plan
     check(make(ptr(win), ptr(w), ptr(o), ctypes.byref(st), n_az, L, n_rng, K, 1 if centred else 0, ptr(data),
                data.numel(), stream_handle(stream)))
