@@ -282,7 +282,8 @@ ROSAR_API rosar_status rosar_bpa_time_planned(const rosar_c32 *raw, const void *
  *   rosar_time_domain_fft_workspace_bytes: scratch of one image call.
  *   rosar_*_time_fft_plan: writes the plan (device, 256-byte aligned); arguments as rosar_*_time_plan.
  *   rosar_*_time_fft: the image from raw (as rosar_*_time_planned), the plan and a workspace (device, 256-byte
- *     aligned, one per call in flight).  The plan states what it was made for: one of the other kind (BPA or SAS), of
+ *     aligned, one per call in flight).  out and workspace must not overlap the plan (checked up to its second plane; it
+ *     has as many as its size says).  The plan states what it was made for: one of the other kind (BPA or SAS), of
  *     other sizes or not written by rosar_*_time_fft_plan is read no further than its first 32 bytes, and the image is NaN.
  */
 ROSAR_API size_t rosar_time_domain_fft_plan_bytes(const rosar_radar *radar, int bpa, int n_az, int L, int n_rng, int K);

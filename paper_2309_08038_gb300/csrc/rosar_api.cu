@@ -377,9 +377,9 @@ rosar_status fft_plan(const char *what, const float *win, const float2 *w, const
 rosar_status fft_image(const char *what, const rosar_c32 *raw, const void *plan, int bpa, int n_az, int L, int n_rng,
                        int K, void *workspace, size_t workspace_bytes, rosar_c32 *out, void *stream) {
     TdParams p;
-    // how many planes the plan holds is known to the device alone: at least two
-    const size_t plane = sizeof(rosar_c32) * (size_t)n_rng * n_az;
-    rosar_status st = planned_params(what, raw, plan, n_rng > 0 && n_az > 0 ? 2 * plane : 1, n_az, L, n_rng, K, out, &p);
+    // how many planes the plan holds is known to the device alone
+    const size_t part = time_domain_lr_plan_least(bpa == 1, n_az, L, n_rng, K);
+    rosar_status st = planned_params(what, raw, plan, part ? part : 1, n_az, L, n_rng, K, out, &p);
     if (st != ROSAR_OK) return st;
     if (!workspace) return set_error(ROSAR_ERR_INVALID_ARG, "%s: null workspace", what);
     const size_t need = time_domain_lr_workspace(bpa == 1, n_az, L, n_rng, K);
@@ -392,7 +392,7 @@ rosar_status fft_image(const char *what, const rosar_c32 *raw, const void *plan,
         return set_error(ROSAR_ERR_INVALID_ARG, "%s: plan and workspace must be 256-byte aligned", what);
     const size_t ob = sizeof(rosar_c32) * (size_t)n_rng * n_az;
     if (overlaps(workspace, need, raw, sizeof(rosar_c32) * (size_t)n_az * L) || overlaps(workspace, need, out, ob) ||
-        overlaps(workspace, need, plan, 2 * plane))
+        overlaps(workspace, need, plan, part))
         return set_error(ROSAR_ERR_INVALID_ARG, "%s: workspace overlaps another argument", what);
     return launch_time_domain_lr(reinterpret_cast<const float2 *>(raw), n_az, L, n_rng, K, bpa == 1, plan, workspace,
                                  reinterpret_cast<float2 *>(out), static_cast<cudaStream_t>(stream));

@@ -771,6 +771,11 @@ size_t time_domain_lr_workspace(bool bpa, int n_az, int L, int n_rng, int K) {
     return sh.valid ? sh.ws_bytes : 0;
 }
 
+size_t time_domain_lr_plan_least(bool bpa, int n_az, int L, int n_rng, int K) {
+    const Shape sh = lr::shape_of(bpa, n_az, L, n_rng, K);
+    return sh.valid ? sh.h_at + 2 * sh.h_plane : 0;      // two planes at least (planes_for)
+}
+
 rosar_status launch_time_domain_lr_plan(const float *win, const float2 *w, const int32_t *o, const TdParams &p, int K,
                                         bool bpa, void *plan, cudaStream_t s) {
     const char *what = bpa ? "bpa_time_plan" : "sas_time_plan";

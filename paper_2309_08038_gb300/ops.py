@@ -154,6 +154,14 @@ def _up256(n):
     return (n + 255) & ~255
 
 
+def _overlaps(a, *others):
+    """Whether the contiguous tensor a shares memory with any of the others."""
+    def span(t):
+        return t.data_ptr(), t.data_ptr() + t.numel() * t.element_size()
+    lo, hi = span(a)
+    return any(lo < e and b < hi for b, e in map(span, others))
+
+
 # Scratch that sas_time may take for itself.  Its plan has planes for offsets up to half a turn, about 30 (n_rng, n_az)
 # planes at the arms and bins of these radars: 0.2 GB at 3600 x 256, 0.7 GB at 4501 x 320, 6.6 GB at 14400 x 2048.
 SCRATCH_LIMIT = 1 << 30
@@ -215,7 +223,7 @@ def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
     st = radar.as_struct()
     nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, n_az, L, n_rng, K) if stride == 0 else 0
     scratch = None
-    if nbytes and raw.data_ptr() % 16 == 0:
+    if nbytes and raw.data_ptr() % 16 == 0 and not _overlaps(out, w, o):      # the direct call says what it refuses
         at, ws = _up256(nbytes), lib.rosar_time_domain_fft_workspace_bytes(0, n_az, L, n_rng, K)
         scratch = _optional_scratch(at + ws, raw.device, stream)
     if scratch is not None:
@@ -286,6 +294,8 @@ def _planned(raw, plan, bpa, out, stream):
         direct = lib.rosar_bpa_time_planned if bpa else lib.rosar_sas_time_planned
         check(direct(ptr(raw), ptr(plan.data), *sizes, ptr(out), stream_handle(stream)))
     else:
+        if _overlaps(out, plan.data):
+            raise _lib.RosarError(1, "ROSAR_ERR_INVALID_ARG", "time-domain call with a plan: out overlaps the plan")
         kind = bpa if plan.bpa is None else plan.bpa
         transforms = lib.rosar_bpa_time_fft if kind else lib.rosar_sas_time_fft
         ws = lib.rosar_time_domain_fft_workspace_bytes(int(kind), *sizes)
