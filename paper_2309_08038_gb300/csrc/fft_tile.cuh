@@ -319,13 +319,11 @@ __device__ __forceinline__ void range_adjoint_tile(const float2 *__restrict__ g,
 #pragma unroll
     for (int r = 0; r < RM; ++r) v[r].y = -v[r].y;
     if (centred) {
-        // c_l = (-1)^l exp(-j*pi*l/L), l = t + r*T (T even: one sign a thread; T = 1: r's)
-        float2 sp[RM];
-        twiddle_powers<RM>(half_twiddle(tab, T), sp);
-        const float2 ct = half_twiddle(tab, t);
+        // c_l = (-1)^l exp(-j*pi*l/L), l = t + r*T, each from the table: powers of exp(-j*pi*T/L) would multiply that
+        // entry's rounding (2.5e-7 rms of the gradient against 4e-8)
 #pragma unroll
         for (int r = 0; r < RM; ++r) {
-            const float2 c = r == 0 ? ct : cmul(ct, sp[r]);
+            const float2 c = half_twiddle(tab, t + r * T);
             v[r] = cmul(v[r], ((t + r * T) & 1) ? make_float2(-c.x, -c.y) : c);
         }
     }

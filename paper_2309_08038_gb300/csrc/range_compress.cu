@@ -62,8 +62,8 @@ rosar_status launch_group_L(const ScanGroup &g, int total, cudaStream_t s, bool 
 }
 
 // Pulses a CTA of the adjoint: 8 are a 64-byte segment of a bin's row, and 4 consecutive samples of a pulse's are a
-// sector.  Bound by memory: 16 scans of 3600 x 256 80 -> 53 us (of 35 at the copy rate), x 128 48 -> 27, 8 scans of
-// x 512 110 -> 65 (75 on two CTAs an SM), 4 of x 1024 103 -> 76 (93 on one), against bins staged pulse by pulse in shared memory
+// sector.  Bound by memory: 16 scans of 3600 x 256 82 -> 54.6 us (of 35 at the copy rate), x 128 49 -> 28.7, 8 scans of
+// x 512 109 -> 66 (75 on two CTAs an SM), 4 of x 1024 102 -> 73 (93 on one), against bins staged pulse by pulse in shared memory
 // before the first pass and after the last.
 template <int L>
 struct AdjointPlan : fft::Tile<L, (L <= 16 ? 32 : L <= 32 ? 16 : L <= 1024 ? 8 : L == 2048 ? 4 : 2)> {
