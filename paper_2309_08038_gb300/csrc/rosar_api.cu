@@ -5,6 +5,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include "raise_limit.cuh"
 #include "rosar_internal.cuh"
 
 namespace rosar {
@@ -32,14 +33,11 @@ rosar_status ensure_smem(const void *func, size_t bytes, int *limits, const char
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return set_error(ROSAR_ERR_CUDA, "%s: cudaGetDevice: %s", what, cudaGetErrorString(e));
     if (dev < 0 || dev >= kMaxDevices) return set_error(ROSAR_ERR_UNSUPPORTED, "%s: device ordinal %d", what, dev);
-    if ((size_t)__atomic_load_n(limits + dev, __ATOMIC_ACQUIRE) >= bytes) return ROSAR_OK;
-    e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    e = (cudaError_t)raise_limit(limits + dev, (int)bytes, [&](int n) {
+        return (int)cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    });
     if (e != cudaSuccess)
         return set_error(ROSAR_ERR_CUDA, "%s: cudaFuncSetAttribute(%zu B): %s", what, bytes, cudaGetErrorString(e));
-    int cur = __atomic_load_n(limits + dev, __ATOMIC_ACQUIRE);
-    while (cur < (int)bytes && !__atomic_compare_exchange_n(limits + dev, &cur, (int)bytes, false, __ATOMIC_ACQ_REL,
-                                                            __ATOMIC_ACQUIRE)) {
-    }
     return ROSAR_OK;
 }
 
