@@ -466,13 +466,15 @@ bpa_errors2_kernel(const float2 *__restrict__ S, BpaParams p, const float *__res
                 for (int b = 0; b < 2; ++b) {
                     const float Rb = b ? R.y : R.x, rhob = b ? rho.y : rho.x;
                     const float num = fmaf(4.f * Rb * pp.z, s2, drn * (pp.z + r0 - 2.f * Rb));
-                    const float Rn2 = fmaf(rhob, rhob, num);
+                    // not rho^2 + num: a pulse that passes close to the pixel would cancel them
+                    const float along = rhob - drn;                       // R - r_n
+                    const float Rn2 = fmaf(4.f * Rb * pp.z, s2, along * along);
                     // branch-free: R_n = 0 (the facing pulse of row 0, or a supplied position on the pixel) gives
                     // delta = num / rho = -rho exactly, or 0 when rho = 0 too, and alpha = 1 by the select
                     const float inv = rsqrtf(fmaxf(Rn2, 1e-30f));
                     const float Rn = Rn2 * inv;
                     const float delta = __fdividef(num, fmaxf(Rn + rhob, 1e-30f));
-                    const float a0 = __saturatef(fmaf(-2.f * Rb, s2, rhob - drn) * inv);
+                    const float a0 = __saturatef(fmaf(-2.f * Rb, s2, along) * inv);
                     const float alpha = Rn2 > 0.f ? a0 : 1.f;
                     const float x = fmaf(delta, p.inv_dR, (float)(r + b));
                     const float2 sv = sample_anywhere<LINEAR>(S, wsm + threadIdx.x + i, wc, wlo, wtop, x, L, n_az,
