@@ -14,7 +14,7 @@ from CUDA events on the launching stream; every step streams 3.9 GB of raw input
 of images (inputs far larger than the 129 MB L2).  Under torchrun every rank images its own copy of
 the batch (weak scaling, no data-path collective) and rank 0 prints the max-over-ranks time.
 Beside the headline: the same batch as 256 per-scan calls and through GPU back-projection, the
-indoor scan (pipelined multi-scan and per-scan paths), the paper's four methods on the indoor scan,
+indoor scan (multi-scan and per-scan calls), the paper's four methods on the indoor scan,
 the high-resolution scan, and the differentiable form (16 indoor scans, forward and backward).
 `--impl reference` times the FP64 CPU oracle on a bounded sample of the batched workload.
 """
@@ -38,7 +38,7 @@ sys.path.insert(0, ROOT)
 
 N_BUF = 16
 L2_BYTES = 129 * 1024 * 1024
-METRIC = "image px/s (batched: 256 uneven scans in one persistent graph-captured launch)"
+METRIC = "image px/s (batched: 256 uneven scans in one graph-captured launch)"
 WORKLOAD = ("batched: 256 scans, n_az in {1800, 3600, 7200}, L in {128, 256, 512, 1024}, K in {32, 64, 128} "
             "taps of M = n_az/6, per-scan offsets and default weights, 480,844,800 px, complex64")
 
@@ -58,7 +58,7 @@ def parse():
     ap.add_argument("--batch-scans", type=int, default=256, help="scans of the batched workload (a prefix of the 256)")
     ap.add_argument("--indoor-steps", type=int, default=2000, help="timed scans of the indoor section")
     ap.add_argument("--per-scan", action="store_true",
-                    help="indoor section: one rosar_image_fft call per scan instead of the pipelined call")
+                    help="indoor section: one rosar_image_fft call per scan instead of one rosar_image_fft_scans call")
     ap.add_argument("--kernel-cases", type=int, default=0, metavar="N",
                     help="profiling mode: run every profiled call twice on small cases (the indoor scan, a 16-scan "
                          "stack, the first N scans of the batched workload), print the launch order and exit")
@@ -856,7 +856,7 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
     torch.cuda.synchronize()
     t_plan = e0.elapsed_time(e1) * 1e-3
     choice = rosar.autotune.choose_azimuth(cfg.L, cfg.n_az, cfg.K)
-    pipelined = rosar.image_fft_scans_pipelined(cfg.L, cfg.n_az) and not args.per_scan
+    sequence = not args.per_scan
     steps = args.indoor_steps
 
     def image_step(b):
@@ -869,7 +869,7 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
         image_step(i % N_BUF)
     torch.cuda.synchronize()
     reps, rem = divmod(steps, N_BUF)
-    if pipelined:
+    if sequence:
         g_full = graph_of(torch, lambda i: scans_call(N_BUF), 1)
         g_rem = graph_of(torch, lambda i: scans_call(rem), 1) if rem else None
         ms, _ = time_loop(torch, lambda i: (g_full if i < reps else g_rem).replay(), reps + (1 if rem else 0), 2,
@@ -878,7 +878,7 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
         ms, _ = graph_loop(torch, lambda i: image_step(i % N_BUF), steps, 16, N_BUF, stream, world, device)
     value = world * px / (ms / steps * 1e-3)
     indoor_img = None
-    if pipelined:
+    if sequence:
         scans_call(N_BUF)
         indoor_img = out_stack[0].cpu().numpy()        # buffer 0 is the unrotated scan on rank 0
 
@@ -911,6 +911,7 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
     fp32_peak = sm_count * 128 * 2 * sm_mhz * 1e6 / 1e12
     sfu_peak = sm_count * 16 * sm_mhz * 1e6 / 1e12             # T SFU ops/s (16 per SM per clock)
     hbm = float(peaks["hbm_gbs"])
+    bf16_peak = float(peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops", 1700.0)))
     k1_bytes = 16.0 * px
     k2_bytes = 16.0 * px + 8.0 * cfg.L * K + 4.0 * K
     k2_flops = 8.0 * K * px
@@ -945,11 +946,11 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
     }
     res = {"workload": "indoor scan: 3600 pulses x 256 ADC samples, K=64 of M=600, 256x3600 polar image",
            "px_s": value, "ms_per_scan": ms / steps, "scans_timed": steps,
-           "timed_path": "rosar_image_fft_scans (16 scans per call, graph replays)" if pipelined else "rosar_image_fft",
+           "timed_path": "rosar_image_fft_scans (16 scans per call, graph replays)" if sequence else "rosar_image_fft",
            "autotune": choice, "kernels": kernels,
            "image_gather_px_s": world * px / t_gather_img, "image_migrating_px_s": world * px / t_mig_img,
            "image_migrating_fft_px_s": world * px / t_migf_img}
-    if pipelined:
+    if sequence:
         def call_ms(n, reps_=64):
             m_, _ = graph_loop(torch, lambda i: scans_call(n), reps_, 3, 1, stream, world, device)
             return m_ / reps_
@@ -1012,16 +1013,23 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
         e1.record(stream)
         torch.cuda.synchronize()
         t_bplan = e0.elapsed_time(e1) * 1e-3
-        plan_mb = (splan.data.numel() / 1e6, bplan.data.numel() / 1e6)
         ms_btp, _ = time_loop(torch, lambda i: rosar.bpa_time_planned(raws[i % N_BUF], bplan, out=bo), 3, 1,
                               stream, world, device)
-        t_stp, t_btp = ms_stp / 20 * 1e-3, ms_btp / 3 * 1e-3
-        del bplan
+        fplan = rosar.bpa_time_plan(win, radar, cfg.n_az, cfg.L, cfg.L, cfg.M_ap, transforms=True)
+        plan_mb = (splan.data.numel() / 1e6, bplan.data.numel() / 1e6, fplan.data.numel() / 1e6)
+        ms_btf, _ = time_loop(torch, lambda i: rosar.bpa_time_planned(raws[i % N_BUF], fplan, out=bo), 20, 2,
+                              stream, world, device)
+        t_stp, t_btp, t_btf = ms_stp / 20 * 1e-3, ms_btp / 3 * 1e-3, ms_btf / 20 * 1e-3
+        del bplan, fplan
         t_bj, t_bn = ms_bj / 20 * 1e-3, ms_bn / 20 * 1e-3
         t_bt, t_st = ms_bt / 3 * 1e-3, ms_st / 20 * 1e-3
 
         def frac16(t):
             return 16.0 * px / t / 1e9 / hbm
+
+        def tensor(t):                                         # of the split-bf16 contraction: three products a term
+            f = 8.0 * cfg.M_ap * cfg.L * px
+            return {"us_per_launch": t * 1e6, "tflops": f / t / 1e12, "tensor_frac": 3 * f / t / 1e12 / bf16_peak}
         pp = float(cfg.M_ap) * px                              # pixel-pulses of one BPA image
         res["compare"] = {
             "fft_bpa_px_s": world * px / (t_bj + t_k1), "fft_bpa_nominal_px_s": world * px / (t_bn + t_k1),
@@ -1037,16 +1045,21 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
                         "lanes x 2 flop, SFU 152 SMs x 16 ops per clock; nominal: per range row circular correlations "
                         "in the azimuth-frequency domain (S in, image out: 16 B/px)",
             "bpa_time_px_s": world * px / t_bt, "sas_time_px_s": world * px / t_st,
-            "time-domain BPA": {"us_per_call": t_bt * 1e6, "hbm_frac_16B_per_px": frac16(t_bt)},
+            "td_tcg_kernel<BPA>": dict(tensor(t_bt), traffic=recorded_traffic("td_tcg_kernel<1>", "indoor",
+                                                                              source_hash("time_domain.cu"))),
             "time-domain SAS": {"us_per_call": t_st * 1e6, "hbm_frac_16B_per_px": frac16(t_st)},
             "planned": {
                 "time-domain SAS": {"us_per_call": t_stp * 1e6, "hbm_frac_16B_per_px": frac16(t_stp),
                                     "plan_us_once": t_splan * 1e6, "plan_MB": plan_mb[0]},
-                "time-domain BPA": {"us_per_call": t_btp * 1e6, "hbm_frac_16B_per_px": frac16(t_btp),
-                                    "plan_us_once": t_bplan * 1e6, "plan_MB": plan_mb[1]},
-                "note": "azimuth transforms of the taps' low-rank planes computed once per weight design; per scan the "
-                        "pulses are transformed, combined with the planes and transformed back; plan_us_once is one "
-                        "plan build (the paper's W_BP / W_SA, computed per image there)"},
+                "td_tcw_kernel<BPA>": dict(tensor(t_btp), plan_us_once=t_bplan * 1e6, plan_MB=plan_mb[1],
+                                           traffic=recorded_traffic("td_tcw_kernel<1>", "indoor",
+                                                                    source_hash("time_domain.cu"))),
+                "time-domain BPA by transforms (on request)": {"us_per_call": t_btf * 1e6,
+                                                               "hbm_frac_16B_per_px": frac16(t_btf), "plan_MB": plan_mb[2]},
+                "note": "SAS: azimuth transforms of the taps' low-rank planes computed once per weight design; per scan the "
+                        "pulses are transformed, combined with the planes and transformed back; BPA: the B operand of the "
+                        "tensor-core contraction computed once; plan_us_once is one plan build (the paper's W_BP / W_SA, "
+                        "computed per image there)"},
             "paper_table_ms_per_image": {"BPA": t_bt * 1e3, "SAS": t_st * 1e3,
                                          "BPA (plan built per image)": (t_bplan + t_btp) * 1e3,
                                          "SAS (plan built per image)": (t_splan + t_stp) * 1e3,
@@ -1054,7 +1067,8 @@ def indoor_section(torch, rosar, args, device, rank, world, stream, peaks, peak_
                                          "FFT+SAS": ms / steps, "FFT+SAS (per-pulse peak bins)": t_migf_img * 1e3},
             "note": "FFT+BPA = range compression + back-projection over M=600 pulses (nominal geometry; the "
                     "supplied-error variant is timed beside it); BPA / SAS = time-domain forms (Eq. (14); "
-                    "Algorithm 2 with W_SA) evaluated by transforms, the plan built within the call, and with a kept plan; "
+                    "Algorithm 2 with W_SA), SAS by transforms, BPA on the tensor cores (tensor_frac of the measured sustained "
+                    "bf16 peak), the plan built within the call, and with a kept plan; "
                     "FFT+SAS = the timed indoor path"}
         res["highres"] = highres_bench(torch, rosar, device, world, hbm)
     return res, indoor_img, (cfg, sc, w, o, win)
@@ -1325,6 +1339,7 @@ def kernel_cases(args):
     ref = torch.randn_like(stack)
     splan = rosar.sas_time_plan(win, w, o, radar, cfg.n_az, cfg.L)
     bplan = rosar.bpa_time_plan(win, radar, cfg.n_az, cfg.L, cfg.L, cfg.M_ap)
+    fplan = rosar.bpa_time_plan(win, radar, cfg.n_az, cfg.L, cfg.L, cfg.M_ap, transforms=True)
     wl = BatchedWorkload(torch, rosar, device, args.kernel_cases)
     b = rosar.Batch(wl.scans, rosar.batch.Tuning())
     ws2 = torch.empty((2, cfg.L, cfg.n_az), dtype=torch.complex64, device=device)
@@ -1346,6 +1361,7 @@ def kernel_cases(args):
         ("time-domain BPA (unplanned call)", lambda: rosar.bpa_time(raws[0], win, radar, cfg.L, cfg.M_ap)),
         ("time-domain SAS (unplanned call)", lambda: rosar.sas_time(raws[0], win, w, o, radar)),
         ("time-domain BPA (planned)", lambda: rosar.bpa_time_planned(raws[0], bplan)),
+        ("time-domain BPA (planned, transforms)", lambda: rosar.bpa_time_planned(raws[0], fplan)),
         ("time-domain SAS (planned)", lambda: rosar.sas_time_planned(raws[0], splan)),
     ]
     for _ in range(2):
