@@ -23,22 +23,22 @@ namespace {
 
 // Pulses per CTA for the standalone kernel: small tiles give enough CTAs to cover
 // the memory latency at the scan sizes of interest.  L = 1024 takes 8 pulses (stores of 64 bytes instead of 32) on 512
-// threads at 64 registers, two CTAs an SM: 14400 pulses 65.6 -> 55.6 us (one CTA an SM at 95 registers: 77).
-template <int L>
-struct Plan : fft::Tile<L, (L <= 16 ? 32 : L <= 64 ? 16 : L <= 256 ? 8 : L == 512 ? 4 : L == 1024 ? 8 : 2)> {
+// threads at 64 registers, two CTAs an SM: 14400 pulses 55.0 -> 52.2 us, or HALF of them (half_tiles below).
+template <int L, bool HALF = false>
+struct Plan : fft::Tile<L, (L <= 16 ? 32 : L <= 64 ? 16 : L <= 256 ? 8 : L == 512 || (L == 1024 && HALF) ? 4 : L == 1024 ? 8 : 2)> {
     // 0: none asked for.  A minimum of one lets the compiler spend 98 registers on L = 256 where it takes 80: 16 scans of
     // 3600 pulses 39.8 -> 45.7 us.
-    static constexpr int MINB = L == 1024 ? 2 : 0;
+    static constexpr int MINB = L == 1024 && !HALF ? 2 : 0;
 };
 
-template <int L>
-__global__ void __launch_bounds__(Plan<L>::THREADS, Plan<L>::MINB)
+template <int L, bool HALF>
+__global__ void __launch_bounds__(Plan<L, HALF>::THREADS, Plan<L, HALF>::MINB)
 range_compress_kernel(const float2 *__restrict__ raw, const float *__restrict__ win, int n_az, int centred,
                       float2 *__restrict__ S, int vec_store) {
     extern __shared__ float2 smem[];
     const size_t scan = (size_t)blockIdx.y * n_az * L;      // grid.y: scans of a stack
-    fft::range_tile<L, Plan<L>::P>(raw + scan, win, n_az, centred != 0, S + scan, blockIdx.x * Plan<L>::P, smem, true,
-                                   vec_store != 0);
+    constexpr int P = Plan<L, HALF>::P;
+    fft::range_tile<L, P>(raw + scan, win, n_az, centred != 0, S + scan, blockIdx.x * P, smem, true, vec_store != 0);
 }
 
 // The same over the scans of a batch that have this length.
@@ -61,18 +61,18 @@ rosar_status launch_group_L(const ScanGroup &g, int total, cudaStream_t s, bool 
     return check_launch("batch range compression");
 }
 
-// Pulses a CTA of the adjoint: 8 are a 64-byte segment of a bin's row, and 4 consecutive samples of a pulse's are a
-// sector.  Bound by memory: 16 scans of 3600 x 256 82 -> 54.6 us (of 35 at the copy rate), x 128 49 -> 28.7, 8 scans of
-// x 512 109 -> 66 (75 on two CTAs an SM), 4 of x 1024 102 -> 73 (93 on one), against bins staged pulse by pulse in shared memory
+// Pulses a CTA of the adjoint: 8 are a 64-byte segment of a bin's row (from L = 1024 on 4 run faster), and 4 consecutive
+// samples of a pulse's are a sector.  Bound by memory: 16 scans of 3600 x 256 82 -> 54.6 us (of 35 at the copy rate), x 128 49 -> 28.7, 8 scans of
+// x 512 109 -> 66 (75 on two CTAs an SM), 14400 x 1024 102 -> 63 (72 with 8 pulses a CTA), against bins staged pulse by pulse in shared memory
 // before the first pass and after the last.
 template <int L>
-struct AdjointPlan : fft::Tile<L, (L <= 16 ? 32 : L <= 32 ? 16 : L <= 1024 ? 8 : L == 2048 ? 4 : 2)> {
-    using Base = fft::Tile<L, (L <= 16 ? 32 : L <= 32 ? 16 : L <= 1024 ? 8 : L == 2048 ? 4 : 2)>;
+struct AdjointPlan : fft::Tile<L, (L <= 16 ? 32 : L <= 32 ? 16 : L <= 512 ? 8 : L <= 2048 ? 4 : 2)> {
+    using Base = fft::Tile<L, (L <= 16 ? 32 : L <= 32 ? 16 : L <= 512 ? 8 : L <= 2048 ? 4 : 2)>;
     static constexpr size_t SMEM = sizeof(float2) * (size_t)(Base::TAB + Base::P * Base::LP);
 };
 
 template <int L>
-__global__ void __launch_bounds__(AdjointPlan<L>::THREADS, L == 1024 ? 2 : L == 512 ? 3 : 0)
+__global__ void __launch_bounds__(AdjointPlan<L>::THREADS, L == 512 ? 3 : 0)
 range_adjoint_kernel(const float2 *__restrict__ g, const float *__restrict__ win, int n_az, int centred,
                      float2 *__restrict__ grad_raw) {
     extern __shared__ float2 smem[];
@@ -96,20 +96,37 @@ rosar_status launch_adjoint_L(const float2 *g, const float *win, int n_az, int c
     return check_launch("range_compress_adjoint");
 }
 
-template <int L>
-rosar_status launch_L(const float2 *raw, const float *win, int n_az, int centred, float2 *S, cudaStream_t s,
-                      int n_scans) {
-    using PL = Plan<L>;
+template <int L, bool HALF>
+rosar_status launch_plan(const float2 *raw, const float *win, int n_az, int centred, float2 *S, cudaStream_t s,
+                         int n_scans, bool vec) {
+    using PL = Plan<L, HALF>;
     static_assert(PL::SMEM <= 227 * 1024, "range-compress tile exceeds shared memory");
     if (PL::SMEM > 48 * 1024) {
         static int done[kMaxDevices] = {};
-        rosar_status st = ensure_smem((const void *)range_compress_kernel<L>, PL::SMEM, done, "range_compress");
+        rosar_status st = ensure_smem((const void *)range_compress_kernel<L, HALF>, PL::SMEM, done, "range_compress");
         if (st != ROSAR_OK) return st;
     }
     const dim3 grid((n_az + PL::P - 1) / PL::P, n_scans);
-    const int vec = ((n_az % 2) == 0) && ((reinterpret_cast<uintptr_t>(S) & 15) == 0);
-    range_compress_kernel<L><<<grid, PL::THREADS, PL::SMEM, s>>>(raw, win, n_az, centred, S, vec);
+    range_compress_kernel<L, HALF><<<grid, PL::THREADS, PL::SMEM, s>>>(raw, win, n_az, centred, S, vec ? 1 : 0);
     return check_launch("range_compress");
+}
+
+// L = 1024: tiles of 4 pulses instead of 8 where the fullest SM would hold half of a last tile of 8 (an odd number of
+// tiles of 4 on it), and for rows of an odd stride, whose stores are single: 360 pulses 5.7 against 4.1 us, 1000 6.0 and
+// 6.0, 1800 8.9 and 7.7, 2000 9.3 and 10.3, 2800 13.2 and 12.6, 3600 13.5 and 14.7, 7200 28.0 and 29.3; 1501 9.5 and 7.5,
+// 3607 13.9 and 13.3, 10001 38.8 and 38.5.
+bool half_tiles(int n_az, int n_scans, bool vec) {
+    const long long tiles = (long long)n_scans * ((n_az + 3) / 4);
+    return !vec || ((tiles + 151) / 152) % 2 == 1;
+}
+
+template <int L>
+rosar_status launch_L(const float2 *raw, const float *win, int n_az, int centred, float2 *S, cudaStream_t s,
+                      int n_scans) {
+    const bool vec = n_az % 2 == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0;
+    if constexpr (L == 1024)
+        if (half_tiles(n_az, n_scans, vec)) return launch_plan<L, true>(raw, win, n_az, centred, S, s, n_scans, vec);
+    return launch_plan<L, false>(raw, win, n_az, centred, S, s, n_scans, vec);
 }
 
 }  // namespace
