@@ -29,6 +29,8 @@
 // Grid: (azimuth tiles of 256 pixels, rows).  Once S is staged in shared memory the nominal kernel is bound by
 // shared-memory bandwidth (two 8-byte window reads per sample) and the supplied-error kernel by FP32 + SFU issue.
 
+#include <type_traits>
+
 #include "bpa_geometry.cuh"
 
 namespace rosar {
@@ -168,7 +170,7 @@ bpa_kernel(const float2 *__restrict__ S, BpaParams p, const float *__restrict__ 
         __syncthreads();
         if (th >= n_az) continue;
         // bin x and weight alpha * exp(-j*2*pi*(2 f/c)*delta) of offset dc + i for this thread's pixel
-        auto sample = [&](int i, float &x, float2 &a) {
+        auto sample = [&](int i, auto checked, float &x, float2 &a) {
             const float4 t = dtab[i];
             if (NOMINAL) {
                 x = t.x;
@@ -178,14 +180,16 @@ bpa_kernel(const float2 *__restrict__ S, BpaParams p, const float *__restrict__ 
                 const float sh = fmaf(t.x, pp.x, t.y * pp.y);            // sin((pi*d/n_az) + eps/2)
                 const float s2 = sh * sh;
                 const float num = fmaf(pp.w, s2, pp.z);                  // R_n^2 - rho^2
-                const float Rn2 = fmaf(rho, rho, num);
+                const float along = pal[threadIdx.x + i];                // R - r_n
+                // off the window a pulse may pass close to the pixel, where rho^2 + num would cancel
+                const float Rn2 = decltype(checked)::value ? fmaf(pp.w, s2, along * along) : fmaf(rho, rho, num);
                 // branch-free: R_n = 0 (the facing pulse of row 0, or a supplied position on the pixel) gives
                 // delta = num / rho = -rho exactly, or 0 when rho = 0 too, and alpha = 1 by the select
                 const float inv = rsqrtf(fmaxf(Rn2, 1e-30f));
                 const float Rn = Rn2 * inv;
                 const float delta = __fdividef(num, fmaxf(Rn + rho, 1e-30f));
                 // alpha = max(0, cos(theta')), cos(theta') <= 1: one saturating multiply
-                const float a0 = __saturatef(fmaf(-2.f * R, s2, pal[threadIdx.x + i]) * inv);
+                const float a0 = __saturatef(fmaf(-2.f * R, s2, along) * inv);
                 const float alpha = Rn2 > 0.f ? a0 : 1.f;
                 x = fmaf(delta, p.inv_dR, rf);
                 a = cscale(expmj2pi_turns(p.two_f_over_c * delta), alpha);
@@ -198,7 +202,7 @@ bpa_kernel(const float2 *__restrict__ S, BpaParams p, const float *__restrict__ 
             for (int i = 0; i < nd; ++i) {
                 float x;
                 float2 a;
-                sample(i, x, a);
+                sample(i, std::false_type{}, x, a);
                 float2 sv;
                 if (LINEAR) {
                     const float fl = floorf(x);
@@ -216,7 +220,7 @@ bpa_kernel(const float2 *__restrict__ S, BpaParams p, const float *__restrict__ 
             for (int i = 0; i < nd; ++i) {
                 float x;
                 float2 a;
-                sample(i, x, a);
+                sample(i, std::true_type{}, x, a);
                 const int col = threadIdx.x + i;
                 float2 sv;
                 if (LINEAR) {
@@ -490,6 +494,29 @@ bpa_errors2_kernel(const float2 *__restrict__ S, BpaParams p, const float *__res
     }
 }
 
+// Whether the two-row kernel's window holds the bins of most chunks of offsets, in the middle row and with pulses a tenth
+// of a bin off: a chunk that it does not hold is summed sample by sample, at about half the rate of the one-row kernel,
+// whose window is a bin wider.  Three chunks in four are enough.  Half a ring, where the outer chunks span three bins:
+// 1800 x 256, M = 900 (two of four held): 970 us against the one-row kernel's 890; 2500 x 256, M = 1250 (three of five)
+// 1514 and 1499; 1031 x 256, M = 340 (none) 348 and 271; 3600 x 100, M = 1800 (all) 909 and 1184; 1800 x 256, M = 594
+// (all) 401 and 518.
+bool pairs_window_holds(const BpaParams &p, int n_rng, int n_az, int M_ap) {
+    const int step = err_step(M_ap), chunks = (M_ap + step - 1) / step;
+    if (chunks > 256) return true;                            // of a degree each
+    const double rho = 0.5 * n_rng * p.dR, R = p.r0 + rho;
+    auto bin = [&](int d) {                                   // of offset d from the row
+        const double s = sin(3.14159265358979323846 * d / n_az);
+        return (sqrt(rho * rho + 4.0 * R * p.r0 * s * s) - rho) / p.dR;
+    };
+    int held = 0;
+    for (int i = 0; i < chunks; ++i) {
+        const int d0 = -(M_ap / 2) + i * step, d1 = min(d0 + step, M_ap - M_ap / 2) - 1;
+        const double a = bin(d0), b = bin(d1), lo = d0 < 0 && d1 > 0 ? 0.0 : fmin(a, b);
+        held += floor(fmax(a, b) + 0.1) + 1.0 - floor(lo - 0.1) <= (double)(ERR_WR - 4);
+    }
+    return 4 * held >= 3 * chunks;
+}
+
 }  // namespace
 
 rosar_status launch_bpa(const float2 *S, const BpaParams &p, const float *dphi, const float *dr, int L, int n_rng,
@@ -502,7 +529,7 @@ rosar_status launch_bpa(const float2 *S, const BpaParams &p, const float *dphi, 
     // us; 1500 x 256, M = 250 (768): 181 -> 147; 1000 x 256, M = 160 (512): 80.6 and 81.7.  Fewer leave warps out and
     // make row 0, whose samples are taken one by one, the last to end: 512 x 128, M = 79: 18 against 32 us.
     const int tiles = (n_az + BPA_THREADS - 1) / BPA_THREADS, pairs = (n_rng + 1) / 2;
-    if (!nominal && (long long)tiles * pairs >= 608) {
+    if (!nominal && (long long)tiles * pairs >= 608 && pairs_window_holds(p, n_rng, n_az, M_ap)) {
         static int done2[2][kMaxDevices] = {};
         const int step = err_step(M_ap), smem = err_smem(step);
         const auto kernel = interp ? bpa_errors2_kernel<true> : bpa_errors2_kernel<false>;

@@ -65,10 +65,10 @@ __device__ __noinline__ void bpa_row_direct(const float2 *__restrict__ S, const 
                 float2 sv;
                 if (linear) {
                     const float fl = floorf(t.x);
-                    const float2 s0 = read_bin(S, (int)fl, L, n, n_az), s1 = read_bin(S, (int)fl + 1, L, n, n_az);
+                    const float2 s0 = read_bin<true>(S, (int)fl, L, n, n_az), s1 = read_bin<true>(S, (int)fl + 1, L, n, n_az);
                     sv = caxpy(t.x - fl, csub(s1, s0), s0);
                 } else {
-                    sv = read_bin(S, (int)floorf(t.x + 0.5f), L, n, n_az);
+                    sv = read_bin<true>(S, (int)floorf(t.x + 0.5f), L, n, n_az);
                 }
                 cmac(acc, make_float2(t.y, t.z), sv);
             }
@@ -276,13 +276,14 @@ const RowsPlan *find_rows(int n_rng, int n_az, int M_ap, bool *circular) {
 // (R_n - rho <= 2 r0 sin(pi d/n_az) falls with rho): M >= 8 planes (whole ring of 97 pulses, 10 planes, 32 rows:
 // 17.7 against 19.2 us direct; 3600 x 256, M = 24: 17.7 against 47.7).  Below about 2e6 pixel-pulses the direct
 // kernel's one short wave is faster than a row's chain of transforms (360 x 64, M = 60: 8.6 against 9.3 us;
-// 480 x 64, M = 80: 9.5 against 9.3; 800 x 64, M = 130: 14.0 against 9.9).
+// 480 x 64, M = 80: 9.5 against 9.3; 800 x 64, M = 130: 14.0 against 9.9), and so is it for a few rows of few pulses
+// (1800 x 32, M = 36: 8.6 against 9.2; 2500 x 32, M = 50: 11.0 against 11.5; 3600 x 32, M = 72: 15.0 against 12.2).
 bool bpa_fft_applies(const BpaParams &p, int n_rng, int n_az, int M_ap) {
     bool circular;
     if (!find_rows(n_rng, n_az, M_ap, &circular)) return false;
     const double half = 3.14159265358979323846 * (double)(M_ap / 2) / (double)n_az;
     const double planes = 2.0 * p.r0 * sin(half) / p.dR + 2.0;
-    return M_ap >= 8.0 * planes && (double)n_rng * n_az * M_ap >= 2e6;
+    return M_ap >= 8.0 * planes && (double)n_rng * n_az * M_ap >= 2e6 && (M_ap >= 64 || n_rng >= 40);
 }
 
 rosar_status launch_bpa_fft(const float2 *S, const BpaParams &p, int L, int n_rng, int n_az, int M_ap, int interp,

@@ -35,3 +35,27 @@ def test_range_compression_of_1024_samples(rosar, n_az):
     l = torch.arange(1024, dtype=torch.float64, device="cuda")
     ref = (ref * torch.polar(torch.ones_like(l), torch.pi * torch.remainder(l * 1023 / 1024, 2.0))).T
     assert torch.linalg.norm(one[0] - ref) <= 2e-6 * torch.linalg.norm(ref)       # the range FFT's bar
+
+
+# errors: the window of two rows holds the chunks of 200 pulses of 800, not those of 264 or 400; nominal: 32 rows of 36
+# pulses are summed directly, 40 rows or 64 pulses go through transforms
+@pytest.mark.parametrize("n_az,L,n_rng,M,errors", [(800, 512, 511, 200, True), (800, 512, 511, 264, True),
+                                                   (800, 512, 512, 400, True), (1800, 64, 32, 36, False),
+                                                   (1800, 64, 40, 36, False), (1800, 64, 36, 64, False)])
+def test_back_projection(rosar, n_az, L, n_rng, M, errors):
+    import oracle as O
+    import torch
+    rng = np.random.default_rng(n_az + M)
+    S = _c(rng, L, n_az)
+    r = synth.TINY.radar
+    api = rosar.Radar(r.fc, r.slope, r.t_sample(L), r.t_start, r.r0, r.c)
+    rad = O.Radar(fc=r.fc, slope=r.slope, t_s=r.t_sample(L), t_start=r.t_start, r0=r.r0, c=r.c)
+    dphi = np.deg2rad(0.05 * rng.standard_normal(n_az)).astype(np.float32) if errors else None
+    dr = (1e-3 * rng.standard_normal(n_az)).astype(np.float32) if errors else None
+    dev = [None if x is None else torch.from_numpy(x).cuda() for x in (dphi, dr)]
+    got = rosar.bpa(torch.from_numpy(S).cuda(), api, n_rng, M, dphi=dev[0], dr=dev[1]).cpu().numpy()
+    rows = np.concatenate([rng.integers(0, n_rng, 60), [0, 0, 1, n_rng - 1, n_rng - 2]])
+    th = np.concatenate([rng.integers(0, n_az, 60), [0, n_az - 1, 5, 7, n_az // 2]])
+    kw = {} if not errors else {"dphi": dphi.astype(np.float64), "dr": dr.astype(np.float64)}
+    ref = O.bpa_pixels(S, rad, n_az, M, rows, th, **kw)
+    assert np.linalg.norm(got[rows, th] - ref) <= 1e-4 * np.linalg.norm(ref)       # the parity tests' bar
