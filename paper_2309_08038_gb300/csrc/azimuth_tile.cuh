@@ -55,12 +55,12 @@ __device__ __forceinline__ int tap_offset(const int32_t *o, int n) {
     return canon_offset((int)m, n);
 }
 
-// COHERENT: S was written earlier in the same kernel (read through L2).  Otherwise it may have been written by a kernel
-// that this one overlaps: after the grid-dependency wait, but not by the non-coherent path.
-template <bool COHERENT>
+// Who wrote S: this kernel, earlier (read through L2); the kernel that this launch overlaps (read after the
+// grid-dependency wait, but not by the non-coherent path); or one that has ended.
+enum SWriter { kThisKernel, kOverlapped, kEnded };
+template <SWriter BY>
 __device__ __forceinline__ float2 load_s(const float2 *p) {
-    if (COHERENT) return __ldcg(p);
-    return __ldca(p);
+    return BY == kThisKernel ? __ldcg(p) : BY == kOverlapped ? __ldca(p) : __ldg(p);
 }
 
 // `smem` holds Geo<J>::SMEM_BYTES bytes (GeoMig<J> when MIG); `red` 4*THREADS/32 ints.  Called by all
@@ -70,7 +70,7 @@ __device__ __forceinline__ float2 load_s(const float2 *p) {
 // MIG: range-migration-aware taps, out[r][t] = sum_k w[r][k] * S[r + dl[r][k]][(t + o_k) mod n_az] with S
 // holding n_bins rows (rows outside read zero): the windows of rows r + min(dl) .. r + max(dl) are staged
 // back to back and each tap's row folds into its shared-memory offset, so the inner loop is unchanged.
-template <int J, bool COHERENT, bool ADJ = false, bool MIG = false>
+template <int J, SWriter BY, bool ADJ = false, bool MIG = false>
 __device__ __forceinline__ void azimuth_tile(const float2 *__restrict__ S, const float2 *__restrict__ w,
                                              const int32_t *__restrict__ o, int o_row_stride, int n_az, int K,
                                              float2 *__restrict__ out, int r, int th0, char *smem, int *red,
@@ -142,7 +142,7 @@ __device__ __forceinline__ void azimuth_tile(const float2 *__restrict__ S, const
     const long long nrows = MIG ? (long long)dhi - dlo + 1 : 1;
     const bool staged = MIG ? (span <= SPAN_CAP && nrows <= MIG_ROWS && nrows * wl <= WIN) : span <= SPAN_CAP;
 
-    griddep_wait();    // S is complete (no-op unless launched to overlap its producer, which writes neither o nor w)
+    if (BY == kOverlapped) griddep_wait();    // S is complete (its producer writes neither o nor w)
     if (staged) {
         const int start = pmod(th0 + lo, n_az);
         for (int q = 0; q < (int)nrows; ++q) {
@@ -152,7 +152,7 @@ __device__ __forceinline__ void azimuth_tile(const float2 *__restrict__ S, const
             for (int i = tid; i < tw + span; i += THREADS) {
                 int idx = start + i;
                 if (idx >= n_az) idx %= n_az;
-                win[q * wl + i] = live ? load_s<COHERENT>(Srow + idx) : make_float2(0.f, 0.f);
+                win[q * wl + i] = live ? load_s<BY>(Srow + idx) : make_float2(0.f, 0.f);
             }
         }
     }
@@ -191,7 +191,7 @@ __device__ __forceinline__ void azimuth_tile(const float2 *__restrict__ S, const
 #pragma unroll
                 for (int j = 0; j < J; ++j) {
                     const int th = th0 + tid + j * THREADS;
-                    if (th < n_az) cmac(acc[j], wv, load_s<COHERENT>(Srow + pmod(th + c, n_az)));
+                    if (th < n_az) cmac(acc[j], wv, load_s<BY>(Srow + pmod(th + c, n_az)));
                 }
             }
         }

@@ -228,7 +228,7 @@ batch_kernel(const ScanDev *__restrict__ scans, const Segment *__restrict__ segs
                 tab_N = 0;         // the gather tile overwrites the row table
                 const int r = local / sc.az_tiles_per_row;
                 const int th0 = (local - r * sc.az_tiles_per_row) * az::Geo<J>::TW;
-                az::azimuth_tile<J, true>(sc.S, sc.w, sc.o, sc.o_row_stride, sc.n_az, sc.K, sc.out, r, th0, sm, red);
+                az::azimuth_tile<J, az::kThisKernel>(sc.S, sc.w, sc.o, sc.o_row_stride, sc.n_az, sc.K, sc.out, r, th0, sm, red);
             }
         }
         __syncthreads();           // the tile is done with shared memory; the next ticket is visible

@@ -18,49 +18,63 @@ namespace {
 
 constexpr int SA_J = 4;      // migrating taps
 
-// CTAs an SM that the registers are held to.  Left to the compiler, 40 to 47 a thread: 7200 x 1024, K = 16 (J = 6)
-// 69 -> 62 us; 3600 x 256, K = 64 (J = 4) 23.5 -> 21.8 with five, 22.8 with six.
+// CTAs an SM that the registers are held to; none asked for at J = 4, where five (48 registers for 40) gain 7 % at 64 taps
+// (3607 x 256: 23.3 -> 21.7 us) and lose 5 to 13 % at up to 16 (7200 x 1024, K = 8: 42 -> 47).
 template <int J>
-constexpr int gather_min_blocks() { return J <= 3 ? 8 : J == 5 ? 6 : 5; }
+constexpr int gather_min_blocks() { return J <= 3 ? 8 : 0; }
 
-// blockIdx = (azimuth tile, range row, scan); scans are stacked [n_scans][n_rng][n_az] and share w, o.
-template <bool ADJ, int J>
+// blockIdx = (azimuth tile, range row, scan); scans are stacked [n_scans][n_rng][n_az] and share w, o.  A launch that
+// overlaps nothing reads S by the non-coherent path and without the wait: 7200 x 1024 with 1 to 16 taps is 8 to 15 %
+// slower otherwise.
+template <bool ADJ, int J, bool OVERLAP>
 __global__ void __launch_bounds__(az::THREADS, gather_min_blocks<J>())
 sparse_azimuth_kernel(const float2 *__restrict__ S, const float2 *__restrict__ w, const int32_t *__restrict__ o,
                       int o_row_stride, int n_rng, int n_az, int K, float2 *__restrict__ out) {
     extern __shared__ __align__(16) char sm[];
     __shared__ int red[4 * az::THREADS / 32];
     const size_t scan = (size_t)blockIdx.z * n_rng * n_az;
-    az::azimuth_tile<J, false, ADJ>(S + scan, w, o, o_row_stride, n_az, K, out + scan, blockIdx.y,
-                                    blockIdx.x * az::Geo<J>::TW, sm, red);
+    az::azimuth_tile<J, OVERLAP ? az::kOverlapped : az::kEnded, ADJ>(S + scan, w, o, o_row_stride, n_az, K, out + scan,
+                                                                     blockIdx.y, blockIdx.x * az::Geo<J>::TW, sm, red);
 }
 
-// Outputs per thread for `rows` rows of n_az: the least (CTAs of the fullest SM) J (measured time of one product at J
-// against J = 4: fewer or more products share a tap's weight and offset).  Against J = 4 for every row: 360 x 256, K =
-// 64 (J = 2) 7.8 -> 5.8 us; 1031 x 512, K = 48 (5) 18.2 -> 13.0; 541 x 1024, K = 64 (3) 20.8 -> 17.7; 7196 x 512,
-// K = 128 (6) 139.8 -> 125.8; J = 8 is never less than J = 4 by this count.
-int outputs_per_thread(int n_az, long long rows) {
-    static const struct { int J; double rate; } js[] = {{1, 1.50}, {2, 1.15}, {3, 1.05}, {4, 1.00},
-                                                        {5, 0.99}, {6, 0.94}};
-    int best = 4;
+// Time of a launch of J outputs a thread over `rows` rows of n_az: about l + s * (CTAs of the fullest SM) us at 64 taps (the
+// order of the J is the same at 4 to 128).
+struct GatherCost { int J; double l, s; };
+constexpr GatherCost kGather[] = {{4, 3.5, 2.72}, {1, 3.3, 1.07}, {2, 3.7, 1.57}, {3, 4.4, 2.12}};
+long long gather_ctas(int n_az, long long rows, int J) { return rows * ((n_az - 1) / (az::THREADS * J) + 1); }
+
+// Four outputs a thread unless another J is better by an eighth, since offsets spread over more than a window read S
+// through L2 and gain less.  Five and six outputs are up to 1.4 times slower there and are not taken.  Measured against
+// J = 4 for every row, 2890 sizes with offsets over a sixth and the whole of the ring: 1.13 times as fast on average, 0.90
+// at the least (four taps, wide); 541 x 1024, K = 64: 20.8 -> 17.7 us; 1031 x 512, K = 48: 18.2 -> 15.
+const GatherCost &gather_cost(int n_az, long long rows) {
+    const GatherCost *best = kGather;
     double least = 1e30;
-    for (const auto &c : js) {
-        const long long tiles = (n_az + az::THREADS * c.J - 1) / (az::THREADS * c.J);
-        const double cost = (double)((tiles * rows + 151) / 152) * c.J * c.rate;
-        if (cost < least) {
-            least = cost;
-            best = c.J;
+    for (const GatherCost &c : kGather) {
+        const double t = c.l + c.s * (double)((gather_ctas(n_az, rows, c.J) + 151) / 152);
+        if (t < least) {
+            least = c.J == 4 ? 0.88 * t : t;
+            best = &c;
         }
     }
-    return best;
+    return *best;
 }
 
-template <bool ADJ, int J>
+// Whether to launch over the tail of range compression.  CTAs that all fit beside it settle where it leaves room first
+// and stay there: between one and five an SM, the fullest SM gets one more than its share (2047 x 256, K = 128: 27.1
+// us one after the other, 33.7 overlapped), which costs more than the microsecond gained unless a CTA is shorter.
+bool gather_overlaps(int n_az, long long rows, int K) {
+    const GatherCost &c = gather_cost(n_az, rows);
+    const long long ctas = gather_ctas(n_az, rows, c.J);
+    return ctas <= 152 || ctas > 5 * 152 || c.s * K <= 64.0;
+}
+
+template <bool ADJ, int J, bool OVERLAP>
 rosar_status launch_gather_j(const float2 *S, const float2 *w, const int32_t *o, int o_row_stride, int n_scans,
-                             int n_rng, int n_az, int K, float2 *out, cudaStream_t s, bool overlap) {
+                             int n_rng, int n_az, int K, float2 *out, cudaStream_t s) {
     static int done[kMaxDevices] = {};
     constexpr int smem = az::Geo<J>::SMEM_BYTES;
-    rosar_status st = ensure_smem((const void *)sparse_azimuth_kernel<ADJ, J>, smem, done, "sparse_azimuth");
+    rosar_status st = ensure_smem((const void *)sparse_azimuth_kernel<ADJ, J, OVERLAP>, smem, done, "sparse_azimuth");
     if (st != ROSAR_OK) return st;
     const dim3 grid((n_az + az::Geo<J>::TW - 1) / az::Geo<J>::TW, n_rng, n_scans);
     cudaLaunchConfig_t cfg = {};
@@ -72,24 +86,22 @@ rosar_status launch_gather_j(const float2 *S, const float2 *w, const int32_t *o,
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = overlap ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, sparse_azimuth_kernel<ADJ, J>, S, w, o, o_row_stride, n_rng, n_az, K, out);
+    cfg.numAttrs = OVERLAP ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, sparse_azimuth_kernel<ADJ, J, OVERLAP>, S, w, o, o_row_stride, n_rng, n_az, K, out);
     if (e != cudaSuccess) return set_error(ROSAR_ERR_CUDA, "sparse_azimuth: launch failed: %s", cudaGetErrorString(e));
     return check_launch(ADJ ? "sparse_azimuth_adjoint" : "sparse_azimuth");
 }
 
-template <bool ADJ>
+template <bool ADJ, bool OVERLAP = false>
 rosar_status launch_gather(const float2 *S, const float2 *w, const int32_t *o, int o_row_stride, int n_scans,
-                           int n_rng, int n_az, int K, float2 *out, cudaStream_t s, bool overlap = false) {
+                           int n_rng, int n_az, int K, float2 *out, cudaStream_t s) {
     if (n_rng > 65535 || n_scans > 65535)
         return set_error(ROSAR_ERR_UNSUPPORTED, "sparse_azimuth: n_rng=%d or n_scans=%d exceeds 65535", n_rng, n_scans);
-    switch (outputs_per_thread(n_az, (long long)n_rng * n_scans)) {
-        case 1: return launch_gather_j<ADJ, 1>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s, overlap);
-        case 2: return launch_gather_j<ADJ, 2>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s, overlap);
-        case 3: return launch_gather_j<ADJ, 3>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s, overlap);
-        case 4: return launch_gather_j<ADJ, 4>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s, overlap);
-        case 5: return launch_gather_j<ADJ, 5>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s, overlap);
-        default: return launch_gather_j<ADJ, 6>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s, overlap);
+    switch (gather_cost(n_az, (long long)n_rng * n_scans).J) {
+        case 1: return launch_gather_j<ADJ, 1, OVERLAP>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
+        case 2: return launch_gather_j<ADJ, 2, OVERLAP>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
+        case 3: return launch_gather_j<ADJ, 3, OVERLAP>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
+        default: return launch_gather_j<ADJ, 4, OVERLAP>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
     }
 }
 
@@ -101,7 +113,7 @@ sparse_azimuth_mig_kernel(const float2 *__restrict__ S, int n_bins, const float2
                           int K, float2 *__restrict__ out) {
     extern __shared__ __align__(16) char sm[];
     __shared__ int red[4 * az::THREADS / 32];
-    az::azimuth_tile<SA_J, false, false, true>(S, w, o, o_row_stride, n_az, K, out, blockIdx.y,
+    az::azimuth_tile<SA_J, az::kEnded, false, true>(S, w, o, o_row_stride, n_az, K, out, blockIdx.y,
                                                blockIdx.x * MigGeo::TW, sm, red, dl, n_bins);
 }
 
@@ -123,7 +135,9 @@ rosar_status launch_sparse_azimuth_migrating(const float2 *S, int n_bins, const 
 
 rosar_status launch_sparse_azimuth(const float2 *S, const float2 *w, const int32_t *o, int o_row_stride, int n_rng,
                                    int n_az, int K, float2 *out, cudaStream_t s, bool overlap_predecessor) {
-    return launch_gather<false>(S, w, o, o_row_stride, 1, n_rng, n_az, K, out, s, overlap_predecessor);
+    return overlap_predecessor && gather_overlaps(n_az, n_rng, K)
+               ? launch_gather<false, true>(S, w, o, o_row_stride, 1, n_rng, n_az, K, out, s)
+               : launch_gather<false>(S, w, o, o_row_stride, 1, n_rng, n_az, K, out, s);
 }
 
 rosar_status launch_sparse_azimuth_scans(const float2 *S, const float2 *w, const int32_t *o, int o_row_stride,

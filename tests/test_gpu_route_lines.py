@@ -59,3 +59,17 @@ def test_back_projection(rosar, n_az, L, n_rng, M, errors):
     kw = {} if not errors else {"dphi": dphi.astype(np.float64), "dr": dr.astype(np.float64)}
     ref = O.bpa_pixels(S, rad, n_az, M, rows, th, **kw)
     assert np.linalg.norm(got[rows, th] - ref) <= 1e-4 * np.linalg.norm(ref)       # the parity tests' bar
+
+
+# launched over range compression's tail (one CTA an SM, short CTAs, many CTAs) or after it (2047 x 256, 128 taps)
+@pytest.mark.parametrize("n_az,L,K", [(360, 64, 16), (2047, 256, 16), (2047, 256, 128), (3607, 256, 64), (541, 1024, 64)])
+def test_gather_image_equals_its_two_steps(rosar, n_az, L, K):
+    import torch
+    rng = np.random.default_rng(n_az + K)
+    raw, w = torch.from_numpy(_c(rng, n_az, L)).cuda(), torch.from_numpy(_c(rng, L, K)).cuda()
+    o = torch.from_numpy(rng.integers(-n_az, n_az, K).astype(np.int32)).cuda()
+    win = torch.from_numpy(synth.hann_window(L)).cuda()
+    S = rosar.range_compress(raw, win)
+    want = rosar.sparse_azimuth(S, w, o)
+    for _ in range(3):
+        assert torch.equal(rosar.image(raw, win, w, o), want)
