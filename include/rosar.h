@@ -279,6 +279,8 @@ ROSAR_API rosar_status rosar_bpa_time_planned(const rosar_c32 *raw, const void *
  *     enough transform, an arm of very many range bins), sizes too small for it to pay, or invalid arguments.  Never
  *     equal to rosar_time_domain_plan_bytes.  P n_rng rows of the padded pulse count, 8 bytes a value: for SAS, whose
  *     offsets may reach half a turn, P is near 30 for an arm of 4 bins (0.2 GB for 3600 x 256), so large scans take GBs.
+ *   rosar_time_domain_fft_pays: 1 where SAS by transforms is offered and expected to be faster than rosar_sas_time and
+ *     rosar_sas_time_planned, whatever the offsets; else 0 (few taps, pulse counts that need a much longer transform).
  *   rosar_time_domain_fft_workspace_bytes: scratch of one image call.
  *   rosar_*_time_fft_plan: writes the plan (device, 256-byte aligned); arguments as rosar_*_time_plan.
  *   rosar_*_time_fft: the image from raw (as rosar_*_time_planned), the plan and a workspace (device, 256-byte
@@ -287,6 +289,7 @@ ROSAR_API rosar_status rosar_bpa_time_planned(const rosar_c32 *raw, const void *
  *     other sizes or not written by rosar_*_time_fft_plan is read no further than its first 32 bytes, and the image is NaN.
  */
 ROSAR_API size_t rosar_time_domain_fft_plan_bytes(const rosar_radar *radar, int bpa, int n_az, int L, int n_rng, int K);
+ROSAR_API int rosar_time_domain_fft_pays(const rosar_radar *radar, int n_az, int L, int n_rng, int K);
 ROSAR_API size_t rosar_time_domain_fft_workspace_bytes(int bpa, int n_az, int L, int n_rng, int K);
 ROSAR_API rosar_status rosar_bpa_time_fft_plan(const float *win, const rosar_radar *radar, int n_az, int L, int n_rng,
                                                int M_ap, void *plan, size_t plan_bytes, void *stream);

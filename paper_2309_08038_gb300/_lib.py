@@ -76,6 +76,7 @@ _PROTOS = {
     "rosar_bpa_time_plan": (_I, [_P, ctypes.POINTER(RadarStruct), _I, _I, _I, _I, _P, ctypes.c_size_t, _P]),
     "rosar_bpa_time_planned": (_I, [_P, _P, _I, _I, _I, _I, _P, _P]),
     "rosar_time_domain_fft_plan_bytes": (ctypes.c_size_t, [ctypes.POINTER(RadarStruct), _I, _I, _I, _I, _I]),
+    "rosar_time_domain_fft_pays": (_I, [ctypes.POINTER(RadarStruct), _I, _I, _I, _I]),
     "rosar_time_domain_fft_workspace_bytes": (ctypes.c_size_t, [_I, _I, _I, _I, _I]),
     "rosar_bpa_time_fft_plan": (_I, [_P, ctypes.POINTER(RadarStruct), _I, _I, _I, _I, _P, ctypes.c_size_t, _P]),
     "rosar_sas_time_fft_plan": (_I, [_P, _P, _P, ctypes.POINTER(RadarStruct), _I, _I, _I, _I, _I, _P, ctypes.c_size_t,

@@ -405,6 +405,14 @@ size_t rosar_time_domain_fft_plan_bytes(const rosar_radar *radar, int bpa, int n
     return ok ? plan : 0;
 }
 
+int rosar_time_domain_fft_pays(const rosar_radar *radar, int n_az, int L, int n_rng, int K) {
+    TdParams p;
+    size_t plan = 0, ws = 0;
+    const bool ok = fft_form(radar, 0, n_az, L, n_rng, K, &p, &plan, &ws) && time_domain_lr_pays(p, K);
+    clear_error();
+    return ok ? 1 : 0;
+}
+
 size_t rosar_time_domain_fft_workspace_bytes(int bpa, int n_az, int L, int n_rng, int K) {
     return time_domain_lr_workspace(bpa == 1, n_az, L, n_rng, K);
 }

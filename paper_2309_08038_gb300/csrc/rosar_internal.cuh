@@ -171,6 +171,7 @@ rosar_status launch_bpa_fft(const float2 *S, const BpaParams &p, int L, int n_rn
 // The same by transforms (time_domain_lr.cu): whether it is taken for these sizes and what it needs, the plan
 // (geometry only), the image from a plan and a workspace.
 bool time_domain_lr_applies(const TdParams &p, bool bpa, int K, size_t *plan_bytes, size_t *ws_bytes);
+bool time_domain_lr_pays(const TdParams &p, int K);      // SAS
 size_t time_domain_lr_workspace(bool bpa, int n_az, int L, int n_rng, int K);
 size_t time_domain_lr_plan_least(bool bpa, int n_az, int L, int n_rng, int K);   // bytes that every plan of these sizes has
 rosar_status launch_time_domain_lr_plan(const float *win, const float2 *w, const int32_t *o, const TdParams &p, int K,

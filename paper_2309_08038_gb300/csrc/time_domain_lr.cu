@@ -766,6 +766,24 @@ bool time_domain_lr_applies(const TdParams &p, bool bpa, int K, size_t *plan_byt
     return true;
 }
 
+// Whether SAS by transforms is the faster form, planned and with the plan built in the call, also where the offsets reach
+// half a turn (the planes that its plan has room for): times in us of both forms as sums of their parts, fitted to 705
+// sizes (97 to 14400 pulses, 16 to 2048 samples, 1 to 2048 rows, 2 to 256 taps, offsets over a sixth and the whole of the
+// ring) to 20 to 30 %.  With the transforms asked to be 1.3 times as fast, 5 of them are slower with wide offsets (0.74 at
+// the least) and none with narrow ones, where all of them by transforms were 128: 4501 x 208, K = 2: 214 us against 45;
+// 14400 x 64, K = 2: 74 and 19; 3600 x 1024, 16 rows, K = 2: 152 and 147.  3600 x 256, K = 64 has 92 against 640.
+bool time_domain_lr_pays(const TdParams &p, int K) {
+    const Shape sh = lr::shape_of(false, p.n_az, p.L, p.n_rng, K);
+    if (!sh.valid) return false;
+    const double P = lr::planes_bound(p, false, K, sh.Lf), N = sh.N, L = p.L, q = p.n_rng, n = p.n_az;
+    const double image = 9.0 + 0.66 * P + 1e-6 * (9.7 * n * L + 8.0 * L * N + 6.2 * q * N + 1.5 * P * N * sh.Lf);
+    const double plan = 21.0 + 1e-6 * (2.9 * P * q * N + 14.5 * P * q * K + 340.0 * N);
+    const double tiles = ceil(n / 128.0) * ceil(q / 64.0), sums = tiles * K * L;     // of the tensor cores
+    const double direct = 40.0 + 2.53e-4 * sums + 3.9e-3 * L * K;
+    const double direct_planned = 22.0 + 1.77e-4 * sums + 3.1e-3 * L * K + 0.034 * tiles;
+    return direct > 1.3 * (image + plan) && direct_planned > 1.3 * image;
+}
+
 size_t time_domain_lr_workspace(bool bpa, int n_az, int L, int n_rng, int K) {
     const Shape sh = lr::shape_of(bpa, n_az, L, n_rng, K);
     return sh.valid ? sh.ws_bytes : 0;

@@ -205,10 +205,19 @@ def bpa_time(raw, win, radar: Radar, n_rng, M_ap, out=None, stream=None, transfo
     return out
 
 
-def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
+def _sas_transforms(lib, st, n_az, L, n_rng, K, transforms):
+    """Bytes of the plan by transforms, 0 for the tensor-core form."""
+    sizes = (n_az, L, n_rng, K)
+    if transforms is False or (transforms is None and not lib.rosar_time_domain_fft_pays(ctypes.byref(st), *sizes)):
+        return 0
+    return lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, *sizes)
+
+
+def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None, transforms=None):
     """rosar_sas_time: time-domain sparse-aperture imaging (Algorithm 2) of the raw cube [n_az, L]; one output
-    row per row of w [n_rng, K].  Shared offsets by transforms (rosar_sas_time_fft) where the library offers that
-    and the plan and workspace, taken for the call, fit SCRATCH_LIMIT and the device."""
+    row per row of w [n_rng, K].  Shared offsets by transforms (rosar_sas_time_fft) where that is faster
+    (rosar_time_domain_fft_pays) and the plan and workspace, taken for the call, fit SCRATCH_LIMIT and the device;
+    transforms=True: wherever the library offers that form; False: never."""
     lib = _lib.load()
     require(raw, torch.complex64, "raw", ndim=2)
     n_az, L = raw.shape
@@ -221,11 +230,11 @@ def sas_time(raw, win, w, o, radar: Radar, centred=True, out=None, stream=None):
         out = _empty((n_rng, n_az), torch.complex64, raw.device, stream)
     require(out, torch.complex64, "out", shape=(n_rng, n_az))
     st = radar.as_struct()
-    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, n_az, L, n_rng, K) if stride == 0 else 0
+    nbytes = _sas_transforms(lib, st, n_az, L, n_rng, K, transforms) if stride == 0 else 0
     scratch = None
     if nbytes and raw.data_ptr() % 16 == 0 and not _overlaps(out, w, o):      # the direct call says what it refuses
         at, ws = _up256(nbytes), lib.rosar_time_domain_fft_workspace_bytes(0, n_az, L, n_rng, K)
-        scratch = _optional_scratch(at + ws, raw.device, stream)
+        scratch = _scratch(at + ws, raw.device, stream) if transforms else _optional_scratch(at + ws, raw.device, stream)
     if scratch is not None:
         h = stream_handle(stream)
         check(lib.rosar_sas_time_fft_plan(ptr(win), ptr(w), ptr(o), ctypes.byref(st), n_az, L, n_rng, K,
@@ -258,9 +267,10 @@ def _plan_tensor(nbytes, n_rng, L, K, device, stream):
     return _scratch(nbytes or int(_lib.load().rosar_time_domain_plan_bytes(n_rng, L, K)), device, stream)
 
 
-def sas_time_plan(win, w, o, radar: Radar, n_az, L, centred=True, stream=None):
-    """rosar_sas_time_fft_plan, where the library offers that form and the device has room for its plan (about 240 bytes a
-    pixel, see SCRATCH_LIMIT), else rosar_sas_time_plan, for the weights w [n_rng, K] and shared offsets o [K]."""
+def sas_time_plan(win, w, o, radar: Radar, n_az, L, centred=True, stream=None, transforms=None):
+    """The plan of rosar_sas_time for the weights w [n_rng, K] and shared offsets o [K]: rosar_sas_time_fft_plan where that
+    form is faster and the device has room for it (about 240 bytes a pixel, see SCRATCH_LIMIT), else rosar_sas_time_plan;
+    transforms as in sas_time."""
     lib = _lib.load()
     require(w, torch.complex64, "w", ndim=2)
     n_rng, K = w.shape
@@ -268,11 +278,11 @@ def sas_time_plan(win, w, o, radar: Radar, n_az, L, centred=True, stream=None):
     if win is not None:
         require(win, torch.float32, "win", shape=(L,))
     st = radar.as_struct()
-    nbytes = lib.rosar_time_domain_fft_plan_bytes(ctypes.byref(st), 0, n_az, L, n_rng, K)
+    nbytes = _sas_transforms(lib, st, n_az, L, n_rng, K, transforms)
     try:
         data = _plan_tensor(nbytes, n_rng, L, K, w.device, stream)
     except torch.cuda.OutOfMemoryError:
-        if not nbytes:
+        if not nbytes or transforms:
             raise
         nbytes = 0
         data = _plan_tensor(0, n_rng, L, K, w.device, stream)

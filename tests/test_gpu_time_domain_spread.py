@@ -48,7 +48,7 @@ def test_large_samples_stay_where_they_are_read(rosar, bpa, n_az, L, size):
     else:
         assert lib.rosar_sas_time(t_raw.data_ptr(), win.data_ptr(), t_w.data_ptr(), t_o.data_ptr(), 0, ctypes.byref(st), n_az,
                                   L, L, K, 1, ref.data_ptr(), s) == 0
-        image = lambda x: rosar.sas_time(x, win, t_w, t_o, api)  # noqa: E731
+        image = lambda x: rosar.sas_time(x, win, t_w, t_o, api, transforms=True)  # noqa: E731
     got, alone = image(t_raw).cpu().numpy(), image(t_clean).cpu().numpy()
     again = image(t_raw).cpu().numpy()
     ref = ref.cpu().numpy()

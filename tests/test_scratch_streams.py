@@ -40,7 +40,7 @@ def test_scratch_comes_from_the_stream_of_the_call(monkeypatch):
     plan = ops.TimeDomainPlan(empty(1024, dtype=torch.uint8), 64, 32, 32, 4)
     monkeypatch.setattr(torch, "empty", lambda *a, **k: (made.append(active[-1]), empty(*a, **k))[1])
     calls = [lambda **k: ops.bpa_time(raw, None, radar, 32, 4, out=out, transforms=True, **k),
-             lambda **k: ops.sas_time(raw, None, w, o, radar, out=out, **k),
+             lambda **k: ops.sas_time(raw, None, w, o, radar, out=out, transforms=True, **k),
              lambda **k: ops.sas_time_planned(raw, plan, out=out, **k),
              lambda **k: ops.bpa_time_planned(raw, plan, out=out, **k)]
     for call in calls:
@@ -65,9 +65,9 @@ def test_calls_on_two_streams_do_not_share_scratch():
     raws = [torch.randn(n_az, L, dtype=torch.complex64, device="cuda", generator=g) for _ in range(2)]
     w = torch.randn(L, K, dtype=torch.complex64, device="cuda", generator=g)
     o = torch.from_numpy(np.arange(-12, 12, dtype=np.int32) * 7).cuda()
-    plan = rosar.sas_time_plan(None, w, o, api, n_az, L)
+    plan = rosar.sas_time_plan(None, w, o, api, n_az, L, transforms=True)
     assert plan.data.numel() != rosar.load().rosar_time_domain_plan_bytes(L, L, K)      # the form with scratch
-    forms = [lambda raw, **k: rosar.sas_time_planned(raw, plan, **k), lambda raw, **k: rosar.sas_time(raw, None, w, o, api, **k)]
+    forms = [lambda raw, **k: rosar.sas_time_planned(raw, plan, **k), lambda raw, **k: rosar.sas_time(raw, None, w, o, api, transforms=True, **k)]
     side = torch.cuda.Stream()
     for form in forms:
         want = [form(raw) for raw in raws]

@@ -39,7 +39,7 @@ def test_sas_time_leaves_an_overlap_to_the_direct_call(lib):
     for args, names in (((w, o), ["rosar_sas_time_fft_plan", "rosar_sas_time_fft"]), ((into_w, o), ["rosar_sas_time"]),
                         ((w, into_o), ["rosar_sas_time"])):
         lib.called.clear()
-        ops.sas_time(raw, None, *args, RADAR, out=out)
+        ops.sas_time(raw, None, *args, RADAR, out=out, transforms=True)
         assert lib.called == names
 
 

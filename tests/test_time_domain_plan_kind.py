@@ -53,7 +53,7 @@ def _case(rosar, n_az, L, n_rng, K):
     raw = torch.randn(n_az, L, dtype=torch.complex64, device="cuda", generator=g)
     w = torch.randn(n_rng, K, dtype=torch.complex64, device="cuda", generator=g)
     o = torch.arange(K, dtype=torch.int32, device="cuda") - K // 2
-    return api, raw, rosar.sas_time_plan(None, w, o, api, n_az, L), rosar.bpa_time_plan(None, api, n_az, L, n_rng, K, transforms=True)
+    return api, raw, rosar.sas_time_plan(None, w, o, api, n_az, L, transforms=True), rosar.bpa_time_plan(None, api, n_az, L, n_rng, K, transforms=True)
 
 
 # 1031: the two kinds pad the row to different lengths; 360: to the same
