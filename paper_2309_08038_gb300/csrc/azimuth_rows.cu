@@ -181,11 +181,12 @@ rosar_status launch_runtime(const RowLaunch &l, const ROWS &rows, const RowPlan 
     return check_launch("azimuth_fft");
 }
 
-// The run-time plan: the staged H row pays where a row's own latency counts.  Against loading the row, the passes,
-// the product and the store as steps of their own: 800 pulses, 256 rows 8.3 -> 7.1 us, 2048 rows 47 -> 22; 4500:
-// 23.9 -> 19.7 and 165 -> 89; 16384: 76 -> 51 (256 rows).
+// The run-time plan: the staged H row pays where a row's own latency counts, up to two rows an SM.  Against loading the
+// row, the passes, the product and the store as steps of their own: 800 pulses, 256 rows 8.3 -> 7.1 us, 2048 rows 47 ->
+// 22; 4500: 23.9 -> 19.7 and 165 -> 89; 16384: 76 -> 51 (256 rows).
 template <typename ROWS>
-rosar_status launch_rows_runtime(const RowLaunch &l, const ROWS &rows, const RowPlan &pl, bool few) {
+rosar_status launch_rows_runtime(const RowLaunch &l, const ROWS &rows, const RowPlan &pl) {
+    const bool few = l.n_rng <= 304;
     const Layout lay = layout_for(l.n_az, few);
     if (l.n_az <= 4096) return launch_runtime<ROWS, 256, 3>(l, rows, pl, lay, !few && l.n_az <= 2048 ? 128 : 256);
     if (l.n_az <= 8192 && !few) return launch_runtime<ROWS, 256, 3>(l, rows, pl, lay, 256);
@@ -194,13 +195,13 @@ rosar_status launch_rows_runtime(const RowLaunch &l, const ROWS &rows, const Row
     return launch_runtime<ROWS, 512, 1>(l, rows, pl, lay, 512);
 }
 
-// Up to two rows an SM, a row's own latency counts: 256 threads and H staged while S is awaited.  With more the SM's
+// Up to three rows an SM, a row's own latency counts: 256 threads and H staged while S is awaited.  With more the SM's
 // rows in flight count: one row of shared memory and at most 64 registers hold 4 CTAs of 3600 pulses (46 % of the
 // warps instead of 30) or 8 of 1800, and H is read in the fused step.  4096 rows of 3600 pulses 82 -> 77 us, 8192 of
-// 1800 97 -> 76; at 256 rows 10.3 and 10.4, 6.4 and 8.2.  7200-pulse rows hold one CTA an SM with H staged: 152 rows
-// 10.2 us (11.3 not staged).  With more rows three CTAs an SM and the passes of radix 8 and 4 together in registers
+// 1800 97 -> 76; 305 rows of 360 3.50 and 3.69, 400 rows of 1800 6.38 and 6.61 (457 rows: 5.13 and 3.82, 8.43 and 7.61).
+// 7200-pulse rows hold one CTA an SM with H staged: 152 rows 10.2 us (11.3 not staged).  With more rows three CTAs an SM and the passes of radix 8 and 4 together in registers
 // (PAIRED): 256 rows 18.4 -> 15.8 -> 13.8, 1024 rows 72 -> 54 -> 47, 4096 rows 271 -> 186 -> 159 (176 on two CTAs).
-constexpr int kFewRows = 304;
+constexpr int kFewRows = 456;
 
 template <typename ROWS>
 rosar_status launch_rows_of(const RowLaunch &l, const ROWS &rows) {
@@ -208,7 +209,7 @@ rosar_status launch_rows_of(const RowLaunch &l, const ROWS &rows) {
     if (!make_plan(l.n_az, &pl))
         return set_error(ROSAR_ERR_UNSUPPORTED, "azimuth_fft: n_az=%d is not 2^a 3^b 5^c in [2, %d]", l.n_az, AF_MAX_N);
     const bool few = l.n_rng <= kFewRows;
-    if (stored_radix(l.n_az, pl) == 0) return launch_rows_runtime<ROWS>(l, rows, pl, few);
+    if (stored_radix(l.n_az, pl) == 0) return launch_rows_runtime<ROWS>(l, rows, pl);
     if (Row3600::is(l.n_az, pl))
         return few ? launch_fixed<ROWS, 256, 2, 3600, kStaged, false, 16, 15, 15>(l, rows)
                    : launch_fixed<ROWS, 256, 4, 3600, kFused, false, 16, 15, 15>(l, rows);

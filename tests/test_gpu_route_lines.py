@@ -73,3 +73,29 @@ def test_gather_image_equals_its_two_steps(rosar, n_az, L, K):
     want = rosar.sparse_azimuth(S, w, o)
     for _ in range(3):
         assert torch.equal(rosar.image(raw, win, w, o), want)
+
+
+# rows of the compile-time lengths: H staged up to 456 rows, read in the fused step from 457 on (7200 and 14400: 152, 153)
+@pytest.mark.parametrize("n_az,rows", [(360, 456), (360, 457), (1800, 456), (1800, 457), (3600, 456), (3600, 457),
+                                       (7200, 152), (7200, 153), (14400, 153), (800, 304), (800, 305)])
+def test_row_filter(rosar, n_az, rows):
+    import oracle as O
+    import torch
+    rng = np.random.default_rng(n_az + rows)
+    w = _c(rng, rows, 6)
+    o = rng.integers(-n_az, n_az, 6).astype(np.int32)
+    S = _c(rng, rows, n_az)
+    tS, tw, to = (torch.from_numpy(x).cuda() for x in (S, w, o))
+    H = rosar.azimuth_plan(tw, to, n_az)
+    got = rosar.sparse_azimuth_fft(tS, H)
+    for a in (0, 100, rows - 50):                    # few rows of it alone
+        assert torch.equal(rosar.sparse_azimuth_fft(tS[a:a + 50].contiguous(), H[a:a + 50].contiguous()), got[a:a + 50])
+    ref = O.sparse_azimuth(S[-3:], w[-3:], o)
+    assert np.linalg.norm(got[-3:].cpu().numpy() - ref) <= 5e-6 * np.linalg.norm(ref)      # the filter's bar
+    X = torch.empty_like(tS)[None]
+    G = torch.empty_like(X)
+    rosar.sparse_azimuth_fft_scans_ex(tS[None], H, spectrum=X)
+    rosar.sparse_azimuth_fft_scans_ex(got[None], H, adjoint=True, spectrum=G)
+    grad = rosar.azimuth_weight_grad_spectra(G, X, to, 6).cpu().numpy()
+    ref = O.sparse_azimuth_adjoint_w(got[-3:].cpu().numpy(), S[-3:], o)
+    assert np.linalg.norm(grad[-3:] - ref) <= 1e-5 * np.linalg.norm(ref)                   # the gradients' bar
