@@ -196,11 +196,12 @@ rosar_status launch_rows_runtime(const RowLaunch &l, const ROWS &rows, const Row
 }
 
 // Up to three rows an SM, a row's own latency counts: 256 threads and H staged while S is awaited.  With more the SM's
-// rows in flight count: one row of shared memory and at most 64 registers hold 4 CTAs of 3600 pulses (46 % of the
-// warps instead of 30) or 8 of 1800, and H is read in the fused step.  4096 rows of 3600 pulses 82 -> 77 us, 8192 of
-// 1800 97 -> 76; 305 rows of 360 3.50 and 3.69, 400 rows of 1800 6.38 and 6.61 (457 rows: 5.13 and 3.82, 8.43 and 7.61).
-// 7200-pulse rows hold one CTA an SM with H staged: 152 rows 10.2 us (11.3 not staged).  With more rows three CTAs an SM and the passes of radix 8 and 4 together in registers
-// (PAIRED): 256 rows 18.4 -> 15.8 -> 13.8, 1024 rows 72 -> 54 -> 47, 4096 rows 271 -> 186 -> 159 (176 on two CTAs).
+// rows in flight count: one row of shared memory and at most 64 registers hold 4 CTAs of 3600 pulses (46 % of the warps
+// instead of 30) or 8 of 1800, and H is read in the fused step.  4096 rows of 3600 pulses 82 -> 77 us, 8192 of 1800 97 ->
+// 76; 305 rows of 360 3.50 and 3.69, 400 rows of 1800 6.38 and 6.61, but 457 rows 5.13 and 3.82, 8.43 and 7.61.
+// 7200-pulse rows hold one CTA an SM with H staged: 152 rows 10.2 us (11.3 not staged).  With more rows three CTAs an SM
+// and the passes of radix 8 and 4 together in registers (PAIRED): 256 rows 18.4 -> 15.8 -> 13.8, 1024 rows 72 -> 54 ->
+// 47, 4096 rows 271 -> 186 -> 159 (176 on two CTAs).
 constexpr int kFewRows = 456;
 
 template <typename ROWS>

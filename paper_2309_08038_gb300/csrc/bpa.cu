@@ -250,8 +250,9 @@ bpa_kernel(const float2 *__restrict__ S, BpaParams p, const float *__restrict__ 
 }
 
 // --------------------------------------------------------------------- supplied errors, two rows a thread --
-// For grids that fill the SMs with half the threads.  Two rows (r, r + 1) a thread: the angle between pixel and pulse is the same in both, so the sine of its half (sh),
-// 4 r_n sh^2 - 2 dr_n (u) and cos of the angle are taken once, and what depends on the row,
+// For grids that fill the SMs with half the threads.  Two rows (r, r + 1) a thread: the angle between pixel and pulse is
+// the same in both, so the sine of its half (sh), 4 r_n sh^2 - 2 dr_n (u) and cos of the angle are taken once, and what
+// depends on the row,
 //   R_n^2 - rho^2 = R u + dr_n (r_n + r0),   rho - dr_n - 2 R sh^2 = R (1 - 2 sh^2) - r_n,
 // through delta, the bin and the phase, runs as packed FP32x2 instructions over the two.  The whole part of the
 // bin and of the phase in turns come from an addition that rounds to an integer in the low mantissa bits (no

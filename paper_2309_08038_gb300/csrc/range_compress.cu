@@ -25,7 +25,8 @@ namespace {
 // the memory latency at the scan sizes of interest.  L = 1024 takes 8 pulses (stores of 64 bytes instead of 32) on 512
 // threads at 64 registers, two CTAs an SM: 14400 pulses 55.0 -> 52.2 us, or HALF of them (half_tiles below).
 template <int L, bool HALF = false>
-struct Plan : fft::Tile<L, (L <= 16 ? 32 : L <= 64 ? 16 : L <= 256 ? 8 : L == 512 || (L == 1024 && HALF) ? 4 : L == 1024 ? 8 : 2)> {
+struct Plan : fft::Tile<L, (L <= 16 ? 32 : L <= 64 ? 16 : L <= 256 ? 8 : L == 512 || (L == 1024 && HALF) ? 4
+                            : L == 1024 ? 8 : 2)> {
     // 0: none asked for.  A minimum of one lets the compiler spend 98 registers on L = 256 where it takes 80: 16 scans of
     // 3600 pulses 39.8 -> 45.7 us.
     static constexpr int MINB = L == 1024 && !HALF ? 2 : 0;
@@ -62,9 +63,9 @@ rosar_status launch_group_L(const ScanGroup &g, int total, cudaStream_t s, bool 
 }
 
 // Pulses a CTA of the adjoint: 8 are a 64-byte segment of a bin's row (from L = 1024 on 4 run faster), and 4 consecutive
-// samples of a pulse's are a sector.  Bound by memory: 16 scans of 3600 x 256 82 -> 54.6 us (of 35 at the copy rate), x 128 49 -> 28.7, 8 scans of
-// x 512 109 -> 66 (75 on two CTAs an SM), 14400 x 1024 102 -> 63 (72 with 8 pulses a CTA), against bins staged pulse by pulse in shared memory
-// before the first pass and after the last.
+// samples of a pulse's are a sector.  Bound by memory: 16 scans of 3600 x 256 82 -> 54.6 us (of 35 at the copy rate),
+// x 128 49 -> 28.7, 8 scans of x 512 109 -> 66 (75 on two CTAs an SM), 14400 x 1024 102 -> 63 (72 with 8 pulses a CTA),
+// against bins staged pulse by pulse in shared memory before the first pass and after the last.
 template <int L>
 struct AdjointPlan : fft::Tile<L, (L <= 16 ? 32 : L <= 32 ? 16 : L <= 512 ? 8 : L <= 2048 ? 4 : 2)> {
     using Base = fft::Tile<L, (L <= 16 ? 32 : L <= 32 ? 16 : L <= 512 ? 8 : L <= 2048 ? 4 : 2)>;

@@ -18,16 +18,17 @@ namespace {
 
 constexpr int SA_J = 4;      // migrating taps
 
-// CTAs an SM that the registers are held to; none asked for at J = 4, where five (48 registers for 40) gain 7 % at 64 taps
-// (3607 x 256: 23.3 -> 21.7 us) and lose 5 to 13 % at up to 16 (7200 x 1024, K = 8: 42 -> 47).
-template <int J>
-constexpr int gather_min_blocks() { return J <= 3 ? 8 : 0; }
+// CTAs an SM that the registers are held to.  At J = 4 none is asked for: five (48 registers for 40) lose 5 to 13 % at up to
+// 16 taps (7200 x 1024, K = 8: 42 -> 47 us) and up to 7 % with offsets over the whole ring; but MANY taps after range
+// compression's tail gain (image of 3607 x 256, K = 128: 45.9 -> 41.8).
+template <int J, bool MANY>
+constexpr int gather_min_blocks() { return J <= 3 ? 8 : MANY ? 5 : 0; }
 
 // blockIdx = (azimuth tile, range row, scan); scans are stacked [n_scans][n_rng][n_az] and share w, o.  A launch that
 // overlaps nothing reads S by the non-coherent path and without the wait: 7200 x 1024 with 1 to 16 taps is 8 to 15 %
 // slower otherwise.
-template <bool ADJ, int J, bool OVERLAP>
-__global__ void __launch_bounds__(az::THREADS, gather_min_blocks<J>())
+template <bool ADJ, int J, bool OVERLAP, bool MANY>
+__global__ void __launch_bounds__(az::THREADS, (gather_min_blocks<J, MANY>()))
 sparse_azimuth_kernel(const float2 *__restrict__ S, const float2 *__restrict__ w, const int32_t *__restrict__ o,
                       int o_row_stride, int n_rng, int n_az, int K, float2 *__restrict__ out) {
     extern __shared__ __align__(16) char sm[];
@@ -41,7 +42,9 @@ sparse_azimuth_kernel(const float2 *__restrict__ S, const float2 *__restrict__ w
 // order of the J is the same at 4 to 128).
 struct GatherCost { int J; double l, s; };
 constexpr GatherCost kGather[] = {{4, 3.5, 2.72}, {1, 3.3, 1.07}, {2, 3.7, 1.57}, {3, 4.4, 2.12}};
-long long gather_ctas(int n_az, long long rows, int J) { return rows * ((n_az - 1) / (az::THREADS * J) + 1); }
+long long gather_ctas(int n_az, long long rows, int J) {
+    return rows * ((n_az - 1) / (az::THREADS * J) + 1);
+}
 
 // Four outputs a thread unless another J is better by an eighth, since offsets spread over more than a window read S
 // through L2 and gain less.  Five and six outputs are up to 1.4 times slower there and are not taken.  Measured against
@@ -69,12 +72,12 @@ bool gather_overlaps(int n_az, long long rows, int K) {
     return ctas <= 152 || ctas > 5 * 152 || c.s * K <= 64.0;
 }
 
-template <bool ADJ, int J, bool OVERLAP>
+template <bool ADJ, int J, bool OVERLAP, bool MANY = false>
 rosar_status launch_gather_j(const float2 *S, const float2 *w, const int32_t *o, int o_row_stride, int n_scans,
                              int n_rng, int n_az, int K, float2 *out, cudaStream_t s) {
     static int done[kMaxDevices] = {};
     constexpr int smem = az::Geo<J>::SMEM_BYTES;
-    rosar_status st = ensure_smem((const void *)sparse_azimuth_kernel<ADJ, J, OVERLAP>, smem, done, "sparse_azimuth");
+    rosar_status st = ensure_smem((const void *)sparse_azimuth_kernel<ADJ, J, OVERLAP, MANY>, smem, done, "sparse_azimuth");
     if (st != ROSAR_OK) return st;
     const dim3 grid((n_az + az::Geo<J>::TW - 1) / az::Geo<J>::TW, n_rng, n_scans);
     cudaLaunchConfig_t cfg = {};
@@ -87,7 +90,8 @@ rosar_status launch_gather_j(const float2 *S, const float2 *w, const int32_t *o,
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = OVERLAP ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, sparse_azimuth_kernel<ADJ, J, OVERLAP>, S, w, o, o_row_stride, n_rng, n_az, K, out);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, sparse_azimuth_kernel<ADJ, J, OVERLAP, MANY>, S, w, o, o_row_stride, n_rng,
+                                             n_az, K, out);
     if (e != cudaSuccess) return set_error(ROSAR_ERR_CUDA, "sparse_azimuth: launch failed: %s", cudaGetErrorString(e));
     return check_launch(ADJ ? "sparse_azimuth_adjoint" : "sparse_azimuth");
 }
@@ -101,8 +105,12 @@ rosar_status launch_gather(const float2 *S, const float2 *w, const int32_t *o, i
         case 1: return launch_gather_j<ADJ, 1, OVERLAP>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
         case 2: return launch_gather_j<ADJ, 2, OVERLAP>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
         case 3: return launch_gather_j<ADJ, 3, OVERLAP>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
-        default: return launch_gather_j<ADJ, 4, OVERLAP>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
+        default: break;
     }
+    if constexpr (OVERLAP)
+        if (K >= 48)
+            return launch_gather_j<ADJ, 4, OVERLAP, true>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
+    return launch_gather_j<ADJ, 4, OVERLAP>(S, w, o, o_row_stride, n_scans, n_rng, n_az, K, out, s);
 }
 
 using MigGeo = az::GeoMig<SA_J>;

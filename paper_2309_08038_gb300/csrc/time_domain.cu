@@ -26,9 +26,9 @@
 // CUDA cores: one row per CTA, the row's phasors staged in shared memory by sample chunk, pulses read through
 // L1/L2.
 //
-// 8 flops per (pixel, tap, sample).  A caller with scratch memory is better served by the transforms of
-// time_domain_lr.cu (rosar_*_time_fft, what the Python functions take); these kernels serve the entries without a
-// workspace, the sizes that form does not have, and scans too small for it.
+// 8 flops per (pixel, tap, sample).  A caller with scratch memory may take the transforms of time_domain_lr.cu
+// (rosar_*_time_fft) instead: the Python SAS does where they are faster, BPA where the caller asks.  These kernels serve
+// the entries without a workspace, BPA by default, and the SAS sizes where the transforms do not pay.
 
 #include <cooperative_groups.h>
 

@@ -500,7 +500,8 @@ lr_combine_kernel(const float2 *__restrict__ X, const uint8_t *__restrict__ plan
 }
 
 __device__ __forceinline__ void fill_nan(float2 *__restrict__ out_row, int n) {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) out_row[i] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
+    const float nan = __int_as_float(0x7fc00000);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out_row[i] = make_float2(nan, nan);
 }
 
 // Whether any pulse is marked, and the terms of the marked pulses' zeroed samples for the pixels of row r whose aperture
@@ -508,7 +509,8 @@ __device__ __forceinline__ void fill_nan(float2 *__restrict__ out_row, int n) {
 // overlaps the one before it, so nothing that this call wrote is read by the non-coherent path.)
 __device__ __forceinline__ bool any_marked(const uint8_t *__restrict__ flags, const Shape &sh) {
     int any = 0;
-    for (int n = threadIdx.x; n < sh.flag_bytes / 4; n += blockDim.x) any |= __ldcg(reinterpret_cast<const int *>(flags) + n);
+    const int *words = reinterpret_cast<const int *>(flags);
+    for (int n = threadIdx.x; n < sh.flag_bytes / 4; n += blockDim.x) any |= __ldcg(words + n);
     return __syncthreads_or(any) != 0;
 }
 __device__ __noinline__ void add_marked(const float2 *__restrict__ raw, const uint8_t *__restrict__ flags,
